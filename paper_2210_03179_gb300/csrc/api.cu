@@ -263,23 +263,24 @@ void read_cscal(chebmg_ctx* c) {
   CK(cudaStreamSynchronize(c->s));
 }
 
-// y = A x on level j; for SEM y must be zero on entry (element contributions accumulate).
+// y = A x on level j; for SEM y must be zero on entry (element contributions accumulate; subtract,
+// SEM only: y -= A x).
 template <typename T>
-void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld) {
+void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld, bool subtract = false) {
   Level& L = c->L[j];
   const int dt = dt_of<T>();
   if (L.type == TYPE_SEM) {
     if (L.Q == 8 && nb > 1)
       sem_ax8_batched<T>(L.E, L.gid, L.lat, static_cast<const T*>(L.G[dt]), x, y, c->dstat, L.beb[dt], nb, ld,
-                         c->s);
+                         c->s, subtract);
     else if (L.Q == 8)
-      sem_ax8<T>(L.E, L.gid, L.lat, static_cast<const T*>(L.G[dt]), x, y, c->dstat, L.eb[dt], c->s);
+      sem_ax8<T>(L.E, L.gid, L.lat, static_cast<const T*>(L.G[dt]), x, y, c->dstat, L.eb[dt], c->s, subtract);
     else if (L.Q == 4 && L.ax4[dt] % 100 == 41)
       sem_ax4<T>(L.E, L.gid, L.ax4[dt] >= 100 ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]),
-                 static_cast<const T*>(L.D[dt]), x, y, c->s, nb, ld);
+                 static_cast<const T*>(L.D[dt]), x, y, c->s, nb, ld, subtract);
     else
       sem_ax<T>(L.Q, L.E, L.gid, static_cast<const T*>(L.G[dt]), static_cast<const T*>(L.D[dt]), x, y, c->s, nb,
-                ld);
+                ld, subtract);
   } else {
     fd_apply<T>(L.mx, L.my, stencil<T>(L), x, y, c->s, nb, ld);
   }
@@ -290,6 +291,12 @@ void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld) {
 template <typename T>
 void apply_into(chebmg_ctx* c, int j, const T* x, T* y) {
   apply_into_ld<T>(c, j, x, y, c->nb, ldv(c, c->L[j]));
+}
+
+// r -= A x on SEM level j for the current batch: the operator's atomics go into r itself.
+template <typename T>
+void apply_subtract(chebmg_ctx* c, int j, const T* x, T* r) {
+  apply_into_ld<T>(c, j, x, r, c->nb, ldv(c, c->L[j]), true);
 }
 
 template <typename T>
@@ -392,14 +399,89 @@ bool smooth_fused(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero
   return true;
 }
 
+// The recurrence of Algorithms 1 and 2 in one form: d_0 = c0 S r_0, then r_i = r_{i-1} - A d_{i-1},
+// d_i = c1(i) d_{i-1} + c2(i) S r_i, and the result is x + sum_i w(i) d_i.  (Algorithm 1 states it
+// with S r in the place of r; here r is the plain residual for both kinds.)
+struct Recurrence {
+  double c0 = 0.0;
+  std::vector<double> c1, c2;   // [1 .. order - 1]
+  std::vector<double> w;        // [0 .. order - 1]
+};
+Recurrence recurrence(chebmg_ctx* c, const Level& L, int order) {
+  Recurrence q;
+  q.c1.resize(order);
+  q.c2.resize(order);
+  q.w.assign(order, 1.0);
+  const double lmax = L.lmax * c->lscale;
+  if (c->o.kind == CHEBMG_CHEB_1ST) {
+    const double lmin = lmin_ratio_for(c, order) * lmax;
+    const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin);
+    const double sigma = theta / delta;
+    double rho = 1.0 / sigma;
+    q.c0 = 1.0 / theta;
+    for (int i = 1; i < order; ++i) {
+      const double rho_new = 1.0 / (2.0 * sigma - rho);
+      q.c1[i] = rho_new * rho;
+      q.c2[i] = 2.0 * rho_new / delta;
+      rho = rho_new;
+    }
+    return q;
+  }
+  const double* beta = (c->o.kind == CHEBMG_CHEB_4TH_OPT) ? kBeta[order - 1] : nullptr;
+  if (!c->beta_ovr.empty() && (int)c->beta_ovr.size() == order) beta = c->beta_ovr.data();
+  q.c0 = 4.0 / (3.0 * lmax);
+  for (int i = 0; i < order; ++i) {
+    if (beta) q.w[i] = beta[i];
+    q.c1[i] = (2.0 * i - 1.0) / (2.0 * i + 3.0);
+    q.c2[i] = (8.0 * i + 4.0) / ((2.0 * i + 3.0) * lmax);
+  }
+  return q;
+}
+
+// smooth() on a SEM level by the separate kernels.  x is updated every other step (a step holds
+// both d_{i-1} and d_i); residual_next leaves r = b, to which the caller applies r -= A x.
+template <typename T>
+void smooth_sem(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero, bool residual_next) {
+  Level& L = c->L[j];
+  const int64_t n = L.n, ld = ldv(c, L);
+  const int nb = c->nb;
+  // one right-hand side: the step kernels launch as programmatic dependents of each other
+  const PdlScope pdl_(g_pdl || nb == 1);
+  T* r = vec<T>(L, VR);
+  T* d = vec<T>(L, VD);
+  const T* S = invD_of<T>(L);
+  const Recurrence q = recurrence(c, L, order);
+  const T* b_next = residual_next ? b : nullptr;
+  if (x_zero) {
+    smooth_begin<T>(n, b, x, r, d, S, q.c0, order == 1, q.w[0], b_next, c->s, nb, ld);
+  } else {
+    cast<T, T>(n, b, r, c->s, nb, ld, ld);
+    apply_subtract<T>(c, j, x, r);
+    smooth_begin_r<T>(n, x, r, d, S, q.c0, order == 1, q.w[0], b_next, c->s, nb, ld);
+  }
+  bool set = x_zero;   // x not written yet
+  for (int i = 1; i < order; ++i) {
+    apply_subtract<T>(c, j, d, r);
+    const bool last = i + 1 == order, both = i % 2 == 1;
+    const int xmode = !both && !last ? SX_NONE : set ? SX_SET : SX_ADD;
+    smooth_step<T>(n, x, r, d, S, q.c1[i], q.c2[i], xmode, both ? q.w[i - 1] : 0.0, q.w[i], last,
+                   last ? b_next : nullptr, c->s, nb, ld);
+    if (xmode != SX_NONE) set = false;
+  }
+  check_launch();
+}
+
 // One smoother application (Algorithm 1 or 2) of the given order on level j.
 template <typename T>
 void smooth(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero) {
   if (smooth_fused<T>(c, j, b, x, order, x_zero, false)) return;
   Level& L = c->L[j];
+  if (L.type == TYPE_SEM) {
+    smooth_sem<T>(c, j, b, x, order, x_zero, false);
+    return;
+  }
   const int64_t n = L.n;
   const int nb = c->nb;
-  // one right-hand side: the step kernels launch as programmatic dependents of each other
   const PdlScope pdl_(g_pdl || nb == 1);
   const int64_t ld = ldv(c, L);
   T* r = vec<T>(L, VR);
@@ -704,18 +786,23 @@ int vcycle_level(chebmg_ctx* c, int j, const T* b, T* x) {
   if (j == (int)c->L.size() - 1) return coarse<T>(c, b, x);
   Level& L = c->L[j];
   Level& C = c->L[j + 1];
-  // the fused kernel computes the restriction residual in the same launch as the pre-smoother
+  // the fused kernel computes the restriction residual in the same launch as the pre-smoother;
+  // the separate SEM kernels leave r = b, from which one more product subtracts A x
+  const bool sem = L.type == TYPE_SEM;
+  T* y = vec<T>(L, VY);
+  T* r = vec<T>(L, VR);
   bool have_r = false;
   if (c->pre > 0) {
     have_r = smooth_fused<T>(c, j, b, x, c->pre, true, true);
-    if (!have_r) smooth<T>(c, j, b, x, c->pre, true);
+    if (!have_r && sem) smooth_sem<T>(c, j, b, x, c->pre, true, true);
+    else if (!have_r) smooth<T>(c, j, b, x, c->pre, true);
   } else {
     zero<T>(c, x, span(c, L));
+    if (sem) cast<T, T>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
   }
-  T* y = vec<T>(L, VY);
-  T* r = vec<T>(L, VR);
-  if (!have_r) {
-    if (c->pre == 0) zero<T>(c, y, span(c, L));   // the smoothers leave y = 0
+  if (!have_r && sem) {
+    apply_subtract<T>(c, j, x, r);
+  } else if (!have_r) {
     apply_into<T>(c, j, x, y);
     residual<T>(L.n, b, y, r, c->s, c->nb, ldv(c, L));
   }
@@ -1651,9 +1738,13 @@ int vcycle_store(chebmg_ctx* c, int j, const double* b, double* x) {
   else zero<double>(c, x, span(c, L));
   double* y = vec<double>(L, VY);
   double* r = vec<double>(L, VR);
-  zero<double>(c, y, span(c, L));
-  apply_into<double>(c, j, x, y);
-  residual<double>(L.n, b, y, r, c->s, c->nb, ldv(c, L));
+  if (L.type == TYPE_SEM) {
+    cast<double, double>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
+    apply_subtract<double>(c, j, x, r);
+  } else {
+    apply_into<double>(c, j, x, y);
+    residual<double>(L.n, b, y, r, c->s, c->nb, ldv(c, L));
+  }
   restrict_to<double>(c, j, r, vec<double>(C, VB));
   const int rc = vcycle_store(c, j + 1, vec<double>(C, VB), vec<double>(C, VX));
   if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;

@@ -183,6 +183,105 @@ __global__ void k_cheb4_step(int64_t n, T* __restrict__ x, T* r, T* __restrict__
   }
 }
 
+// ---- SEM smoothing: the operator subtracts A d from r in place ----
+// Bytes bound these kernels.  Against the form with a product vector y (y zeroed, accumulated,
+// read back and zeroed again, r rewritten) a step moves 4 n-vectors instead of 8 beside the x
+// update, and x is touched every other step only: a step has both d_{i-1} and d_i at hand.
+// Measured on 32^3 elements of order 7, order 6 from a zero guess, FP32: 748.7 -> 614.7 us; a whole
+// mixed solve of that size 33.19 -> 31.60 ms; 64 right-hand sides on 8^3 elements 28.73 -> 27.43 ms.
+
+// Zero guess: r = b (rin = b), d = c0 S b; or (from_r) from the residual r: d = c0 S r.  order1:
+// x = w d (x += w d from a residual) instead of storing d.  b_next leaves r = b_next for the
+// restriction residual.
+template <typename T, bool VEC>
+__global__ void k_smooth_begin(int64_t n, const T* rin, T* __restrict__ x, T* r, T* __restrict__ d,
+                               const T* __restrict__ invD, T c0, T w, int from_r, int order1, const T* b_next, int64_t ld) {
+  pdl_wait();
+  { const int64_t off_ = (int64_t)blockIdx.y * ld; rin += off_; x += off_; r += off_; d += off_; if (b_next) b_next += off_; }
+  using VT = typename V16<T>::type;
+  constexpr int L = V16<T>::L;
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t nv = VEC ? n / L : 0;
+  const uint64_t last = l2_policy_last();
+  for (int64_t q = tid; q < nv; q += stride) {
+    VT rv = reinterpret_cast<const VT*>(rin)[q], dv, xv = {};
+    const VT sv = reinterpret_cast<const VT*>(invD)[q];
+    if (order1 && from_r) xv = reinterpret_cast<const VT*>(x)[q];
+    if (b_next && from_r) {
+      const VT bv = reinterpret_cast<const VT*>(b_next)[q];
+      st16(reinterpret_cast<VT*>(r) + q, bv, last);
+    } else if (!from_r && (b_next || !order1)) {
+      st16(reinterpret_cast<VT*>(r) + q, rv, last);
+    }
+    T* rs = reinterpret_cast<T*>(&rv);
+    T* ds = reinterpret_cast<T*>(&dv);
+    T* xs = reinterpret_cast<T*>(&xv);
+    const T* ss = reinterpret_cast<const T*>(&sv);
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      ds[l] = c0 * ss[l] * rs[l];
+      xs[l] = from_r ? xs[l] + w * ds[l] : w * ds[l];
+    }
+    if (order1) reinterpret_cast<VT*>(x)[q] = xv;
+    else st16(reinterpret_cast<VT*>(d) + q, dv, last);
+  }
+  for (int64_t g = nv * L + tid; g < n; g += stride) {
+    const T rv = rin[g], dv = c0 * invD[g] * rv;
+    if (b_next && from_r) r[g] = b_next[g];
+    else if (!from_r && (b_next || !order1)) r[g] = rv;
+    if (!order1) d[g] = dv;
+    else x[g] = from_r ? x[g] + w * dv : w * dv;
+  }
+}
+
+// One recurrence step: d' = c1 d + c2 S r, then (XM) x += or = w0 d + w1 d'.  LAST: d' is not
+// stored (nothing reads it).
+template <typename T, bool VEC, int XM, bool LAST>
+__global__ void k_smooth_step(int64_t n, T* __restrict__ x, T* __restrict__ r, T* __restrict__ d,
+                              const T* __restrict__ invD, T c1, T c2, T w0, T w1, const T* __restrict__ b_next,
+                              int64_t ld) {
+  // Triggering the next kernel early (griddepcontrol.launch_dependents) was measured slower: its
+  // waiting blocks cost this grid's last wave more than they saved.
+  pdl_wait();
+  { const int64_t off_ = (int64_t)blockIdx.y * ld; x += off_; r += off_; d += off_; if (b_next) b_next += off_; }
+  using VT = typename V16<T>::type;
+  constexpr int L = V16<T>::L;
+  const int64_t nv = VEC ? n / L : 0;
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const uint64_t first = l2_policy_first(), last = l2_policy_last();
+  auto one = [&](T& xg, T& dg, T rg, T sg) {
+    const T dn = c1 * dg + c2 * sg * rg;
+    if (XM == SX_ADD) xg = (xg + w0 * dg) + w1 * dn;
+    if (XM == SX_SET) xg = w0 * dg + w1 * dn;
+    dg = dn;
+  };
+  for (int64_t q = tid; q < nv; q += stride) {
+    VT xv = {}, rv = ld16(reinterpret_cast<const VT*>(r) + q, last);
+    VT dv = ld16(reinterpret_cast<const VT*>(d) + q, last);
+    if (XM == SX_ADD) xv = ld16(reinterpret_cast<const VT*>(x) + q, first);
+    const VT sv = ld16(reinterpret_cast<const VT*>(invD) + q, first);
+    VT bv = {};
+    if (LAST && b_next) bv = ld16(reinterpret_cast<const VT*>(b_next) + q, first);
+    T* xs = reinterpret_cast<T*>(&xv);
+    T* ds = reinterpret_cast<T*>(&dv);
+    const T* rs = reinterpret_cast<const T*>(&rv);
+    const T* ss = reinterpret_cast<const T*>(&sv);
+#pragma unroll
+    for (int l = 0; l < L; ++l) one(xs[l], ds[l], rs[l], ss[l]);
+    if (XM != SX_NONE) st16(reinterpret_cast<VT*>(x) + q, xv, LAST ? last : first);
+    if (!LAST) st16(reinterpret_cast<VT*>(d) + q, dv, last);
+    if (LAST && b_next) st16(reinterpret_cast<VT*>(r) + q, bv, last);
+  }
+  for (int64_t g = nv * L + tid; g < n; g += stride) {
+    T xg = XM == SX_ADD ? x[g] : T(0), dg = d[g];
+    one(xg, dg, r[g], invD[g]);
+    if (XM != SX_NONE) x[g] = xg;
+    if (!LAST) d[g] = dg;
+    if (LAST && b_next) r[g] = b_next[g];
+  }
+}
+
 template <typename T>
 __global__ void k_cheb1_init(int64_t n, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ r,
                              T* __restrict__ d, T* __restrict__ y, const T* __restrict__ invD,
@@ -305,6 +404,54 @@ void cheb4_step(int64_t n, T* x, T* r, T* d, T* y, const T* invD, double beta, d
   else
     launch_cheb4_step<T, false>(n, x, r, d, y, invD, beta, c1, c2, s, nb, ld, beta_next, r);
 }
+// Whether every pointer and the batch stride allow 16-byte accesses.
+template <typename T, typename... P>
+static bool vec_ok(int nb, int64_t ld, const P*... p) {
+  return (((uintptr_t)p | ...) % 16) == 0 && (nb == 1 || (ld * sizeof(T)) % 16 == 0);
+}
+template <typename T>
+static void launch_begin(int64_t n, const T* rin, T* x, T* r, T* d, const T* invD, double c0, double w, int from_r,
+                         int order1, const T* b_next, cudaStream_t s, int nb, int64_t ld) {
+  if (!ld) ld = n;
+  if (vec_ok<T>(nb, ld, rin, x, r, d, invD, b_next))
+    launch_dep(k_smooth_begin<T, true>, dim3(grid_for(n / V16<T>::L + 1, kVecThreads), nb), dim3(kVecThreads), 0, s,
+               n, rin, x, r, d, invD, (T)c0, (T)w, from_r, order1, b_next, ld);
+  else
+    launch_dep(k_smooth_begin<T, false>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, rin, x, r,
+               d, invD, (T)c0, (T)w, from_r, order1, b_next, ld);
+}
+template <typename T>
+void smooth_begin(int64_t n, const T* b, T* x, T* r, T* d, const T* invD, double c0, bool order1, double w,
+                  const T* b_next, cudaStream_t s, int nb, int64_t ld) {
+  launch_begin<T>(n, b, x, r, d, invD, c0, w, 0, order1 ? 1 : 0, b_next, s, nb, ld);
+}
+template <typename T>
+void smooth_begin_r(int64_t n, T* x, T* r, T* d, const T* invD, double c0, bool order1, double w, const T* b_next,
+                    cudaStream_t s, int nb, int64_t ld) {
+  launch_begin<T>(n, r, x, r, d, invD, c0, w, 1, order1 ? 1 : 0, b_next, s, nb, ld);
+}
+template <typename T, int XM, bool LAST>
+static void launch_smooth_step(int64_t n, T* x, T* r, T* d, const T* invD, double c1, double c2, double w0, double w1,
+                               const T* b_next, cudaStream_t s, int nb, int64_t ld) {
+  if (!ld) ld = n;
+  if (vec_ok<T>(nb, ld, x, r, d, invD, b_next))
+    launch_dep(k_smooth_step<T, true, XM, LAST>, dim3(grid_for(n / V16<T>::L + 1, kVecThreads), nb),
+               dim3(kVecThreads), 0, s, n, x, r, d, invD, (T)c1, (T)c2, (T)w0, (T)w1, b_next, ld);
+  else
+    launch_dep(k_smooth_step<T, false, XM, LAST>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, x,
+               r, d, invD, (T)c1, (T)c2, (T)w0, (T)w1, b_next, ld);
+}
+template <typename T>
+void smooth_step(int64_t n, T* x, T* r, T* d, const T* invD, double c1, double c2, int xmode, double w0, double w1,
+                 bool last, const T* b_next, cudaStream_t s, int nb, int64_t ld) {
+  if (xmode == SX_NONE) launch_smooth_step<T, SX_NONE, false>(n, x, r, d, invD, c1, c2, w0, w1, nullptr, s, nb, ld);
+  else if (xmode == SX_ADD && last)
+    launch_smooth_step<T, SX_ADD, true>(n, x, r, d, invD, c1, c2, w0, w1, b_next, s, nb, ld);
+  else if (xmode == SX_ADD)
+    launch_smooth_step<T, SX_ADD, false>(n, x, r, d, invD, c1, c2, w0, w1, nullptr, s, nb, ld);
+  else if (last) launch_smooth_step<T, SX_SET, true>(n, x, r, d, invD, c1, c2, w0, w1, b_next, s, nb, ld);
+  else launch_smooth_step<T, SX_SET, false>(n, x, r, d, invD, c1, c2, w0, w1, nullptr, s, nb, ld);
+}
 template <typename T>
 void cheb1_init(int64_t n, const T* b, T* x, T* r, T* d, T* y, const T* invD, double inv_theta,
                 int x_is_zero, cudaStream_t s, int nb, int64_t ld) {
@@ -351,6 +498,12 @@ void masked_copy(int64_t n, const double* in, const double* invD, double* out, c
   template void cheb1_init<T>(int64_t, const T*, T*, T*, T*, T*, const T*, double, int, cudaStream_t, int,    \
                               int64_t);                                                                 \
   template void cheb1_step<T>(int64_t, T*, T*, T*, T*, const T*, double, double, cudaStream_t, int, int64_t); \
+  template void smooth_begin<T>(int64_t, const T*, T*, T*, T*, const T*, double, bool, double, const T*,    \
+                                cudaStream_t, int, int64_t);                                            \
+  template void smooth_begin_r<T>(int64_t, T*, T*, T*, const T*, double, bool, double, const T*, cudaStream_t, \
+                                  int, int64_t);                                                        \
+  template void smooth_step<T>(int64_t, T*, T*, T*, const T*, double, double, int, double, double, bool,      \
+                               const T*, cudaStream_t, int, int64_t);                                   \
   template void axpy<T>(int64_t, double, const T*, T*, cudaStream_t, int, int64_t);                     \
   template void residual<T>(int64_t, const T*, T*, T*, cudaStream_t, int, int64_t);
 

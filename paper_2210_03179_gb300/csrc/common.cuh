@@ -70,6 +70,16 @@ enum PostOp { POST_NONE = 0, POST_ALPHA, POST_BETA_CG, POST_SET_RZ_FROM_ZR, POST
 
 constexpr int kRedBlocks = 1216;   // 152 SMs x 8: partial sums per reduction pass (full occupancy)
 
+#ifdef __CUDACC__
+// v, or -v when neg is the sign bit: one integer operation, exact (an FP64 multiplication would
+// go through the slow FP64 pipe).
+__device__ __forceinline__ float flip_sign(float v, uint32_t neg) { return __uint_as_float(__float_as_uint(v) ^ neg); }
+__device__ __forceinline__ double flip_sign(double v, uint32_t neg) {
+  return __hiloint2double(__double2hiint(v) ^ (int)neg, __double2loint(v));
+}
+#endif
+constexpr uint32_t kSignBit = 0x80000000u;
+
 template <typename T>
 struct Stencil9 {
   T c[9];
@@ -79,12 +89,12 @@ struct Stencil9 {
 // aligned p), else by a memset.
 void zero_bytes(void* p, int64_t bytes, cudaStream_t s);
 
-// ---- SEM kernels (y must be zeroed by the caller; results accumulate) ----
+// ---- SEM kernels (results accumulate into y: y += A u, or y -= A u when subtract is set) ----
 // Every operator, transfer and vector kernel also runs on a batch of nb right-hand sides:
 // vector b of the batch starts at offset b * ld (ld = 0 means n; per-node data shared).
 template <typename T>
 void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
-            cudaStream_t s, int nb = 1, int64_t ld = 0);
+            cudaStream_t s, int nb = 1, int64_t ld = 0, bool subtract = false);
 template <typename T>
 void sem_restrict(int Qf, int Qc, int64_t E, const uint32_t* gidf, const uint32_t* gidc,
                   const T* J, const T* rf, T* rc, cudaStream_t s, int nb = 1, int64_t ldf = 0, int64_t ldc = 0);
@@ -105,7 +115,7 @@ struct Lattice {
 // sem_ax for Q = 4; ids from the box lattice when lat is given, else from gid.
 template <typename T>
 void sem_ax4(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* D, const T* u, T* y,
-             cudaStream_t s, int nb = 1, int64_t ld = 0);
+             cudaStream_t s, int nb = 1, int64_t ld = 0, bool subtract = false);
 // The order-7 operator in FP64-class arithmetic on FP32 pairs (sem_ax8_x2.cu): G in that
 // format (sem_to_x2 converts an FP64 array of n values), u and y FP64; variant as sem_ax8's
 // non-persistent codes (1, 2, 4; +100 box lattice ids); batches of nb vectors at stride ld,
@@ -122,14 +132,14 @@ void sem_ax8_x2(int64_t E, const uint32_t* gid, const Lattice& lat, const void* 
 // the persistent ones start their first geometric-factor copy before pdl_wait().
 template <typename T>
 void sem_ax8(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-             unsigned* err, int variant, cudaStream_t s);
+             unsigned* err, int variant, cudaStream_t s, bool subtract = false);
 // Batched form: nb right-hand sides at leading dimension ld.  variant = 1000 * RB + (100 if
 // implicit ids) + EB: a block stages the geometric factors of EB elements once and applies them
 // to RB right-hand sides; EB + 10 (EB 1 or 2) takes the right-hand sides two at a time through
 // each line pass (RB at least 2); EB + 20 (EB 1 or 2) keeps the factors in registers instead.
 template <typename T>
 void sem_ax8_batched(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                     unsigned* err, int variant, int nb, int64_t ld, cudaStream_t s);
+                     unsigned* err, int variant, int nb, int64_t ld, cudaStream_t s, bool subtract = false);
 // Whether variant `eb` fits the device's per-block shared-memory limit.
 template <typename T>
 bool sem_ax8_variant_fits(int eb);
@@ -237,6 +247,22 @@ void cheb1_init(int64_t n, const T* b, T* x, T* r, T* d, T* y, const T* invD, do
 template <typename T>
 void cheb1_step(int64_t n, T* x, T* r, T* d, T* y, const T* invD, double c1, double c2,
                 cudaStream_t s, int nb = 1, int64_t ld = 0);
+// SEM smoothing (both kinds): the operator subtracts A d from r itself (atomics into r), so there
+// is no product vector.  Every pointer below is a level vector; b_next, if given, leaves r = b_next
+// for the product that follows (the restriction residual).
+// Zero guess: r = b, d = c0 S b; order1 (a smoother of order 1): x = w d instead.
+template <typename T>
+void smooth_begin(int64_t n, const T* b, T* x, T* r, T* d, const T* invD, double c0, bool order1, double w,
+                  const T* b_next, cudaStream_t s, int nb, int64_t ld);
+// From the residual r: d = c0 S r; order1: x += w d instead.
+template <typename T>
+void smooth_begin_r(int64_t n, T* x, T* r, T* d, const T* invD, double c0, bool order1, double w, const T* b_next,
+                    cudaStream_t s, int nb, int64_t ld);
+// d' = c1 d + c2 S r (not stored when last), then x = or += w0 d + w1 d'.
+enum SmoothX { SX_NONE = 0, SX_ADD = 1, SX_SET = 2 };
+template <typename T>
+void smooth_step(int64_t n, T* x, T* r, T* d, const T* invD, double c1, double c2, int xmode, double w0, double w1,
+                 bool last, const T* b_next, cudaStream_t s, int nb, int64_t ld);
 // x += a * d
 template <typename T>
 void axpy(int64_t n, double a, const T* d, T* x, cudaStream_t s, int nb = 1, int64_t ld = 0);

@@ -47,7 +47,7 @@ struct SemShape {
 template <typename T, int Q>
 __global__ void __launch_bounds__(SemShape<Q>::THREADS)
 k_sem_ax(int64_t E, const uint32_t* __restrict__ gid, const T* __restrict__ G,
-         const T* __restrict__ Dg, const T* __restrict__ u, T* __restrict__ y, int64_t ld) {
+         const T* __restrict__ Dg, const T* __restrict__ u, T* __restrict__ y, int64_t ld, uint32_t neg) {
   constexpr int NP = SemShape<Q>::NP;
   u += (int64_t)blockIdx.y * ld;   // right-hand side of a batch
   y += (int64_t)blockIdx.y * ld;
@@ -108,15 +108,15 @@ k_sem_ax(int64_t E, const uint32_t* __restrict__ gid, const T* __restrict__ G,
     acc += sD[l * Q + j] * ss[(k * Q + l) * Q + i];
     acc += sD[l * Q + k] * st[(l * Q + j) * Q + i];
   }
-  if (valid && !(id & kGidDirichlet)) atomicAdd(&y[id & kGidMask], acc);
+  if (valid && !(id & kGidDirichlet)) atomicAdd(&y[id & kGidMask], flip_sign(acc, neg));
 }
 
 template <typename T, int Q>
 static void launch_sem_ax(int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
-                          cudaStream_t s, int nb, int64_t ld) {
+                          cudaStream_t s, int nb, int64_t ld, uint32_t neg) {
   using S = SemShape<Q>;
   const unsigned blocks = (unsigned)((E + S::EPB - 1) / S::EPB);
-  launch_dep(k_sem_ax<T, Q>, dim3(blocks, nb), dim3(S::THREADS), 0, s, E, gid, G, D, u, y, ld);
+  launch_dep(k_sem_ax<T, Q>, dim3(blocks, nb), dim3(S::THREADS), 0, s, E, gid, G, D, u, y, ld, neg);
 }
 
 // Order-3 element operator (N = 3, 4 points per direction) by line passes: 16 threads per
@@ -133,7 +133,7 @@ constexpr int kAx4Plane = 20;                    // padded k-plane stride: confl
 template <typename T, bool IMPLICIT>
 __global__ void __launch_bounds__(kAx4Threads)
 k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-          const T* __restrict__ Dg, const T* __restrict__ u, T* __restrict__ y, int64_t ld) {
+          const T* __restrict__ Dg, const T* __restrict__ u, T* __restrict__ y, int64_t ld, uint32_t neg) {
   constexpr int PK = kAx4Plane, EL = 4 * kAx4Plane;
   __shared__ __align__(16) T sU[kAx4Threads / 16][EL];
   __shared__ __align__(16) T sR[kAx4Threads / 16][EL];
@@ -261,32 +261,34 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < 4; ++k)
-    if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], su[k * PK + b * 4 + a] + yt[k]);
+    if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(su[k * PK + b * 4 + a] + yt[k], neg));
 }
 
 template <typename T>
 void sem_ax4(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* D, const T* u, T* y,
-             cudaStream_t s, int nb, int64_t ld) {
+             cudaStream_t s, int nb, int64_t ld, bool subtract) {
   const dim3 blocks((unsigned)((E + kAx4Threads / 16 - 1) / (kAx4Threads / 16)), nb);
+  const uint32_t neg = subtract ? kSignBit : 0u;
   if (lat)
-    launch_dep(k_sem_ax4<T, true>, blocks, dim3(kAx4Threads), 0, s, E, gid, *lat, G, D, u, y, ld);
+    launch_dep(k_sem_ax4<T, true>, blocks, dim3(kAx4Threads), 0, s, E, gid, *lat, G, D, u, y, ld, neg);
   else
-    launch_dep(k_sem_ax4<T, false>, blocks, dim3(kAx4Threads), 0, s, E, gid, Lattice{}, G, D, u, y, ld);
+    launch_dep(k_sem_ax4<T, false>, blocks, dim3(kAx4Threads), 0, s, E, gid, Lattice{}, G, D, u, y, ld, neg);
 }
 
 template <typename T>
 void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
-            cudaStream_t s, int nb, int64_t ld) {
+            cudaStream_t s, int nb, int64_t ld, bool subtract) {
+  const uint32_t neg = subtract ? kSignBit : 0u;
   switch (Q) {
-    case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 3: launch_sem_ax<T, 3>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 5: launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 6: launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 8: launch_sem_ax<T, 8>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 9: launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld); break;
-    case 10: launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld); break;
+    case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 3: launch_sem_ax<T, 3>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 5: launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 6: launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 8: launch_sem_ax<T, 8>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 9: launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 10: launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg); break;
     default: break;
   }
 }
@@ -1385,9 +1387,9 @@ void scale(int64_t n, double a, const double* x, double* y, cudaStream_t s) {
 // ===========================================================================
 #define CHEBMG_INST(T)                                                                                \
   template void sem_ax4<T>(int64_t, const uint32_t*, const Lattice*, const T*, const T*, const T*, T*,           \
-                           cudaStream_t, int, int64_t);                                                    \
+                           cudaStream_t, int, int64_t, bool);                                              \
   template void sem_ax<T>(int, int64_t, const uint32_t*, const T*, const T*, const T*, T*, cudaStream_t, int,  \
-                          int64_t);                                                                   \
+                          int64_t, bool);                                                             \
   template void sem_restrict<T>(int, int, int64_t, const uint32_t*, const uint32_t*, const T*, const T*,  \
                                 T*, cudaStream_t, int, int64_t, int64_t);                              \
   template void sem_prolong<T>(int, int, int64_t, const uint32_t*, const uint32_t*, const T*, const T*,   \

@@ -31,7 +31,7 @@ namespace {
 template <typename T, int EB_, bool IMPLICIT>
 __global__ void __launch_bounds__(64 * EB_)
 k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-          const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err) {
+          const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err, uint32_t neg) {
   using C = Ax8<T, EB_>;
   constexpr int EB = C::EB, R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -140,7 +140,7 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const T v = su[k * P + b * R + a] + yt[k];
-      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], v);
+      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(v, neg));
     }
   }
 }
@@ -153,7 +153,7 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
 template <typename T, int EB_, bool IMPLICIT>
 __global__ void __launch_bounds__(64 * EB_)
 k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-           const T* __restrict__ u, T* __restrict__ y) {
+           const T* __restrict__ u, T* __restrict__ y, uint32_t neg) {
   using C = Ax8<T, EB_>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -227,7 +227,7 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const T v = su[k * P + b * R + a] + yt[k];
-      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], v);
+      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(v, neg));
     }
   }
 }
@@ -242,7 +242,7 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 template <typename T, int EB, bool IMPLICIT, int NB = 2>
 __global__ void __launch_bounds__(64 * EB)
 k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-           const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err) {
+           const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err, uint32_t neg) {
   static_assert(NB == 1 || NB == 2, "one or two geometric-factor buffers");
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
@@ -368,7 +368,7 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const T v = su[k * P + b * R + a] + yt[k];
-      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], v);
+      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(v, neg));
     }
     __syncthreads();             // stage buffers and this G buffer are free for reuse
 #pragma unroll
@@ -386,7 +386,8 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 template <typename T, int EB, bool IMPLICIT>
 __global__ void __launch_bounds__(64 * EB)
 k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-           const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err, int nb, int64_t ld, int rb) {
+           const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err, int nb, int64_t ld, int rb,
+           uint32_t neg) {
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -499,7 +500,7 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const T v = su[k * P + b * R + a] + yt[k];
-        if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], v);
+        if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], flip_sign(v, neg));
       }
     }
     __syncthreads();             // stage buffers free for the next right-hand side
@@ -517,7 +518,7 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 template <typename T, int EB, bool IMPLICIT>
 __global__ void __launch_bounds__(64 * EB)
 k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-            const T* __restrict__ u, T* __restrict__ y, int nb, int64_t ld, int rb) {
+            const T* __restrict__ u, T* __restrict__ y, int nb, int64_t ld, int rb, uint32_t neg) {
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -603,7 +604,7 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const T v = su[k * P + b * R + a] + yt[k];
-        if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], v);
+        if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], flip_sign(v, neg));
       }
     }
     __syncthreads();             // stage buffers free for the next right-hand side
@@ -619,7 +620,8 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
 template <typename T, int EB, bool IMPLICIT>
 __global__ void __launch_bounds__(64 * EB)
 k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
-            const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err, int nb, int64_t ld, int rb) {
+            const T* __restrict__ u, T* __restrict__ y, unsigned* __restrict__ err, int nb, int64_t ld, int rb,
+           uint32_t neg) {
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -750,7 +752,7 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const T v = su[h][k * P + b * R + a] + yt[h][k];
-          if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], v);
+          if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], flip_sign(v, neg));
         }
       }
     }
@@ -792,7 +794,7 @@ cudaError_t sem_ax8_set_D(const double* D) {
 
 template <typename T, int EB, bool IM>
 static void launch_ax8(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                       unsigned* err, cudaStream_t s) {
+                       unsigned* err, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   static bool configured = false;
   if (!configured) {
@@ -800,12 +802,12 @@ static void launch_ax8(int64_t E, const uint32_t* gid, const Lattice& lat, const
     configured = true;
   }
   const unsigned blocks = (unsigned)((E + EB - 1) / EB);
-  launch_dep(k_sem_ax8<T, EB, IM>, dim3(blocks), dim3(64 * EB), C::smem_bytes(), s, E, gid, lat, G, u, y, err);
+  launch_dep(k_sem_ax8<T, EB, IM>, dim3(blocks), dim3(64 * EB), C::smem_bytes(), s, E, gid, lat, G, u, y, err, neg);
 }
 
 template <typename T, int EB, bool IM>
 static void launch_ax8g(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                        cudaStream_t s) {
+                        cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * 3 * C::STAGE;
   static bool configured = false;
@@ -814,12 +816,12 @@ static void launch_ax8g(int64_t E, const uint32_t* gid, const Lattice& lat, cons
     configured = true;
   }
   const unsigned blocks = (unsigned)((E + EB - 1) / EB);
-  launch_dep(k_sem_ax8g<T, EB, IM>, dim3(blocks), dim3(64 * EB), smem, s, E, gid, lat, G, u, y);
+  launch_dep(k_sem_ax8g<T, EB, IM>, dim3(blocks), dim3(64 * EB), smem, s, E, gid, lat, G, u, y, neg);
 }
 
 template <typename T, int EB, bool IM, int NB = 2>
 static void launch_ax8p(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                        unsigned* err, cudaStream_t s) {
+                        unsigned* err, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * (NB * C::GELEM + 3 * C::STAGE);
   static int grid = 0;
@@ -833,12 +835,12 @@ static void launch_ax8p(int64_t E, const uint32_t* gid, const Lattice& lat, cons
   }
   const int64_t nbatch = (E + EB - 1) / EB;
   const unsigned blocks = (unsigned)(nbatch < grid ? nbatch : grid);
-  launch_dep(k_sem_ax8p<T, EB, IM, NB>, dim3(blocks), dim3(64 * EB), smem, s, E, gid, lat, G, u, y, err);
+  launch_dep(k_sem_ax8p<T, EB, IM, NB>, dim3(blocks), dim3(64 * EB), smem, s, E, gid, lat, G, u, y, err, neg);
 }
 
 template <typename T, int EB, bool IM>
 static void launch_ax8b(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                        unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s) {
+                        unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   static bool configured = false;
   if (!configured) {
@@ -848,13 +850,13 @@ static void launch_ax8b(int64_t E, const uint32_t* gid, const Lattice& lat, cons
   }
   if (rb < 1) rb = 1;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
-  k_sem_ax8b<T, EB, IM><<<blocks, 64 * EB, C::smem_bytes(), s>>>(E, gid, lat, G, u, y, err, nb, ld, rb);
+  k_sem_ax8b<T, EB, IM><<<blocks, 64 * EB, C::smem_bytes(), s>>>(E, gid, lat, G, u, y, err, nb, ld, rb, neg);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
 template <typename T, int EB, bool IM>
 static void launch_ax8b2(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                         unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s) {
+                         unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * (C::GELEM + 6 * C::STAGE);
   static bool configured = false;
@@ -864,13 +866,13 @@ static void launch_ax8b2(int64_t E, const uint32_t* gid, const Lattice& lat, con
   }
   if (rb < 2) rb = 2;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
-  k_sem_ax8b2<T, EB, IM><<<blocks, 64 * EB, smem, s>>>(E, gid, lat, G, u, y, err, nb, ld, rb);
+  k_sem_ax8b2<T, EB, IM><<<blocks, 64 * EB, smem, s>>>(E, gid, lat, G, u, y, err, nb, ld, rb, neg);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
 template <typename T, int EB, bool IM>
 static void launch_ax8bg(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y, int nb,
-                         int64_t ld, int rb, cudaStream_t s) {
+                         int64_t ld, int rb, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * 3 * C::STAGE;
   static bool configured = false;
@@ -880,7 +882,7 @@ static void launch_ax8bg(int64_t E, const uint32_t* gid, const Lattice& lat, con
   }
   if (rb < 1) rb = 1;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
-  k_sem_ax8bg<T, EB, IM><<<blocks, 64 * EB, smem, s>>>(E, gid, lat, G, u, y, nb, ld, rb);
+  k_sem_ax8bg<T, EB, IM><<<blocks, 64 * EB, smem, s>>>(E, gid, lat, G, u, y, nb, ld, rb, neg);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
@@ -921,30 +923,32 @@ bool sem_ax8_variant_fits(int eb) {
 
 template <typename T, bool IM>
 static void dispatch_ax8(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                         unsigned* err, int eb, cudaStream_t s) {
+                         unsigned* err, int eb, cudaStream_t s, uint32_t neg) {
   switch (eb) {
-    case 21: launch_ax8g<T, 1, IM>(E, gid, lat, G, u, y, s); break;
-    case 22: launch_ax8g<T, 2, IM>(E, gid, lat, G, u, y, s); break;
-    case 1: launch_ax8<T, 1, IM>(E, gid, lat, G, u, y, err, s); break;
-    case 4: launch_ax8<T, 4, IM>(E, gid, lat, G, u, y, err, s); break;
-    case 12: launch_ax8p<T, 2, IM>(E, gid, lat, G, u, y, err, s); break;
-    case 14: launch_ax8p<T, 4, IM>(E, gid, lat, G, u, y, err, s); break;
-    case 31: launch_ax8p<T, 1, IM, 1>(E, gid, lat, G, u, y, err, s); break;
-    case 32: launch_ax8p<T, 2, IM, 1>(E, gid, lat, G, u, y, err, s); break;
-    default: launch_ax8<T, 2, IM>(E, gid, lat, G, u, y, err, s); break;
+    case 21: launch_ax8g<T, 1, IM>(E, gid, lat, G, u, y, s, neg); break;
+    case 22: launch_ax8g<T, 2, IM>(E, gid, lat, G, u, y, s, neg); break;
+    case 1: launch_ax8<T, 1, IM>(E, gid, lat, G, u, y, err, s, neg); break;
+    case 4: launch_ax8<T, 4, IM>(E, gid, lat, G, u, y, err, s, neg); break;
+    case 12: launch_ax8p<T, 2, IM>(E, gid, lat, G, u, y, err, s, neg); break;
+    case 14: launch_ax8p<T, 4, IM>(E, gid, lat, G, u, y, err, s, neg); break;
+    case 31: launch_ax8p<T, 1, IM, 1>(E, gid, lat, G, u, y, err, s, neg); break;
+    case 32: launch_ax8p<T, 2, IM, 1>(E, gid, lat, G, u, y, err, s, neg); break;
+    default: launch_ax8<T, 2, IM>(E, gid, lat, G, u, y, err, s, neg); break;
   }
 }
 
 template <typename T>
 void sem_ax8(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y, unsigned* err,
-             int variant, cudaStream_t s) {
-  if (variant >= 100) dispatch_ax8<T, true>(E, gid, lat, G, u, y, err, variant - 100, s);
-  else dispatch_ax8<T, false>(E, gid, lat, G, u, y, err, variant, s);
+             int variant, cudaStream_t s, bool subtract) {
+  const uint32_t neg = subtract ? kSignBit : 0u;
+  if (variant >= 100) dispatch_ax8<T, true>(E, gid, lat, G, u, y, err, variant - 100, s, neg);
+  else dispatch_ax8<T, false>(E, gid, lat, G, u, y, err, variant, s, neg);
 }
 
 template <typename T>
 void sem_ax8_batched(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
-                     unsigned* err, int variant, int nb, int64_t ld, cudaStream_t s) {
+                     unsigned* err, int variant, int nb, int64_t ld, cudaStream_t s, bool subtract) {
+  const uint32_t neg = subtract ? kSignBit : 0u;
   const int rb = variant / 1000;
   const bool im = (variant % 1000) >= 100;
   const int form = (variant % 100) / 10;   // 0 single, 1 paired, 2 factors in registers
@@ -954,33 +958,33 @@ void sem_ax8_batched(int64_t E, const uint32_t* gid, const Lattice& lat, const T
     // FP32 only: 48 FP64 factors per thread do not fit the register file
     if constexpr (sizeof(T) == 4) {
       if (im) {
-        if (eb == 1) launch_ax8bg<T, 1, true>(E, gid, lat, G, u, y, nb, ld, rb, s);
-        else launch_ax8bg<T, 2, true>(E, gid, lat, G, u, y, nb, ld, rb, s);
+        if (eb == 1) launch_ax8bg<T, 1, true>(E, gid, lat, G, u, y, nb, ld, rb, s, neg);
+        else launch_ax8bg<T, 2, true>(E, gid, lat, G, u, y, nb, ld, rb, s, neg);
       } else {
-        if (eb == 1) launch_ax8bg<T, 1, false>(E, gid, lat, G, u, y, nb, ld, rb, s);
-        else launch_ax8bg<T, 2, false>(E, gid, lat, G, u, y, nb, ld, rb, s);
+        if (eb == 1) launch_ax8bg<T, 1, false>(E, gid, lat, G, u, y, nb, ld, rb, s, neg);
+        else launch_ax8bg<T, 2, false>(E, gid, lat, G, u, y, nb, ld, rb, s, neg);
       }
     }
     return;
   }
   if (pair) {
     if (im) {
-      if (eb == 1) launch_ax8b2<T, 1, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
-      else launch_ax8b2<T, 2, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
+      if (eb == 1) launch_ax8b2<T, 1, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
+      else launch_ax8b2<T, 2, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
     } else {
-      if (eb == 1) launch_ax8b2<T, 1, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
-      else launch_ax8b2<T, 2, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
+      if (eb == 1) launch_ax8b2<T, 1, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
+      else launch_ax8b2<T, 2, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
     }
     return;
   }
   if (im) {
-    if (eb == 1) launch_ax8b<T, 1, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
-    else if (eb == 4) launch_ax8b<T, 4, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
-    else launch_ax8b<T, 2, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
+    if (eb == 1) launch_ax8b<T, 1, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
+    else if (eb == 4) launch_ax8b<T, 4, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
+    else launch_ax8b<T, 2, true>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
   } else {
-    if (eb == 1) launch_ax8b<T, 1, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
-    else if (eb == 4) launch_ax8b<T, 4, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
-    else launch_ax8b<T, 2, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s);
+    if (eb == 1) launch_ax8b<T, 1, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
+    else if (eb == 4) launch_ax8b<T, 4, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
+    else launch_ax8b<T, 2, false>(E, gid, lat, G, u, y, err, nb, ld, rb, s, neg);
   }
 }
 
@@ -1002,12 +1006,12 @@ template bool sem_ax8_batched_fits<double>(int);
 template bool sem_ax8_variant_fits<float>(int);
 template bool sem_ax8_variant_fits<double>(int);
 template void sem_ax8<float>(int64_t, const uint32_t*, const Lattice&, const float*, const float*, float*,
-                             unsigned*, int, cudaStream_t);
+                             unsigned*, int, cudaStream_t, bool);
 template void sem_ax8<double>(int64_t, const uint32_t*, const Lattice&, const double*, const double*, double*,
-                              unsigned*, int, cudaStream_t);
+                              unsigned*, int, cudaStream_t, bool);
 template void sem_ax8_batched<float>(int64_t, const uint32_t*, const Lattice&, const float*, const float*, float*,
-                                     unsigned*, int, int, int64_t, cudaStream_t);
+                                     unsigned*, int, int, int64_t, cudaStream_t, bool);
 template void sem_ax8_batched<double>(int64_t, const uint32_t*, const Lattice&, const double*, const double*,
-                                      double*, unsigned*, int, int, int64_t, cudaStream_t);
+                                      double*, unsigned*, int, int, int64_t, cudaStream_t, bool);
 
 }  // namespace chebmg
