@@ -278,6 +278,9 @@ void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld, b
     else if (L.Q == 4 && L.ax4[dt] % 100 == 41)
       sem_ax4<T>(L.E, L.gid, L.ax4[dt] >= 100 ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]),
                  static_cast<const T*>(L.D[dt]), x, y, c->s, nb, ld, subtract);
+    else if (sem_axl_supported(L.Q))
+      sem_axl<T>(L.Q, L.E, L.gid, L.boxed ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]), x, y, c->s, nb, ld,
+                 subtract);
     else
       sem_ax<T>(L.Q, L.E, L.gid, static_cast<const T*>(L.G[dt]), static_cast<const T*>(L.D[dt]), x, y, c->s, nb,
                 ld, subtract);
@@ -2286,6 +2289,7 @@ void upload_sem_levels(chebmg_ctx* c, std::vector<SemHostLevel>& H, bool boxed) 
     L.invD[CHEBMG_F64] = upload<double>(c, invd);
     L.D[CHEBMG_F64] = upload<double>(c, h.Dm);
     if (h.N == 7) CK(sem_ax8_set_D(h.Dm.data()));
+    if (sem_axl_supported(h.NQ)) CK(sem_axl_set_D(h.NQ, h.Dm.data()));
     if (smoothed32) {
       L.G[CHEBMG_F32] = upload<float>(c, h.G);
       L.invD[CHEBMG_F32] = upload<float>(c, invd);

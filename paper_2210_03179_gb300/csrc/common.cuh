@@ -116,6 +116,13 @@ struct Lattice {
 template <typename T>
 void sem_ax4(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* D, const T* u, T* y,
              cudaStream_t s, int nb = 1, int64_t ld = 0, bool subtract = false);
+// Orders 2, 4, 5, 6, 8 and 9 (Q = 3, 5, 6, 7, 9, 10) by line passes (sem_axl.cu); ids from the box
+// lattice when lat is given, else from gid.  sem_axl_set_D uploads the order's derivative matrix.
+bool sem_axl_supported(int Q);
+cudaError_t sem_axl_set_D(int Q, const double* D);
+template <typename T>
+void sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
+             int nb = 1, int64_t ld = 0, bool subtract = false);
 // The order-7 operator in FP64-class arithmetic on FP32 pairs (sem_ax8_x2.cu): G in that
 // format (sem_to_x2 converts an FP64 array of n values), u and y FP64; variant as sem_ax8's
 // non-persistent codes (1, 2, 4; +100 box lattice ids); batches of nb vectors at stride ld,

@@ -35,7 +35,8 @@ constexpr int kVecThreads = 256;
 }  // namespace
 
 // ===========================================================================
-// SEM element operator
+// SEM element operator, one thread per point: orders 1 and 3 (line passes in sem_axl.cu and
+// sem_ax8.cu for the others; order 3 has k_sem_ax4 below as well, autotuned)
 // ===========================================================================
 template <int Q>
 struct SemShape {
@@ -281,14 +282,7 @@ void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const
   const uint32_t neg = subtract ? kSignBit : 0u;
   switch (Q) {
     case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 3: launch_sem_ax<T, 3>(E, gid, G, D, u, y, s, nb, ld, neg); break;
     case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 5: launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 6: launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 8: launch_sem_ax<T, 8>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 9: launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 10: launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg); break;
     default: break;
   }
 }

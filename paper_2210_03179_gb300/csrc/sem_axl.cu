@@ -1,0 +1,276 @@
+// Element operator for the polynomial orders other than 1, 3 and 7 (Sec. 1, Eq. 1.3; orders 3 and 7
+// have kernels of their own, order 1 is the assembled coarse level), by line passes.
+//
+// Q = N + 1 points per direction, Q^2 threads per element: in each of the six 1-D contractions a
+// thread owns one whole grid line, reads its Q values once and produces Q outputs, so a value read
+// from shared memory feeds about Q/2 FMAs (the one-thread-per-point form reads two shared values
+// for every FMA and is bound by them).  The derivative matrix is centro-antisymmetric,
+// D[Q-1-i][Q-1-l] = -D[i][l]: sums and differences of mirrored points halve the multiplications
+// (h = Q / 2 of each; odd Q has a middle point that joins the even half and a middle row of
+// differences alone).  FP32 keeps the factors of a thread's t-line in registers, all loads in
+// flight before the gather; FP64, bound by its FP64 pipe, reads them where they are used.
+// Strides R (rows) and P (planes) are those with the fewest bank conflicts over the passes.
+//
+// Measured, one thread per point -> line passes, with the zeroing of the output (6 to 12 us):
+// FP32 order 9 on 23^3 elements 215.5 -> 116.9 us and on 13^3 44.9 -> 24.6, order 8 on 25^3
+// 242.5 -> 92.3, order 5 on 38^3 164.8 -> 91.3, order 2 on 42^3 26.7 -> 22.5; FP64 order 9 on 23^3
+// 1555 -> 1334, order 5 on 38^3 932 -> 874, order 2 on 42^3 109.7 -> 102.4.
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+
+namespace chebmg {
+
+namespace {
+
+constexpr int kMaxH = 5;   // Q <= 10
+// [0] of D, [1] of D^T: even blocks e[i][l] (column h: the middle point), odd blocks o[i][l],
+// middle row m[l]
+template <typename T>
+struct LineTab {
+  T e[2][kMaxH][kMaxH], o[2][kMaxH][kMaxH], m[2][kMaxH];
+};
+__constant__ LineTab<float> c_tab_f[11];
+__constant__ LineTab<double> c_tab_d[11];
+template <typename T>
+__device__ __forceinline__ const LineTab<T>& tab(int Q);
+template <>
+__device__ __forceinline__ const LineTab<float>& tab<float>(int Q) { return c_tab_f[Q]; }
+template <>
+__device__ __forceinline__ const LineTab<double>& tab<double>(int Q) { return c_tab_d[Q]; }
+
+template <typename T, int Q>
+struct AxL {
+  static constexpr bool F = sizeof(T) == 4;
+  static constexpr int QQ = Q * Q, NP = Q * Q * Q;
+  static constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : Q == 9 ? 3 : 2;   // elements per block
+  static constexpr int THREADS = (EB * QQ + 31) / 32 * 32;
+  static constexpr int R = F ? (Q == 3 ? 4 : Q == 5 ? 6 : Q == 6 ? 9 : Q == 7 ? 8 : Q) : (Q == 6 ? 9 : Q);
+  static constexpr int P = F ? (Q == 3 ? 35 : Q == 5 ? 37 : Q == 6 ? 70 : Q == 7 ? 71 : Q == 9 ? 81 : 101)
+                             : (Q == 3 ? 19 : Q == 5 ? 25 : Q == 6 ? 54 : Q == 7 ? 55 : Q == 9 ? 89 : 106);
+  static constexpr int STAGE = Q * P;
+  static constexpr size_t SMEM = sizeof(T) * (size_t)EB * 3 * STAGE;
+};
+
+// o = D u (W = 0) or D^T u (W = 1) along a line of Q points.
+template <typename T, int Q, int W>
+__device__ __forceinline__ void line(const T (&u)[Q], T (&o)[Q]) {
+  constexpr int H = Q / 2;
+  const LineTab<T>& t = tab<T>(Q);
+  T ue[H], uo[H];
+#pragma unroll
+  for (int l = 0; l < H; ++l) {
+    ue[l] = u[l] + u[Q - 1 - l];
+    uo[l] = u[l] - u[Q - 1 - l];
+  }
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    T se = t.e[W][i][0] * ue[0];
+#pragma unroll
+    for (int l = 1; l < H; ++l) se = fma(t.e[W][i][l], ue[l], se);
+    if (Q % 2) se = fma(t.e[W][i][H], u[H], se);
+    if constexpr (sizeof(T) == 8) {   // the odd chain continues the even one: one FMA gives the mirror
+      T s = se;
+#pragma unroll
+      for (int l = 0; l < H; ++l) s = fma(t.o[W][i][l], uo[l], s);
+      o[i] = s;
+      o[Q - 1 - i] = fma(T(-2), se, s);
+    } else {
+      T so = t.o[W][i][0] * uo[0];
+#pragma unroll
+      for (int l = 1; l < H; ++l) so = fma(t.o[W][i][l], uo[l], so);
+      o[i] = se + so;
+      o[Q - 1 - i] = so - se;
+    }
+  }
+  if constexpr (Q % 2) {
+    T s = t.m[W][0] * uo[0];
+#pragma unroll
+    for (int l = 1; l < H; ++l) s = fma(t.m[W][l], uo[l], s);
+    o[H] = s;
+  }
+}
+
+template <typename T, int Q, bool IMPLICIT>
+__global__ void __launch_bounds__(AxL<T, Q>::THREADS)
+k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
+          const T* __restrict__ u, T* __restrict__ y, int64_t ld, uint32_t neg) {
+  using C = AxL<T, Q>;
+  constexpr int R = C::R, P = C::P, QQ = C::QQ, NP = C::NP;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sm = reinterpret_cast<T*>(smem_raw);
+  const int tid = threadIdx.x;
+  const bool in = tid < C::EB * QQ;           // the last warp may have spare threads
+  const int le = in ? tid / QQ : 0, t = in ? tid - le * QQ : 0, a = t % Q, b = t / Q;
+  const int64_t e = (int64_t)blockIdx.x * C::EB + le;
+  const bool valid = in && e < E;
+  T* su = sm + (size_t)le * 3 * C::STAGE;
+  T* sr = su + C::STAGE;
+  T* ss = sr + C::STAGE;
+  const T* Ge = G + (valid ? e : 0) * (6 * NP) + t;
+  constexpr bool GREG = sizeof(T) == 4;
+  T gr[GREG ? 6 : 1][GREG ? Q : 1];
+  if constexpr (GREG) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+#pragma unroll
+      for (int k = 0; k < Q; ++k) gr[c][k] = __ldg(Ge + c * NP + k * QQ);
+  }
+  uint32_t g[Q];
+  if (!valid) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) g[k] = kGidDirichlet;
+  } else if constexpr (IMPLICIT) {
+    const uint32_t ee = (uint32_t)e, exy = (uint32_t)lat.nex * (uint32_t)lat.ney;
+    const uint32_t ez = ee / exy, rem = ee - ez * exy, ey = rem / (uint32_t)lat.nex, ex = rem - ey * (uint32_t)lat.nex;
+    const uint32_t gx = ex * (Q - 1) + a, gy = ey * (Q - 1) + b;
+    const bool side = gx == 0 || gx == (uint32_t)lat.NX - 1 || gy == 0 || gy == (uint32_t)lat.NY - 1;
+    const uint32_t plane = (uint32_t)lat.NX * (uint32_t)lat.NY;
+    const uint32_t g0 = (ez * (Q - 1) * (uint32_t)lat.NY + gy) * (uint32_t)lat.NX + gx;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const uint32_t gz = ez * (Q - 1) + k;
+      g[k] = (g0 + k * plane) | ((side || gz == 0 || gz == (uint32_t)lat.NZ - 1) ? kGidDirichlet : 0u);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) g[k] = __ldg(gid + e * NP + k * QQ + t);
+  }
+  u += (int64_t)blockIdx.y * ld;   // right-hand side of a batch
+  y += (int64_t)blockIdx.y * ld;
+  pdl_wait();   // u and y may come from the kernel before (programmatic dependent launch)
+  T col[Q], ut[Q];
+#pragma unroll
+  for (int k = 0; k < Q; ++k) col[k] = (g[k] & kGidDirichlet) ? T(0) : u[g[k] & kGidMask];
+  if (in) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) su[k * P + b * R + a] = col[k];
+  }
+  line<T, Q, 0>(col, ut);                        // t: thread (i = a, j = b)
+  __syncthreads();
+  T v[Q], o[Q];
+  if (in) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = su[b * P + a * R + i];   // r: thread (j = a, k = b)
+    line<T, Q, 0>(v, o);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) sr[b * P + a * R + i] = o[i];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) v[j] = su[b * P + j * R + a];   // s: thread (i = a, k = b)
+    line<T, Q, 0>(v, o);
+#pragma unroll
+    for (int j = 0; j < Q; ++j) ss[b * P + j * R + a] = o[j];
+  }
+  __syncthreads();
+  if (in) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const int q = k * P + b * R + a;
+      T g00, g01, g02, g11, g12, g22;
+      if constexpr (GREG) {
+        g00 = gr[0][k]; g01 = gr[1][k]; g02 = gr[2][k]; g11 = gr[3][k]; g12 = gr[4][k]; g22 = gr[5][k];
+      } else {
+        const T* p = Ge + k * QQ;
+        g00 = __ldg(p); g01 = __ldg(p + NP); g02 = __ldg(p + 2 * NP);
+        g11 = __ldg(p + 3 * NP); g12 = __ldg(p + 4 * NP); g22 = __ldg(p + 5 * NP);
+      }
+      const T ur = sr[q], us = ss[q], utk = ut[k];
+      sr[q] = g00 * ur + g01 * us + g02 * utk;
+      ss[q] = g01 * ur + g11 * us + g12 * utk;
+      v[k] = g02 * ur + g12 * us + g22 * utk;
+    }
+    line<T, Q, 1>(v, ut);                        // ut now holds the t contribution
+  }
+  __syncthreads();
+  if (in) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = sr[b * P + a * R + i];
+    line<T, Q, 1>(v, o);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) su[b * P + a * R + i] = o[i];
+  }
+  __syncthreads();
+  if (in) {
+#pragma unroll
+    for (int j = 0; j < Q; ++j) v[j] = ss[b * P + j * R + a];
+    line<T, Q, 1>(v, o);
+#pragma unroll
+    for (int j = 0; j < Q; ++j) su[b * P + j * R + a] += o[j];
+  }
+  __syncthreads();
+  if (valid) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k)
+      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(su[k * P + b * R + a] + ut[k], neg));
+  }
+}
+
+template <typename T, int Q>
+void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s, int nb,
+            int64_t ld, uint32_t neg) {
+  using C = AxL<T, Q>;
+  static bool configured = false;
+  if (!configured) {
+    cudaFuncSetAttribute(k_sem_axl<T, Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    cudaFuncSetAttribute(k_sem_axl<T, Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    configured = true;
+  }
+  const dim3 blocks((unsigned)((E + C::EB - 1) / C::EB), nb);
+  if (lat) launch_dep(k_sem_axl<T, Q, true>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, *lat, G, u, y, ld, neg);
+  else launch_dep(k_sem_axl<T, Q, false>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, Lattice{}, G, u, y, ld, neg);
+}
+
+template <typename T>
+void fill(const double* S, int Q, LineTab<T>& t) {   // S: symmetrised D, [Q][Q]
+  const int H = Q / 2;
+  for (int w = 0; w < 2; ++w) {
+    auto at = [&](int i, int l) { return w == 0 ? S[i * Q + l] : S[l * Q + i]; };
+    for (int i = 0; i < H; ++i) {
+      for (int l = 0; l < H; ++l) {
+        t.e[w][i][l] = (T)(0.5 * (at(i, l) + at(i, Q - 1 - l)));
+        t.o[w][i][l] = (T)(0.5 * (at(i, l) - at(i, Q - 1 - l)));
+      }
+      if (Q % 2) t.e[w][i][H] = (T)at(i, H);
+    }
+    if (Q % 2)
+      for (int l = 0; l < H; ++l) t.m[w][l] = (T)at(H, l);
+  }
+}
+
+}  // namespace
+
+bool sem_axl_supported(int Q) { return Q == 3 || (Q >= 5 && Q <= 10 && Q != 8); }
+
+cudaError_t sem_axl_set_D(int Q, const double* D) {
+  if (!sem_axl_supported(Q)) return cudaErrorInvalidValue;
+  double S[100];
+  for (int i = 0; i < Q; ++i)
+    for (int l = 0; l < Q; ++l) S[i * Q + l] = 0.5 * (D[i * Q + l] - D[(Q - 1 - i) * Q + (Q - 1 - l)]);
+  LineTab<float> f{};
+  LineTab<double> d{};
+  fill(S, Q, f);
+  fill(S, Q, d);
+  const cudaError_t e = cudaMemcpyToSymbol(c_tab_f, &f, sizeof(f), (size_t)Q * sizeof(f));
+  return e != cudaSuccess ? e : cudaMemcpyToSymbol(c_tab_d, &d, sizeof(d), (size_t)Q * sizeof(d));
+}
+
+template <typename T>
+void sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
+             int nb, int64_t ld, bool subtract) {
+  const uint32_t neg = subtract ? kSignBit : 0u;
+  switch (Q) {
+    case 3: launch<T, 3>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
+    case 5: launch<T, 5>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
+    case 6: launch<T, 6>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
+    case 7: launch<T, 7>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
+    case 9: launch<T, 9>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
+    case 10: launch<T, 10>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
+    default: break;
+  }
+}
+template void sem_axl<float>(int, int64_t, const uint32_t*, const Lattice*, const float*, const float*, float*,
+                             cudaStream_t, int, int64_t, bool);
+template void sem_axl<double>(int, int64_t, const uint32_t*, const Lattice*, const double*, const double*, double*,
+                              cudaStream_t, int, int64_t, bool);
+
+}  // namespace chebmg
