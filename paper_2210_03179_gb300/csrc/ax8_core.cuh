@@ -11,12 +11,14 @@
 
 #include <cstdint>
 
+#include "common.cuh"
+
 namespace chebmg {
 namespace {
 
 // even-odd blocks: [0] E of D, [1] O of D, [2] E of D^T, [3] O of D^T, each [i][l], i,l < 4
 __constant__ float c_eo_f[4][4][4];
-__constant__ double c_eo_d[4][4][4];
+__device__ double g_eo_d[64];
 
 template <typename T, int EB_ = 2>
 struct Ax8 {
@@ -28,44 +30,77 @@ struct Ax8 {
   static size_t smem_bytes() { return sizeof(T) * (size_t)EB * (GELEM + 3 * STAGE); }
 };
 
+// The line coefficients as a kernel uses them: FP32 constant-bank operands; FP64 in shared memory
+// (an FP64 FMA issues faster with register operands than with constant ones, see Fp64Unit), rows
+// loaded 16 bytes at a time where they are used.  Every thread of the block calls the constructor,
+// and a block barrier separates it from the first line8.
 template <typename T>
-__device__ __forceinline__ T eo(int w, int i, int l);
+struct Coef8;
 template <>
-__device__ __forceinline__ float eo<float>(int w, int i, int l) { return c_eo_f[w][i][l]; }
+struct Coef8<float> : Arith<float> {
+  static constexpr int SHARED = 1;
+  __device__ __forceinline__ explicit Coef8(float*) {}
+  template <int W>
+  __device__ __forceinline__ void row(int i, float (&v)[4]) const {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) v[l] = c_eo_f[W][i][l];
+  }
+};
 template <>
-__device__ __forceinline__ double eo<double>(int w, int i, int l) { return c_eo_d[w][i][l]; }
+struct Coef8<double> : Arith<double> {
+  static constexpr int SHARED = 64;
+  const double* t;
+  __device__ __forceinline__ explicit Coef8(double* sh) : t(sh) {
+    for (int q = threadIdx.x; q < 64; q += blockDim.x) sh[q] = __ldg(&g_eo_d[q]);
+  }
+  template <int W>
+  __device__ __forceinline__ void row(int i, double (&v)[4]) const {
+    const double2* p = reinterpret_cast<const double2*>(t + W * 16 + i * 4);
+    const double2 a = p[0], b = p[1];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+  }
+};
 
 // o = D u (W = 0) or o = D^T u (W = 1) along one line of 8 points.
 template <typename T, int W>
-__device__ __forceinline__ void line8(const T (&u)[8], T (&o)[8]) {
+__device__ __forceinline__ void line8(const Coef8<T>& c, const T (&u)[8], T (&o)[8]) {
   T ue[4], uo[4];
 #pragma unroll
   for (int l = 0; l < 4; ++l) {
-    ue[l] = u[l] + u[7 - l];
-    uo[l] = u[l] - u[7 - l];
+    ue[l] = c.add(u[l], u[7 - l]);
+    uo[l] = c.sub(u[l], u[7 - l]);
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    T se = eo<T>(2 * W, i, 0) * ue[0];
+    T e[4], d[4];
+    c.template row<2 * W>(i, e);
+    c.template row<2 * W + 1>(i, d);
+    T se = c.mul(e[0], ue[0]);
 #pragma unroll
-    for (int l = 1; l < 4; ++l) se = fma(eo<T>(2 * W, i, l), ue[l], se);
+    for (int l = 1; l < 4; ++l) se = fma(e[l], ue[l], se);
     if constexpr (sizeof(T) == 8) {
       // FP64 (bound by its FP64 issue rate): the odd chain continues from se, giving
       // o[i] = se + so directly, and o[7-i] = so - se = o[i] - 2 se in one more FMA
       // (9 operations per output pair instead of 10)
       T s = se;
 #pragma unroll
-      for (int l = 0; l < 4; ++l) s = fma(eo<T>(2 * W + 1, i, l), uo[l], s);
+      for (int l = 0; l < 4; ++l) s = fma(d[l], uo[l], s);
       o[i] = s;
-      o[7 - i] = fma(T(-2), se, s);
+      o[7 - i] = fma(c.k.m2, se, s);
     } else {
-      T so = eo<T>(2 * W + 1, i, 0) * uo[0];
+      T so = d[0] * uo[0];
 #pragma unroll
-      for (int l = 1; l < 4; ++l) so = fma(eo<T>(2 * W + 1, i, l), uo[l], so);
+      for (int l = 1; l < 4; ++l) so = fma(d[l], uo[l], so);
       o[i] = se + so;
       o[7 - i] = so - se;
     }
   }
+}
+
+// The three weighted derivatives at a point: (G row) . (ur, us, ut).
+template <typename T>
+__device__ __forceinline__ T dot3(const Coef8<T>& c, T g0, T a0, T g1, T a1, T g2, T a2) {
+  return fma(g2, a2, fma(g1, a1, c.mul(g0, a0)));
 }
 
 __device__ __forceinline__ void ld_row(const float* p, float (&v)[8]) {

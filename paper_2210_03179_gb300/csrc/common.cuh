@@ -71,6 +71,37 @@ enum PostOp { POST_NONE = 0, POST_ALPHA, POST_BETA_CG, POST_SET_RZ_FROM_ZR, POST
 constexpr int kRedBlocks = 1216;   // 152 SMs x 8: partial sums per reduction pass (full occupancy)
 
 #ifdef __CUDACC__
+// FP64 issue forms.  On GB300 an FP64 instruction with three register sources issues at 598 G/s
+// over the whole chip, one with two sources (DADD, DMUL) or with a constant-bank or immediate
+// operand at 504 G/s (measured, any number of threads).  Kernels bound by that pipe therefore take
+// their coefficients from shared memory or registers and add and multiply through the FMA with 1,
+// -0 and -2 that the compiler cannot see as constants (all exact).  FP32 needs none of this.
+// Order-7 operator on 32^3 elements (44 FP64 instructions a point): 1385 -> 1203 us, 613 of the
+// 629 G/s that two FP64 instructions per SM and clock make.
+struct Fp64Unit {
+  double one, nz, m2;
+};
+static __device__ double g_fp64_unit[3] = {1.0, -0.0, -2.0};
+__device__ __forceinline__ Fp64Unit fp64_unit() {
+  return {__ldg(&g_fp64_unit[0]), __ldg(&g_fp64_unit[1]), __ldg(&g_fp64_unit[2])};
+}
+template <typename T>
+struct Arith;
+template <>
+struct Arith<float> {
+  __device__ __forceinline__ Arith() {}
+  __device__ __forceinline__ float add(float a, float b) const { return a + b; }
+  __device__ __forceinline__ float sub(float a, float b) const { return a - b; }
+  __device__ __forceinline__ float mul(float a, float b) const { return a * b; }
+};
+template <>
+struct Arith<double> {
+  Fp64Unit k;
+  __device__ __forceinline__ Arith() : k(fp64_unit()) {}
+  __device__ __forceinline__ double add(double a, double b) const { return fma(a, k.one, b); }
+  __device__ __forceinline__ double sub(double a, double b) const { return fma(b, -k.one, a); }
+  __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, k.nz); }
+};
 // v, or -v when neg is the sign bit: one integer operation, exact (an FP64 multiplication would
 // go through the slow FP64 pipe).
 __device__ __forceinline__ float flip_sign(float v, uint32_t neg) { return __uint_as_float(__float_as_uint(v) ^ neg); }

@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(kAx4Threads)
 k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
           const T* __restrict__ Dg, const T* __restrict__ u, T* __restrict__ y, int64_t ld, uint32_t neg) {
   constexpr int PK = kAx4Plane, EL = 4 * kAx4Plane;
+  const Arith<T> ar;
   __shared__ __align__(16) T sU[kAx4Threads / 16][EL];
   __shared__ __align__(16) T sR[kAx4Threads / 16][EL];
   __shared__ __align__(16) T sS[kAx4Threads / 16][EL];
@@ -188,7 +189,7 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     su[k * PK + b * 4 + a] = col[k];
-    T acc = D[k][0] * col[0];
+    T acc = ar.mul(D[k][0], col[0]);
 #pragma unroll
     for (int l = 1; l < 4; ++l) acc = fma(D[k][l], col[l], acc);
     ut[k] = acc;
@@ -200,7 +201,7 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     for (int l = 0; l < 4; ++l) v[l] = su[b * PK + a * 4 + l];         // r-line (j = a, k = b)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      T acc = D[i][0] * v[0];
+      T acc = ar.mul(D[i][0], v[0]);
 #pragma unroll
       for (int l = 1; l < 4; ++l) acc = fma(D[i][l], v[l], acc);
       sr[b * PK + a * 4 + i] = acc;
@@ -209,7 +210,7 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     for (int l = 0; l < 4; ++l) v[l] = su[b * PK + l * 4 + a];         // s-line (i = a, k = b)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      T acc = D[j][0] * v[0];
+      T acc = ar.mul(D[j][0], v[0]);
 #pragma unroll
       for (int l = 1; l < 4; ++l) acc = fma(D[j][l], v[l], acc);
       ss[b * PK + j * 4 + a] = acc;
@@ -221,14 +222,14 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   for (int k = 0; k < 4; ++k) {                                         // own t-line points
     const int q = k * PK + b * 4 + a;
     const T ur = sr[q], us = ss[q], utk = ut[k];
-    sr[q] = gr[0][k] * ur + gr[1][k] * us + gr[2][k] * utk;
-    ss[q] = gr[1][k] * ur + gr[3][k] * us + gr[4][k] * utk;
-    wt[k] = gr[2][k] * ur + gr[4][k] * us + gr[5][k] * utk;
+    sr[q] = fma(gr[2][k], utk, fma(gr[1][k], us, ar.mul(gr[0][k], ur)));
+    ss[q] = fma(gr[4][k], utk, fma(gr[3][k], us, ar.mul(gr[1][k], ur)));
+    wt[k] = fma(gr[5][k], utk, fma(gr[4][k], us, ar.mul(gr[2][k], ur)));
   }
   T yt[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {                                         // D^T along t
-    T acc = D[0][k] * wt[0];
+    T acc = ar.mul(D[0][k], wt[0]);
 #pragma unroll
     for (int l = 1; l < 4; ++l) acc = fma(D[l][k], wt[l], acc);
     yt[k] = acc;
@@ -240,7 +241,7 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     for (int l = 0; l < 4; ++l) v[l] = sr[b * PK + a * 4 + l];         // D^T along r
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      T acc = D[0][i] * v[0];
+      T acc = ar.mul(D[0][i], v[0]);
 #pragma unroll
       for (int l = 1; l < 4; ++l) acc = fma(D[l][i], v[l], acc);
       su[b * PK + a * 4 + i] = acc;
@@ -253,16 +254,16 @@ k_sem_ax4(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     for (int l = 0; l < 4; ++l) v[l] = ss[b * PK + l * 4 + a];         // D^T along s
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      T acc = D[0][j] * v[0];
+      T acc = ar.mul(D[0][j], v[0]);
 #pragma unroll
       for (int l = 1; l < 4; ++l) acc = fma(D[l][j], v[l], acc);
-      su[b * PK + j * 4 + a] += acc;
+      su[b * PK + j * 4 + a] = ar.add(su[b * PK + j * 4 + a], acc);
     }
   }
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < 4; ++k)
-    if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(su[k * PK + b * 4 + a] + yt[k], neg));
+    if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(ar.add(su[k * PK + b * 4 + a], yt[k]), neg));
 }
 
 template <typename T>

@@ -35,6 +35,8 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   using C = Ax8<T, EB_>;
   constexpr int EB = C::EB, R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   __shared__ __align__(8) uint64_t bar;
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sU = sG + EB * C::GELEM;
@@ -75,18 +77,18 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     su[k * P + b * R + a] = col[k];
   }
   T ut[8];
-  line8<T, 0>(col, ut);
+  line8<T, 0>(cf, col, ut);
   __syncthreads();
   {
     T v[8], o[8];
     // r: thread (j = a, k = b) owns the row along i
     ld_row(su + b * P + a * R, v);
-    line8<T, 0>(v, o);
+    line8<T, 0>(cf, v, o);
     st_row(sr + b * P + a * R, o);
     // s: thread (i = a, k = b) owns the line along j
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = su[b * P + j * R + a];
-    line8<T, 0>(v, o);
+    line8<T, 0>(cf, v, o);
 #pragma unroll
     for (int j = 0; j < 8; ++j) ss[b * P + j * R + a] = o[j];
   }
@@ -113,17 +115,17 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     const T ur = sr[q], us = ss[q], utk = ut[k];
     const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
     const T g11 = gG[1536 + p], g12 = gG[2048 + p], g22 = gG[2560 + p];
-    sr[q] = g00 * ur + g01 * us + g02 * utk;
-    ss[q] = g01 * ur + g11 * us + g12 * utk;
-    wt[k] = g02 * ur + g12 * us + g22 * utk;
+    sr[q] = dot3(cf, g00, ur, g01, us, g02, utk);
+    ss[q] = dot3(cf, g01, ur, g11, us, g12, utk);
+    wt[k] = dot3(cf, g02, ur, g12, us, g22, utk);
   }
   T yt[8];
-  line8<T, 1>(wt, yt);
+  line8<T, 1>(cf, wt, yt);
   __syncthreads();
   {
     T v[8], o[8];
     ld_row(sr + b * P + a * R, v);          // transposed r, thread (j = a, k = b)
-    line8<T, 1>(v, o);
+    line8<T, 1>(cf, v, o);
     st_row(su + b * P + a * R, o);
   }
   __syncthreads();
@@ -131,15 +133,15 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     T v[8], o[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = ss[b * P + j * R + a];   // transposed s, thread (i = a, k = b)
-    line8<T, 1>(v, o);
+    line8<T, 1>(cf, v, o);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) su[b * P + j * R + a] += o[j];
+    for (int j = 0; j < 8; ++j) su[b * P + j * R + a] = cf.add(su[b * P + j * R + a], o[j]);
   }
   __syncthreads();
   if (valid) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const T v = su[k * P + b * R + a] + yt[k];
+      const T v = cf.add(su[k * P + b * R + a], yt[k]);
       if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(v, neg));
     }
   }
@@ -157,6 +159,8 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   using C = Ax8<T, EB_>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   T* sU = reinterpret_cast<T*>(smem_raw);
   T* sR = sU + EB_ * C::STAGE;
   T* sS = sR + EB_ * C::STAGE;
@@ -176,17 +180,17 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     col[k] = (g[k] & kGidDirichlet) ? T(0) : u[g[k] & kGidMask];
     su[k * P + b * R + a] = col[k];
   }
-  T ut[8];
-  line8<T, 0>(col, ut);
   __syncthreads();
+  T ut[8];
+  line8<T, 0>(cf, col, ut);
   {
     T v[8], o[8];
     ld_row(su + b * P + a * R, v);
-    line8<T, 0>(v, o);
+    line8<T, 0>(cf, v, o);
     st_row(sr + b * P + a * R, o);
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = su[b * P + j * R + a];
-    line8<T, 0>(v, o);
+    line8<T, 0>(cf, v, o);
 #pragma unroll
     for (int j = 0; j < 8; ++j) ss[b * P + j * R + a] = o[j];
   }
@@ -200,17 +204,17 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     const T ur = sr[q], us = ss[q], utk = ut[k];
     const T g00 = __ldg(gG + p), g01 = __ldg(gG + 512 + p), g02 = __ldg(gG + 1024 + p);
     const T g11 = __ldg(gG + 1536 + p), g12 = __ldg(gG + 2048 + p), g22 = __ldg(gG + 2560 + p);
-    sr[q] = g00 * ur + g01 * us + g02 * utk;
-    ss[q] = g01 * ur + g11 * us + g12 * utk;
-    wt[k] = g02 * ur + g12 * us + g22 * utk;
+    sr[q] = dot3(cf, g00, ur, g01, us, g02, utk);
+    ss[q] = dot3(cf, g01, ur, g11, us, g12, utk);
+    wt[k] = dot3(cf, g02, ur, g12, us, g22, utk);
   }
   T yt[8];
-  line8<T, 1>(wt, yt);
+  line8<T, 1>(cf, wt, yt);
   __syncthreads();
   {
     T v[8], o[8];
     ld_row(sr + b * P + a * R, v);
-    line8<T, 1>(v, o);
+    line8<T, 1>(cf, v, o);
     st_row(su + b * P + a * R, o);
   }
   __syncthreads();
@@ -218,15 +222,15 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     T v[8], o[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = ss[b * P + j * R + a];
-    line8<T, 1>(v, o);
+    line8<T, 1>(cf, v, o);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) su[b * P + j * R + a] += o[j];
+    for (int j = 0; j < 8; ++j) su[b * P + j * R + a] = cf.add(su[b * P + j * R + a], o[j]);
   }
   __syncthreads();
   if (valid) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const T v = su[k * P + b * R + a] + yt[k];
+      const T v = cf.add(su[k * P + b * R + a], yt[k]);
       if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(v, neg));
     }
   }
@@ -247,6 +251,8 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   __shared__ __align__(8) uint64_t bar[2];
   T* sG = reinterpret_cast<T*>(smem_raw);                 // [NB][EB * GELEM]
   T* sU = sG + NB * EB * C::GELEM;
@@ -297,7 +303,7 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 #pragma unroll
     for (int k = 0; k < 8; ++k) su[k * P + b * R + a] = col[k];
     T ut[8];
-    line8<T, 0>(col, ut);
+    line8<T, 0>(cf, col, ut);
     uint32_t gn[8];
     T cn[8];
     gather(next, gn, cn);        // next batch's loads overlap this batch's work
@@ -305,11 +311,11 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     {
       T v[8], o[8];
       ld_row(su + b * P + a * R, v);
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
       st_row(sr + b * P + a * R, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = su[b * P + j * R + a];
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) ss[b * P + j * R + a] = o[j];
     }
@@ -340,19 +346,19 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
       const T ur = sr[q], us = ss[q], utk = ut[k];
       const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
       const T g11 = gG[1536 + p], g12 = gG[2048 + p], g22 = gG[2560 + p];
-      sr[q] = g00 * ur + g01 * us + g02 * utk;
-      ss[q] = g01 * ur + g11 * us + g12 * utk;
-      wt[k] = g02 * ur + g12 * us + g22 * utk;
+      sr[q] = dot3(cf, g00, ur, g01, us, g02, utk);
+      ss[q] = dot3(cf, g01, ur, g11, us, g12, utk);
+      wt[k] = dot3(cf, g02, ur, g12, us, g22, utk);
     }
     T yt[8];
-    line8<T, 1>(wt, yt);
+    line8<T, 1>(cf, wt, yt);
     __syncthreads();
     // single buffer: every thread has read it (the barrier above), so batch i+1's copy starts
     if (NB == 1 && tid == 0 && next < nbatch) issue(next, 0);
     {
       T v[8], o[8];
       ld_row(sr + b * P + a * R, v);
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
       st_row(su + b * P + a * R, o);
     }
     __syncthreads();
@@ -360,14 +366,14 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
       T v[8], o[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = ss[b * P + j * R + a];
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) su[b * P + j * R + a] += o[j];
+      for (int j = 0; j < 8; ++j) su[b * P + j * R + a] = cf.add(su[b * P + j * R + a], o[j]);
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const T v = su[k * P + b * R + a] + yt[k];
+      const T v = cf.add(su[k * P + b * R + a], yt[k]);
       if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(v, neg));
     }
     __syncthreads();             // stage buffers and this G buffer are free for reuse
@@ -391,6 +397,8 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   __shared__ __align__(8) uint64_t bar;
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sU = sG + EB * C::GELEM;
@@ -432,18 +440,18 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
 #pragma unroll
     for (int k = 0; k < 8; ++k) su[k * P + b * R + a] = col[k];
     T ut[8];
-    line8<T, 0>(col, ut);
+    line8<T, 0>(cf, col, ut);
     T cn[8];
     gather(q + 1, cn);           // next right-hand side's loads overlap this one's work
     __syncthreads();
     {
       T v[8], o[8];
       ld_row(su + b * P + a * R, v);
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
       st_row(sr + b * P + a * R, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = su[b * P + j * R + a];
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) ss[b * P + j * R + a] = o[j];
     }
@@ -472,17 +480,17 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
       const T ur = sr[qq], us = ss[qq], utk = ut[k];
       const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
       const T g11 = gG[1536 + p], g12 = gG[2048 + p], g22 = gG[2560 + p];
-      sr[qq] = g00 * ur + g01 * us + g02 * utk;
-      ss[qq] = g01 * ur + g11 * us + g12 * utk;
-      wt[k] = g02 * ur + g12 * us + g22 * utk;
+      sr[qq] = dot3(cf, g00, ur, g01, us, g02, utk);
+      ss[qq] = dot3(cf, g01, ur, g11, us, g12, utk);
+      wt[k] = dot3(cf, g02, ur, g12, us, g22, utk);
     }
     T yt[8];
-    line8<T, 1>(wt, yt);
+    line8<T, 1>(cf, wt, yt);
     __syncthreads();
     {
       T v[8], o[8];
       ld_row(sr + b * P + a * R, v);
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
       st_row(su + b * P + a * R, o);
     }
     __syncthreads();
@@ -490,16 +498,16 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
       T v[8], o[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = ss[b * P + j * R + a];
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) su[b * P + j * R + a] += o[j];
+      for (int j = 0; j < 8; ++j) su[b * P + j * R + a] = cf.add(su[b * P + j * R + a], o[j]);
     }
     __syncthreads();
     if (valid) {
       T* yq = y + (int64_t)q * ld;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        const T v = su[k * P + b * R + a] + yt[k];
+        const T v = cf.add(su[k * P + b * R + a], yt[k]);
         if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], flip_sign(v, neg));
       }
     }
@@ -522,6 +530,8 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   T* sU = reinterpret_cast<T*>(smem_raw);
   T* sR = sU + EB * C::STAGE;
   T* sS = sR + EB * C::STAGE;
@@ -555,18 +565,18 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
 #pragma unroll
     for (int k = 0; k < 8; ++k) su[k * P + b * R + a] = col[k];
     T ut[8];
-    line8<T, 0>(col, ut);
+    line8<T, 0>(cf, col, ut);
     T cn[8];
     gather(q + 1, cn);           // next right-hand side's loads overlap this one's work
     __syncthreads();
     {
       T v[8], o[8];
       ld_row(su + b * P + a * R, v);
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
       st_row(sr + b * P + a * R, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = su[b * P + j * R + a];
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) ss[b * P + j * R + a] = o[j];
     }
@@ -581,12 +591,12 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
       wt[k] = gr[2][k] * ur + gr[4][k] * us + gr[5][k] * utk;
     }
     T yt[8];
-    line8<T, 1>(wt, yt);
+    line8<T, 1>(cf, wt, yt);
     __syncthreads();
     {
       T v[8], o[8];
       ld_row(sr + b * P + a * R, v);
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
       st_row(su + b * P + a * R, o);
     }
     __syncthreads();
@@ -594,16 +604,16 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
       T v[8], o[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = ss[b * P + j * R + a];
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) su[b * P + j * R + a] += o[j];
+      for (int j = 0; j < 8; ++j) su[b * P + j * R + a] = cf.add(su[b * P + j * R + a], o[j]);
     }
     __syncthreads();
     if (valid) {
       T* yq = y + (int64_t)q * ld;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        const T v = su[k * P + b * R + a] + yt[k];
+        const T v = cf.add(su[k * P + b * R + a], yt[k]);
         if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], flip_sign(v, neg));
       }
     }
@@ -625,6 +635,8 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   __shared__ __align__(8) uint64_t bar;
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sStage = sG + EB * C::GELEM;   // [2 right-hand sides][3 stages][EB][STAGE]
@@ -673,7 +685,7 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
     for (int h = 0; h < 2; ++h) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) su[h][k * P + b * R + a] = col[h][k];
-      line8<T, 0>(col[h], ut[h]);
+      line8<T, 0>(cf, col[h], ut[h]);
     }
     gather(q + 2, cn[0]);        // the next pair's loads overlap this pair's work
     gather(q + 3, cn[1]);
@@ -682,11 +694,11 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
     for (int h = 0; h < 2; ++h) {
       T v[8], o[8];
       ld_row(su[h] + b * P + a * R, v);
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
       st_row(sr[h] + b * P + a * R, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = su[h][b * P + j * R + a];
-      line8<T, 0>(v, o);
+      line8<T, 0>(cf, v, o);
 #pragma unroll
       for (int j = 0; j < 8; ++j) ss[h][b * P + j * R + a] = o[j];
     }
@@ -717,20 +729,20 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const T ur = sr[h][qq], us = ss[h][qq], utk = ut[h][k];
-        sr[h][qq] = g00 * ur + g01 * us + g02 * utk;
-        ss[h][qq] = g01 * ur + g11 * us + g12 * utk;
-        wt[h][k] = g02 * ur + g12 * us + g22 * utk;
+        sr[h][qq] = dot3(cf, g00, ur, g01, us, g02, utk);
+        ss[h][qq] = dot3(cf, g01, ur, g11, us, g12, utk);
+        wt[h][k] = dot3(cf, g02, ur, g12, us, g22, utk);
       }
     }
     T yt[2][8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) line8<T, 1>(wt[h], yt[h]);
+    for (int h = 0; h < 2; ++h) line8<T, 1>(cf, wt[h], yt[h]);
     __syncthreads();
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       T v[8], o[8];
       ld_row(sr[h] + b * P + a * R, v);
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
       st_row(su[h] + b * P + a * R, o);
     }
     __syncthreads();
@@ -739,9 +751,9 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
       T v[8], o[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = ss[h][b * P + j * R + a];
-      line8<T, 1>(v, o);
+      line8<T, 1>(cf, v, o);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) su[h][b * P + j * R + a] += o[j];
+      for (int j = 0; j < 8; ++j) su[h][b * P + j * R + a] = cf.add(su[h][b * P + j * R + a], o[j]);
     }
     __syncthreads();
     if (valid) {
@@ -751,7 +763,7 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
         T* yq = y + (int64_t)(q + h) * ld;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const T v = su[h][k * P + b * R + a] + yt[h][k];
+          const T v = cf.add(su[h][k * P + b * R + a], yt[h][k]);
           if (!(g[k] & kGidDirichlet)) atomicAdd(&yq[g[k] & kGidMask], flip_sign(v, neg));
         }
       }
@@ -783,7 +795,7 @@ cudaError_t sem_ax8_set_D(const double* D) {
   for (int w = 0; w < 4; ++w)
     for (int i = 0; i < 4; ++i)
       for (int l = 0; l < 4; ++l) f[w][i][l] = (float)h[w][i][l];
-  cudaError_t e = cudaMemcpyToSymbol(c_eo_d, h, sizeof(h));
+  cudaError_t e = cudaMemcpyToSymbol(g_eo_d, h, sizeof(h));
   if (e != cudaSuccess) return e;
   e = cudaMemcpyToSymbol(c_eo_f, f, sizeof(f));
   if (e != cudaSuccess) return e;

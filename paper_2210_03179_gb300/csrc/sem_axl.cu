@@ -14,7 +14,9 @@
 // Measured, one thread per point -> line passes, with the zeroing of the output (6 to 12 us):
 // FP32 order 9 on 23^3 elements 215.5 -> 116.9 us and on 13^3 44.9 -> 24.6, order 8 on 25^3
 // 242.5 -> 92.3, order 5 on 38^3 164.8 -> 91.3, order 2 on 42^3 26.7 -> 22.5; FP64 order 9 on 23^3
-// 1555 -> 1334, order 5 on 38^3 932 -> 874, order 2 on 42^3 109.7 -> 102.4.
+// 1555 -> 1334, order 5 on 38^3 932 -> 874, order 2 on 42^3 109.7 -> 102.4.  Then, with the FP64
+// coefficients in shared memory: order 9 1334 -> 1216 us, order 5 874 -> 833; and with three blocks of
+// the FP32 order-9 form per SM (80 registers, a little spilling): 116.9 -> 105.0 and 24.6 -> 20.0 us.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -23,27 +25,60 @@ namespace chebmg {
 
 namespace {
 
-constexpr int kMaxH = 5;   // Q <= 10
+constexpr int kMaxH = 5, kRow = 6;   // Q <= 10; rows padded to 16-byte multiples
 // [0] of D, [1] of D^T: even blocks e[i][l] (column h: the middle point), odd blocks o[i][l],
 // middle row m[l]
 template <typename T>
 struct LineTab {
-  T e[2][kMaxH][kMaxH], o[2][kMaxH][kMaxH], m[2][kMaxH];
+  T e[2][kMaxH][kRow], o[2][kMaxH][kRow], m[2][kRow];
 };
 __constant__ LineTab<float> c_tab_f[11];
-__constant__ LineTab<double> c_tab_d[11];
-template <typename T>
-__device__ __forceinline__ const LineTab<T>& tab(int Q);
-template <>
-__device__ __forceinline__ const LineTab<float>& tab<float>(int Q) { return c_tab_f[Q]; }
-template <>
-__device__ __forceinline__ const LineTab<double>& tab<double>(int Q) { return c_tab_d[Q]; }
+__device__ LineTab<double> g_tab_d[11];
+
+// The line coefficients as a kernel uses them: FP32 constant-bank operands; FP64 staged in shared
+// memory (register operands issue faster, see Fp64Unit), rows loaded where they are used.  Every
+// thread of the block calls the constructor; a block barrier separates it from the first line.
+template <typename T, int Q>
+struct Coef;
+template <int Q>
+struct Coef<float, Q> : Arith<float> {
+  using Shared = float;
+  __device__ __forceinline__ explicit Coef(float*) {}
+  template <int W, int K>   // K: 0 even, 1 odd, 2 middle
+  __device__ __forceinline__ void row(int i, float (&v)[kRow]) const {
+    const LineTab<float>& t = c_tab_f[Q];
+#pragma unroll
+    for (int l = 0; l < Q / 2 + (K == 0 ? Q % 2 : 0); ++l) v[l] = K == 0 ? t.e[W][i][l] : K == 1 ? t.o[W][i][l] : t.m[W][l];
+  }
+};
+template <int Q>
+struct Coef<double, Q> : Arith<double> {
+  using Shared = LineTab<double>;
+  const Shared* t;
+  __device__ __forceinline__ explicit Coef(Shared* sh) : t(sh) {
+    const double* src = reinterpret_cast<const double*>(&g_tab_d[Q]);
+    for (int q = threadIdx.x; q < (int)(sizeof(Shared) / sizeof(double)); q += blockDim.x)
+      reinterpret_cast<double*>(sh)[q] = __ldg(src + q);
+  }
+  template <int W, int K>
+  __device__ __forceinline__ void row(int i, double (&v)[kRow]) const {
+    const double2* p = reinterpret_cast<const double2*>(K == 0 ? t->e[W][i] : K == 1 ? t->o[W][i] : t->m[W]);
+#pragma unroll
+    for (int l = 0; l < (Q / 2 + (K == 0 ? Q % 2 : 0) + 1) / 2; ++l) {
+      const double2 x = p[l];
+      v[2 * l] = x.x;
+      v[2 * l + 1] = x.y;
+    }
+  }
+};
 
 template <typename T, int Q>
 struct AxL {
   static constexpr bool F = sizeof(T) == 4;
   static constexpr int QQ = Q * Q, NP = Q * Q * Q;
-  static constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : Q == 9 ? 3 : 2;   // elements per block
+  // elements per block: nearly whole warps (FP64 pays for every idle lane of its last warp)
+  static constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : Q == 9 ? 3 : F ? 2 : 5;
+  static constexpr int MINB = Q == 9 ? 2 : Q == 10 && F ? 3 : 1;   // blocks per SM to fit registers for
   static constexpr int THREADS = (EB * QQ + 31) / 32 * 32;
   static constexpr int R = F ? (Q == 3 ? 4 : Q == 5 ? 6 : Q == 6 ? 9 : Q == 7 ? 8 : Q) : (Q == 6 ? 9 : Q);
   static constexpr int P = F ? (Q == 3 ? 35 : Q == 5 ? 37 : Q == 6 ? 70 : Q == 7 ? 71 : Q == 9 ? 81 : 101)
@@ -54,50 +89,56 @@ struct AxL {
 
 // o = D u (W = 0) or D^T u (W = 1) along a line of Q points.
 template <typename T, int Q, int W>
-__device__ __forceinline__ void line(const T (&u)[Q], T (&o)[Q]) {
+__device__ __forceinline__ void line(const Coef<T, Q>& c, const T (&u)[Q], T (&o)[Q]) {
   constexpr int H = Q / 2;
-  const LineTab<T>& t = tab<T>(Q);
   T ue[H], uo[H];
 #pragma unroll
   for (int l = 0; l < H; ++l) {
-    ue[l] = u[l] + u[Q - 1 - l];
-    uo[l] = u[l] - u[Q - 1 - l];
+    ue[l] = c.add(u[l], u[Q - 1 - l]);
+    uo[l] = c.sub(u[l], u[Q - 1 - l]);
   }
 #pragma unroll
   for (int i = 0; i < H; ++i) {
-    T se = t.e[W][i][0] * ue[0];
+    T e[kRow], d[kRow];
+    c.template row<W, 0>(i, e);
+    c.template row<W, 1>(i, d);
+    T se = c.mul(e[0], ue[0]);
 #pragma unroll
-    for (int l = 1; l < H; ++l) se = fma(t.e[W][i][l], ue[l], se);
-    if (Q % 2) se = fma(t.e[W][i][H], u[H], se);
+    for (int l = 1; l < H; ++l) se = fma(e[l], ue[l], se);
+    if (Q % 2) se = fma(e[H], u[H], se);
     if constexpr (sizeof(T) == 8) {   // the odd chain continues the even one: one FMA gives the mirror
       T s = se;
 #pragma unroll
-      for (int l = 0; l < H; ++l) s = fma(t.o[W][i][l], uo[l], s);
+      for (int l = 0; l < H; ++l) s = fma(d[l], uo[l], s);
       o[i] = s;
-      o[Q - 1 - i] = fma(T(-2), se, s);
+      o[Q - 1 - i] = fma(c.k.m2, se, s);
     } else {
-      T so = t.o[W][i][0] * uo[0];
+      T so = d[0] * uo[0];
 #pragma unroll
-      for (int l = 1; l < H; ++l) so = fma(t.o[W][i][l], uo[l], so);
+      for (int l = 1; l < H; ++l) so = fma(d[l], uo[l], so);
       o[i] = se + so;
       o[Q - 1 - i] = so - se;
     }
   }
   if constexpr (Q % 2) {
-    T s = t.m[W][0] * uo[0];
+    T d[kRow];
+    c.template row<W, 2>(0, d);
+    T s = c.mul(d[0], uo[0]);
 #pragma unroll
-    for (int l = 1; l < H; ++l) s = fma(t.m[W][l], uo[l], s);
+    for (int l = 1; l < H; ++l) s = fma(d[l], uo[l], s);
     o[H] = s;
   }
 }
 
 template <typename T, int Q, bool IMPLICIT>
-__global__ void __launch_bounds__(AxL<T, Q>::THREADS)
+__global__ void __launch_bounds__(AxL<T, Q>::THREADS, AxL<T, Q>::MINB)
 k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
           const T* __restrict__ u, T* __restrict__ y, int64_t ld, uint32_t neg) {
   using C = AxL<T, Q>;
   constexpr int R = C::R, P = C::P, QQ = C::QQ, NP = C::NP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) typename Coef<T, Q>::Shared sCoef;
+  const Coef<T, Q> cf(&sCoef);
   T* sm = reinterpret_cast<T*>(smem_raw);
   const int tid = threadIdx.x;
   const bool in = tid < C::EB * QQ;           // the last warp may have spare threads
@@ -146,18 +187,18 @@ k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
 #pragma unroll
     for (int k = 0; k < Q; ++k) su[k * P + b * R + a] = col[k];
   }
-  line<T, Q, 0>(col, ut);                        // t: thread (i = a, j = b)
   __syncthreads();
+  line<T, Q, 0>(cf, col, ut);                    // t: thread (i = a, j = b)
   T v[Q], o[Q];
   if (in) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) v[i] = su[b * P + a * R + i];   // r: thread (j = a, k = b)
-    line<T, Q, 0>(v, o);
+    line<T, Q, 0>(cf, v, o);
 #pragma unroll
     for (int i = 0; i < Q; ++i) sr[b * P + a * R + i] = o[i];
 #pragma unroll
     for (int j = 0; j < Q; ++j) v[j] = su[b * P + j * R + a];   // s: thread (i = a, k = b)
-    line<T, Q, 0>(v, o);
+    line<T, Q, 0>(cf, v, o);
 #pragma unroll
     for (int j = 0; j < Q; ++j) ss[b * P + j * R + a] = o[j];
   }
@@ -175,17 +216,17 @@ k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
         g11 = __ldg(p + 3 * NP); g12 = __ldg(p + 4 * NP); g22 = __ldg(p + 5 * NP);
       }
       const T ur = sr[q], us = ss[q], utk = ut[k];
-      sr[q] = g00 * ur + g01 * us + g02 * utk;
-      ss[q] = g01 * ur + g11 * us + g12 * utk;
-      v[k] = g02 * ur + g12 * us + g22 * utk;
+      sr[q] = fma(g02, utk, fma(g01, us, cf.mul(g00, ur)));
+      ss[q] = fma(g12, utk, fma(g11, us, cf.mul(g01, ur)));
+      v[k] = fma(g22, utk, fma(g12, us, cf.mul(g02, ur)));
     }
-    line<T, Q, 1>(v, ut);                        // ut now holds the t contribution
+    line<T, Q, 1>(cf, v, ut);                    // ut now holds the t contribution
   }
   __syncthreads();
   if (in) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) v[i] = sr[b * P + a * R + i];
-    line<T, Q, 1>(v, o);
+    line<T, Q, 1>(cf, v, o);
 #pragma unroll
     for (int i = 0; i < Q; ++i) su[b * P + a * R + i] = o[i];
   }
@@ -193,15 +234,15 @@ k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   if (in) {
 #pragma unroll
     for (int j = 0; j < Q; ++j) v[j] = ss[b * P + j * R + a];
-    line<T, Q, 1>(v, o);
+    line<T, Q, 1>(cf, v, o);
 #pragma unroll
-    for (int j = 0; j < Q; ++j) su[b * P + j * R + a] += o[j];
+    for (int j = 0; j < Q; ++j) su[b * P + j * R + a] = cf.add(su[b * P + j * R + a], o[j]);
   }
   __syncthreads();
   if (valid) {
 #pragma unroll
     for (int k = 0; k < Q; ++k)
-      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(su[k * P + b * R + a] + ut[k], neg));
+      if (!(g[k] & kGidDirichlet)) atomicAdd(&y[g[k] & kGidMask], flip_sign(cf.add(su[k * P + b * R + a], ut[k]), neg));
   }
 }
 
@@ -251,7 +292,7 @@ cudaError_t sem_axl_set_D(int Q, const double* D) {
   fill(S, Q, f);
   fill(S, Q, d);
   const cudaError_t e = cudaMemcpyToSymbol(c_tab_f, &f, sizeof(f), (size_t)Q * sizeof(f));
-  return e != cudaSuccess ? e : cudaMemcpyToSymbol(c_tab_d, &d, sizeof(d), (size_t)Q * sizeof(d));
+  return e != cudaSuccess ? e : cudaMemcpyToSymbol(g_tab_d, &d, sizeof(d), (size_t)Q * sizeof(d));
 }
 
 template <typename T>

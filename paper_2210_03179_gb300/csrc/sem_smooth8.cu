@@ -353,6 +353,8 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
   using C = Ax8<T, EB>;
   constexpr int R = C::R, P = C::P, NC = 64 * EB;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
+  const Coef8<T> cf(sCoef);
   __shared__ __align__(8) uint64_t ready[2], done[2];
   __shared__ Item sh_item[2];
   T* sG = reinterpret_cast<T*>(smem_raw);   // [2][EB * GELEM], buffer = slot
@@ -501,7 +503,7 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
 #pragma unroll
         for (int k = 0; k < 8; ++k) su[k * P + cb * R + ca] = col[k];
         T ut[8];
-        line8<T, 0>(col, ut);
+        line8<T, 0>(cf, col, ut);
         T nxt[8];
         if (q + 1 < q1) {   // the next right-hand side's values, in flight during this one
           const T* src = srcb + (int64_t)(q + 1) * a.ld;
@@ -512,11 +514,11 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
         {
           T v[8], o[8];
           ld_row(su + cb * P + ca * R, v);
-          line8<T, 0>(v, o);
+          line8<T, 0>(cf, v, o);
           st_row(sr + cb * P + ca * R, o);
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) v[jj] = su[cb * P + jj * R + ca];
-          line8<T, 0>(v, o);
+          line8<T, 0>(cf, v, o);
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) ss[cb * P + jj * R + ca] = o[jj];
         }
@@ -529,17 +531,17 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
           const T ur = sr[qq], us = ss[qq], utk = ut[k];
           const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
           const T g11 = gG[1536 + p], g12 = gG[2048 + p], g22 = gG[2560 + p];
-          sr[qq] = g00 * ur + g01 * us + g02 * utk;
-          ss[qq] = g01 * ur + g11 * us + g12 * utk;
-          wt[k] = g02 * ur + g12 * us + g22 * utk;
+          sr[qq] = dot3(cf, g00, ur, g01, us, g02, utk);
+          ss[qq] = dot3(cf, g01, ur, g11, us, g12, utk);
+          wt[k] = dot3(cf, g02, ur, g12, us, g22, utk);
         }
         T yt[8];
-        line8<T, 1>(wt, yt);
+        line8<T, 1>(cf, wt, yt);
         named_sync(1, NC);
         {
           T v[8], o[8];
           ld_row(sr + cb * P + ca * R, v);
-          line8<T, 1>(v, o);
+          line8<T, 1>(cf, v, o);
           st_row(su + cb * P + ca * R, o);
         }
         named_sync(1, NC);
@@ -547,16 +549,16 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
           T v[8], o[8];
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj) v[jj] = ss[cb * P + jj * R + ca];
-          line8<T, 1>(v, o);
+          line8<T, 1>(cf, v, o);
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) su[cb * P + jj * R + ca] += o[jj];
+          for (int jj = 0; jj < 8; ++jj) su[cb * P + jj * R + ca] = cf.add(su[cb * P + jj * R + ca], o[jj]);
         }
         named_sync(1, NC);
         if (valid) {
           T* Yq = Y + (int64_t)q * a.ld;
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
-            const T v = su[k * P + cb * R + ca] + yt[k];
+            const T v = cf.add(su[k * P + cb * R + ca], yt[k]);
             if (!(g[k] & kGidDirichlet)) atomicAdd(&Yq[g[k] & kGidMask], v);
           }
         }
@@ -665,7 +667,7 @@ bool sem_smooth8<double>(FusedSmooth& a, int variant, cudaStream_t s) {
 cudaError_t sem_smooth8_set_eo(const double* eo) {
   float f[64];
   for (int i = 0; i < 64; ++i) f[i] = (float)eo[i];
-  cudaError_t e = cudaMemcpyToSymbol(c_eo_d, eo, sizeof(double) * 64);
+  cudaError_t e = cudaMemcpyToSymbol(g_eo_d, eo, sizeof(double) * 64);
   if (e != cudaSuccess) return e;
   return cudaMemcpyToSymbol(c_eo_f, f, sizeof(f));
 }
