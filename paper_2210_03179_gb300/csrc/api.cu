@@ -2733,6 +2733,7 @@ int chebmg_set_outer_operator(chebmg_ctx* c, int kind) {
 int chebmg_apply_outer(chebmg_ctx* c, const double* x, double* y) {
   return guard([&]() -> int {
     enter(c);
+    const PdlScope pdl_(c->nb == 1);
     if (!x || !y) throw Error(CHEBMG_EINVAL, "NULL vector");
     zero<double>(c, y, c->L[0].n);
     apply_outer(c, x, y);
@@ -2744,6 +2745,7 @@ int chebmg_apply_outer(chebmg_ctx* c, const double* x, double* y) {
 int chebmg_apply_A(chebmg_ctx* c, int level, int dtype, const void* x, void* y) {
   return guard([&]() -> int {
     enter(c);
+    const PdlScope pdl_(c->nb == 1);
     Level& L = level_checked(c, level);
     check_dtype(c, dtype);
     if (!x || !y) throw Error(CHEBMG_EINVAL, "NULL vector");
@@ -2793,6 +2795,7 @@ int chebmg_smooth(chebmg_ctx* c, int level, int dtype, const void* b, void* x, i
 int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* rc) {
   return guard([&]() -> int {
     enter(c);
+    const PdlScope pdl_(c->nb == 1);
     level_checked(c, level);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
@@ -2806,6 +2809,7 @@ int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* r
 int chebmg_prolong(chebmg_ctx* c, int level, int dtype, const void* zc, void* zf, int accumulate) {
   return guard([&]() -> int {
     enter(c);
+    const PdlScope pdl_(c->nb == 1);
     level_checked(c, level);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
