@@ -230,17 +230,26 @@ const T* invD_of(const Level& L) {
 int64_t ldv(const chebmg_ctx* c, const Level& L) { return c->nb > 1 ? L.ld : L.n; }
 int64_t span(const chebmg_ctx* c, const Level& L) { return c->nb > 1 ? (int64_t)c->nb * L.ld : L.n; }
 
-template <typename T>
-Stencil9<T> stencil(const Level& L) {
-  Stencil9<T> st;
-  for (int q = 0; q < 9; ++q) st.c[q] = (T)L.st[q];
+Stencil9<double> stencil(const Level& L) {
+  Stencil9<double> st;
+  for (int q = 0; q < 9; ++q) st.c[q] = L.st[q];
   return st;
 }
 
+// The scalars, the device error flags and the coarse kernels' control words lie one after another
+// (common_alloc), so that reading them back is one copy; each part starts on a 16-byte boundary.
+constexpr size_t kScalBytes = (sizeof(double) * S_NSLOTS + 15) / 16 * 16, kFlagBytes = sizeof(unsigned) * 4,
+                 kCtlBytes = sizeof(unsigned) * 5;
 void read_scal(chebmg_ctx* c) {
-  CK(cudaMemcpyAsync(c->hscal, c->scal, sizeof(double) * S_NSLOTS, cudaMemcpyDeviceToHost, c->s));
-  if (c->cctl) CK(cudaMemcpyAsync(c->hcctl, c->cctl, sizeof(unsigned) * 5, cudaMemcpyDeviceToHost, c->s));
-  CK(cudaMemcpyAsync(c->hdstat, c->dstat, sizeof(unsigned) * 4, cudaMemcpyDeviceToHost, c->s));
+  CK(cudaMemcpyAsync(c->hscal, c->scal, kScalBytes + kFlagBytes + (c->cctl ? kCtlBytes : 0), cudaMemcpyDeviceToHost,
+                     c->s));
+  CK(cudaStreamSynchronize(c->s));
+}
+
+// The error flags alone; an FD cycle has no kernel that could raise one.
+void read_flags(chebmg_ctx* c) {
+  if (c->type != TYPE_FD)
+    CK(cudaMemcpyAsync(c->hdstat, c->dstat, kFlagBytes + (c->cctl ? kCtlBytes : 0), cudaMemcpyDeviceToHost, c->s));
   CK(cudaStreamSynchronize(c->s));
 }
 
@@ -285,7 +294,7 @@ void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld, b
       sem_ax<T>(L.Q, L.E, L.gid, static_cast<const T*>(L.G[dt]), static_cast<const T*>(L.D[dt]), x, y, c->s, nb,
                 ld, subtract);
   } else {
-    fd_apply<T>(L.mx, L.my, stencil<T>(L), x, y, c->s, nb, ld);
+    fd_apply<T>(L.mx, L.my, stencil(L), x, y, c->s, nb, ld);
   }
   check_launch();
 }
@@ -474,58 +483,49 @@ void smooth_sem(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero, 
   check_launch();
 }
 
+// smooth() on an FD level: one kernel per step, d alternating between VD and VY.
+template <typename T>
+void smooth_fd(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero) {
+  Level& L = c->L[j];
+  const int64_t n = L.n, ld = ldv(c, L);
+  const int nb = c->nb;
+  const PdlScope pdl_(g_pdl || nb == 1);
+  T *r = vec<T>(L, VR), *d = vec<T>(L, VD), *dn = vec<T>(L, VY);
+  const Stencil9<double> st = stencil(L);
+  const Recurrence q = recurrence(c, L, order);
+  // the first step reads b's neighbours and writes x: vectors that overlap take the pointwise start
+  const char *pb = reinterpret_cast<const char*>(b), *px = reinterpret_cast<const char*>(x);
+  const int64_t bytes = (int64_t)sizeof(T) * span(c, L);
+  const bool apart = pb + bytes <= px || px + bytes <= pb;
+  int i = 1;
+  bool set = x_zero;   // x not written yet
+  if (x_zero && order > 1 && apart) {
+    fd_first<T>(L.mx, L.my, st, b, x, r, d, q.c0, q.c1[1], q.c2[1], q.w[0], q.w[1], order == 2, c->s, nb, ld);
+    i = 2;
+    set = false;
+  } else if (x_zero) {
+    smooth_begin<T>(n, b, x, r, d, invD_of<T>(L), q.c0, order == 1, q.w[0], nullptr, c->s, nb, ld);
+  } else {
+    fd_resid<T>(L.mx, L.my, st, b, x, r, d, q.c0, c->s, nb, ld);
+    if (order == 1) axpy<T>(n, q.w[0], d, x, c->s, nb, ld);
+  }
+  for (; i < order; ++i) {
+    const bool last = i + 1 == order, both = i % 2 == 1;
+    const int xmode = !both && !last ? SX_NONE : set ? SX_SET : SX_ADD;
+    fd_step<T>(L.mx, L.my, st, d, dn, r, r, x, q.c1[i], q.c2[i], xmode, both ? q.w[i - 1] : 0.0, q.w[i], last, c->s,
+               nb, ld);
+    if (xmode != SX_NONE) set = false;
+    std::swap(d, dn);
+  }
+  check_launch();
+}
+
 // One smoother application (Algorithm 1 or 2) of the given order on level j.
 template <typename T>
 void smooth(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero) {
   if (smooth_fused<T>(c, j, b, x, order, x_zero, false)) return;
-  Level& L = c->L[j];
-  if (L.type == TYPE_SEM) {
-    smooth_sem<T>(c, j, b, x, order, x_zero, false);
-    return;
-  }
-  const int64_t n = L.n;
-  const int nb = c->nb;
-  const PdlScope pdl_(g_pdl || nb == 1);
-  const int64_t ld = ldv(c, L);
-  T* r = vec<T>(L, VR);
-  T* d = vec<T>(L, VD);
-  T* y = vec<T>(L, VY);
-  const T* S = invD_of<T>(L);
-  const double lmax = L.lmax * c->lscale;
-  zero<T>(c, y, span(c, L));
-  if (!x_zero) apply_into<T>(c, j, x, y);
-  if (c->o.kind == CHEBMG_CHEB_1ST) {
-    const double lmin = lmin_ratio_for(c, order) * lmax;
-    const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin);
-    const double sigma = theta / delta;
-    double rho = 1.0 / sigma;
-    cheb1_init<T>(n, b, x, r, d, y, S, 1.0 / theta, x_zero ? 1 : 0, c->s, nb, ld);
-    for (int i = 1; i < order; ++i) {
-      apply_into<T>(c, j, d, y);
-      const double rho_new = 1.0 / (2.0 * sigma - rho);
-      cheb1_step<T>(n, x, r, d, y, S, rho_new * rho, 2.0 * rho_new / delta, c->s, nb, ld);
-      rho = rho_new;
-    }
-    axpy<T>(n, 1.0, d, x, c->s, nb, ld);
-  } else {
-    const double* beta = (c->o.kind == CHEBMG_CHEB_4TH_OPT) ? kBeta[order - 1] : nullptr;
-    if (!c->beta_ovr.empty() && (int)c->beta_ovr.size() == order) beta = c->beta_ovr.data();
-    // from x = 0 with more than one step, the init writes only d and the first step reads b
-    // for r and writes x (two vector writes and a read fewer than x = 0, r = b in the init)
-    const bool lean = x_zero && order > 1;
-    cheb4_init<T>(n, b, x, r, d, y, S, 4.0 / (3.0 * lmax), lean ? 2 : x_zero ? 1 : 0, c->s, nb, ld);
-    const double beta_k = beta ? beta[order - 1] : 1.0;
-    for (int i = 1; i < order; ++i) {
-      apply_into<T>(c, j, d, y);
-      const double c1 = (2.0 * i - 1.0) / (2.0 * i + 3.0);
-      const double c2 = (8.0 * i + 4.0) / ((2.0 * i + 3.0) * lmax);
-      // the last step also applies the final update x += beta_k d_k (one pass fewer)
-      cheb4_step<T>(n, x, r, d, y, S, beta ? beta[i - 1] : 1.0, c1, c2, c->s, nb, ld,
-                    i + 1 == order ? beta_k : 0.0, lean && i == 1 ? b : nullptr);
-    }
-    if (order == 1 || beta_k == 0.0) axpy<T>(n, beta_k, d, x, c->s, nb, ld);
-  }
-  check_launch();
+  if (c->L[j].type == TYPE_SEM) smooth_sem<T>(c, j, b, x, order, x_zero, false);
+  else smooth_fd<T>(c, j, b, x, order, x_zero);
 }
 
 // rc = P^T rf (level j -> j+1)
@@ -783,33 +783,43 @@ void apply_outer(chebmg_ctx* c, const double* p, double* q) {
   apply_into<double>(c, 0, p, q);
 }
 
+// VB of level j + 1 = P^T (b - A x), r = b - A x already in VR where have_r.
+template <typename T>
+void residual_restrict(chebmg_ctx* c, int j, const T* b, const T* x, bool have_r) {
+  Level& L = c->L[j];
+  Level& C = c->L[j + 1];
+  T *r = vec<T>(L, VR), *rc = vec<T>(C, VB);
+  if (!have_r && L.c_next == 2) {
+    fd_resid_restrict<T>(L.mx, L.my, C.mx, C.my, stencil(L), b, x, rc, c->s, c->nb, ldv(c, L), ldv(c, C));
+    check_launch();
+    return;
+  }
+  if (!have_r) fd_resid<T>(L.mx, L.my, stencil(L), b, x, r, static_cast<T*>(nullptr), 0.0, c->s, c->nb, ldv(c, L));
+  restrict_to<T>(c, j, r, rc);
+}
+
 // z = V-cycle(b) from level j (Eq. 2.2), in precision T.
 template <typename T>
 int vcycle_level(chebmg_ctx* c, int j, const T* b, T* x) {
   if (j == (int)c->L.size() - 1) return coarse<T>(c, b, x);
   Level& L = c->L[j];
   Level& C = c->L[j + 1];
-  // the fused kernel computes the restriction residual in the same launch as the pre-smoother;
-  // the separate SEM kernels leave r = b, from which one more product subtracts A x
+  // the fused kernel computes the restriction residual in the same launch as the pre-smoother; the
+  // separate SEM kernels leave r = b, from which one more product subtracts A x; the FD restriction
+  // by two forms the residual itself
   const bool sem = L.type == TYPE_SEM;
-  T* y = vec<T>(L, VY);
   T* r = vec<T>(L, VR);
   bool have_r = false;
   if (c->pre > 0) {
     have_r = smooth_fused<T>(c, j, b, x, c->pre, true, true);
     if (!have_r && sem) smooth_sem<T>(c, j, b, x, c->pre, true, true);
-    else if (!have_r) smooth<T>(c, j, b, x, c->pre, true);
+    else if (!have_r) smooth_fd<T>(c, j, b, x, c->pre, true);
   } else {
     zero<T>(c, x, span(c, L));
     if (sem) cast<T, T>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
   }
-  if (!have_r && sem) {
-    apply_subtract<T>(c, j, x, r);
-  } else if (!have_r) {
-    apply_into<T>(c, j, x, y);
-    residual<T>(L.n, b, y, r, c->s, c->nb, ldv(c, L));
-  }
-  restrict_to<T>(c, j, r, vec<T>(C, VB));
+  if (!have_r && sem) apply_subtract<T>(c, j, x, r);
+  residual_restrict<T>(c, j, b, x, sem);
   int rc = vcycle_level<T>(c, j + 1, vec<T>(C, VB), vec<T>(C, VX));
   if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
   prolong_to<T>(c, j, vec<T>(C, VX), x, 1);
@@ -910,17 +920,16 @@ void alloc_vectors(chebmg_ctx* c, Level& L, bool with32) {
 }
 
 void common_alloc(chebmg_ctx* c) {
-  c->dstat = dalloc<unsigned>(c, 4);
-  CK(cudaMemsetAsync(c->dstat, 0, sizeof(unsigned) * 4, c->s));
   c->partial = dalloc<double>(c, 2 * kRedBlocks);
-  c->scal = dalloc<double>(c, S_NSLOTS);
-  CK(cudaMemsetAsync(c->scal, 0, sizeof(double) * S_NSLOTS, c->s));
+  constexpr size_t block = kScalBytes + kFlagBytes + kCtlBytes;
+  c->scal = reinterpret_cast<double*>(dalloc<unsigned char>(c, block));
+  c->dstat = reinterpret_cast<unsigned*>(c->scal + kScalBytes / sizeof(double));
+  CK(cudaMemsetAsync(c->scal, 0, block, c->s));
   void* h = nullptr;
-  CK(cudaMallocHost(&h, sizeof(double) * S_NSLOTS));
+  CK(cudaMallocHost(&h, block));
   c->hscal = static_cast<double*>(h);
-  CK(cudaMallocHost(&h, sizeof(unsigned) * 4));
-  c->hdstat = static_cast<unsigned*>(h);
-  std::memset(c->hdstat, 0, sizeof(unsigned) * 4);
+  c->hdstat = reinterpret_cast<unsigned*>(c->hscal + kScalBytes / sizeof(double));
+  std::memset(h, 0, block);
   c->cpartial = dalloc<double>(c, 2 * kRedBlocks);
   c->cscal = dalloc<double>(c, S_NSLOTS);
   CK(cudaMemsetAsync(c->cscal, 0, sizeof(double) * S_NSLOTS, c->s));
@@ -947,11 +956,8 @@ void common_alloc(chebmg_ctx* c) {
     c->coop_ok = coop != 0 && grid > 0;
     if (c->cc_val64)
       c->cc_ok = coarse_cluster_plan(c->cc_nx, c->cc_ny, c->cc_nz, &c->cc_ctas, &c->cc_rmax, &c->cc_smem);
-    c->cctl = dalloc<unsigned>(c, 5);
-    CK(cudaMemsetAsync(c->cctl, 0, sizeof(unsigned) * 5, c->s));
-    CK(cudaMallocHost(&h, sizeof(unsigned) * 5));
-    c->hcctl = static_cast<unsigned*>(h);
-    std::memset(c->hcctl, 0, sizeof(unsigned) * 5);
+    c->cctl = c->dstat + 4;   // zeroed above
+    c->hcctl = c->hdstat + 4;
     c->cpart = dalloc<double>(c, 6 * std::max(1, grid));   // two generations of 3 partials per block
     for (int q = 0; q < 2; ++q) {   // tag 0 (zeroed words) is never used
       c->cexf[q] = dalloc<unsigned long long>(c, nc);
@@ -1238,8 +1244,6 @@ void destroy_ctx(chebmg_ctx* c) {
   for (void* p : c->allocs) cudaFree(p);
   if (c->hscal) cudaFreeHost(c->hscal);
   if (c->hcscal) cudaFreeHost(c->hcscal);
-  if (c->hcctl) cudaFreeHost(c->hcctl);
-  if (c->hdstat) cudaFreeHost(c->hdstat);
   if (c->hbscal) cudaFreeHost(c->hbscal);
   if (c->hbstat) cudaFreeHost(c->hbstat);
   for (auto& g : c->gexec)
@@ -1739,16 +1743,13 @@ int vcycle_store(chebmg_ctx* c, int j, const double* b, double* x) {
   Level& C = c->L[j + 1];
   if (c->pre > 0) smooth<double>(c, j, b, x, c->pre, true);
   else zero<double>(c, x, span(c, L));
-  double* y = vec<double>(L, VY);
-  double* r = vec<double>(L, VR);
-  if (L.type == TYPE_SEM) {
+  const bool sem = L.type == TYPE_SEM;
+  if (sem) {
+    double* r = vec<double>(L, VR);
     cast<double, double>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
     apply_subtract<double>(c, j, x, r);
-  } else {
-    apply_into<double>(c, j, x, y);
-    residual<double>(L.n, b, y, r, c->s, c->nb, ldv(c, L));
   }
-  restrict_to<double>(c, j, r, vec<double>(C, VB));
+  residual_restrict<double>(c, j, b, x, sem);
   const int rc = vcycle_store(c, j + 1, vec<double>(C, VB), vec<double>(C, VX));
   if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
   prolong_to<double>(c, j, vec<double>(C, VX), x, 1);
@@ -2828,9 +2829,8 @@ int chebmg_coarse_solve(chebmg_ctx* c, const double* r, double* z, int* iters) {
     if (!r || !z) throw Error(CHEBMG_EINVAL, "NULL vector");
     reset_coarse_sticky(c);
     int rc = coarse_solve64(c, r, z);
-    CK(cudaStreamSynchronize(c->s));
+    read_flags(c);
     if (c->coop_ok && c->L.back().type == TYPE_SEM) {
-      read_scal(c);
       c->last_coarse_iters = (int)c->hcctl[3];
       const unsigned st = c->hcctl[2];
       rc = st == CS_OK ? CHEBMG_OK : st == CS_NOTCONV ? CHEBMG_ENOTCONV
@@ -2849,7 +2849,7 @@ int chebmg_vcycle(chebmg_ctx* c, const double* r, double* z) {
     reset_coarse_sticky(c);
     int rc = vcycle_top(c, r, z);
     check_launch();
-    read_scal(c);
+    read_flags(c);
     if (rc == CHEBMG_OK || rc == CHEBMG_ENOTCONV) rc = coarse_sticky_error(c);
     return rc;
   });

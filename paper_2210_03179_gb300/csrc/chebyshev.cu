@@ -325,32 +325,6 @@ __global__ void k_axpy(int64_t n, T a, const T* __restrict__ d, T* __restrict__ 
     x[g] += a * d[g];
 }
 
-template <typename T, bool VEC>
-__global__ void k_residual(int64_t n, const T* __restrict__ b, T* __restrict__ y, T* __restrict__ r, int64_t ld) {
-  pdl_wait();
-  { const int64_t off_ = (int64_t)blockIdx.y * ld; b += off_; y += off_; r += off_; }
-  using VT = typename V16<T>::type;
-  constexpr int L = V16<T>::L;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t nv = VEC ? n / L : 0;
-  for (int64_t q = tid; q < nv; q += stride) {
-    const VT bv = reinterpret_cast<const VT*>(b)[q], yv = reinterpret_cast<const VT*>(y)[q];
-    const T* bs = reinterpret_cast<const T*>(&bv);
-    const T* ys = reinterpret_cast<const T*>(&yv);
-    VT rv;
-    T* rs = reinterpret_cast<T*>(&rv);
-#pragma unroll
-    for (int l = 0; l < L; ++l) rs[l] = bs[l] - ys[l];
-    reinterpret_cast<VT*>(r)[q] = rv;
-    reinterpret_cast<VT*>(y)[q] = VT{};
-  }
-  for (int64_t g = nv * L + tid; g < n; g += stride) {
-    r[g] = b[g] - y[g];
-    y[g] = T(0);
-  }
-}
-
-
 template <typename Tin, typename Tout>
 __global__ void k_cast(int64_t n, const Tin* __restrict__ in, Tout* __restrict__ out, int64_t ldi, int64_t ldo) {
   pdl_wait();
@@ -468,16 +442,6 @@ template <typename T>
 void axpy(int64_t n, double a, const T* d, T* x, cudaStream_t s, int nb, int64_t ld) {
   launch_dep(k_axpy<T>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, (T)a, d, x, ld ? ld : n);
 }
-template <typename T>
-void residual(int64_t n, const T* b, T* y, T* r, cudaStream_t s, int nb, int64_t ld) {
-  if (!ld) ld = n;
-  const uintptr_t align = (uintptr_t)b | (uintptr_t)y | (uintptr_t)r;
-  if (align % 16 == 0 && (nb == 1 || (ld * sizeof(T)) % 16 == 0))
-    launch_dep(k_residual<T, true>, dim3(grid_for(n / V16<T>::L + 1, kVecThreads), nb), dim3(kVecThreads), 0, s, n,
-               b, y, r, ld);
-  else
-    launch_dep(k_residual<T, false>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, b, y, r, ld);
-}
 template <typename Tin, typename Tout>
 void cast(int64_t n, const Tin* in, Tout* out, cudaStream_t s, int nb, int64_t ldi, int64_t ldo) {
   launch_dep(k_cast<Tin, Tout>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, in, out,
@@ -504,8 +468,7 @@ void masked_copy(int64_t n, const double* in, const double* invD, double* out, c
                                   int, int64_t);                                                        \
   template void smooth_step<T>(int64_t, T*, T*, T*, const T*, double, double, int, double, double, bool,      \
                                const T*, cudaStream_t, int, int64_t);                                   \
-  template void axpy<T>(int64_t, double, const T*, T*, cudaStream_t, int, int64_t);                     \
-  template void residual<T>(int64_t, const T*, T*, T*, cudaStream_t, int, int64_t);
+  template void axpy<T>(int64_t, double, const T*, T*, cudaStream_t, int, int64_t);
 
 CHEBMG_CHEB_INST(float)
 CHEBMG_CHEB_INST(double)

@@ -252,10 +252,27 @@ template <typename T>
 void prolong_box(int Qf, int Qc, int64_t E, const Lattice& Lf, const Lattice& Lc, const T* zc, T* zf,
                  int accumulate, cudaStream_t s, int nb = 1, int64_t ldf = 0, int64_t ldc = 0);
 
-// ---- FD kernels ----
+// ---- FD kernels (fd.cu); st is the level's operator A ----
 template <typename T>
-void fd_apply(int mx, int my, const Stencil9<T>& st, const T* u, T* y, cudaStream_t s, int nb = 1,
+void fd_apply(int mx, int my, const Stencil9<double>& st, const T* u, T* y, cudaStream_t s, int nb = 1,
               int64_t ld = 0);
+// The steps of Algorithms 1 and 2 in the form of smooth_step below, S = 1 / st.c[4] inside.
+// From a zero guess: d_0 = c0 S b, r = b - A d_0, d = c1 d_0 + c2 S r, x = w0 d_0 + w1 d.
+template <typename T>
+void fd_first(int mx, int my, const Stencil9<double>& st, const T* b, T* x, T* r, T* d, double c0, double c1, double c2,
+              double w0, double w1, bool last, cudaStream_t s, int nb, int64_t ld);
+// r = rin - A d, dn = c1 d + c2 S r, x = or += w0 d + w1 dn (xmode); last: x alone.  dn is not d.
+template <typename T>
+void fd_step(int mx, int my, const Stencil9<double>& st, const T* d, T* dn, const T* rin, T* r, T* x, double c1,
+             double c2, int xmode, double w0, double w1, bool last, cudaStream_t s, int nb, int64_t ld);
+// r = b - A x, and d = c0 S r unless d is null.
+template <typename T>
+void fd_resid(int mx, int my, const Stencil9<double>& st, const T* b, const T* x, T* r, T* d, double c0, cudaStream_t s,
+              int nb, int64_t ld);
+// rc = P^T (b - A x), coarsening by two.
+template <typename T>
+void fd_resid_restrict(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* b, const T* x, T* rc,
+                       cudaStream_t s, int nb, int64_t ldf, int64_t ldc);
 template <typename T>
 void fd_restrict(int mfx, int mfy, int mcx, int mcy, int c, const T* rf, T* rc, cudaStream_t s, int nb = 1,
                  int64_t ldf = 0, int64_t ldc = 0);
@@ -304,9 +321,6 @@ void smooth_step(int64_t n, T* x, T* r, T* d, const T* invD, double c1, double c
 // x += a * d
 template <typename T>
 void axpy(int64_t n, double a, const T* d, T* x, cudaStream_t s, int nb = 1, int64_t ld = 0);
-// r = b - y; y = 0
-template <typename T>
-void residual(int64_t n, const T* b, T* y, T* r, cudaStream_t s, int nb = 1, int64_t ld = 0);
 // Batched forms: nb vectors at leading dimension ld (0 = n); per-node data (S) shared.
 template <typename Tin, typename Tout>
 void cast(int64_t n, const Tin* in, Tout* out, cudaStream_t s, int nb = 1, int64_t ldi = 0, int64_t ldo = 0);

@@ -1,0 +1,384 @@
+// Finite-difference kernels (Sec. 3): a constant 3x3 stencil per level (five points on the finest
+// grid, Galerkin nine-point below), its transfers, and the steps of Algorithms 1 and 2 with the
+// stencil inside.
+//
+// Grids up to a few hundred points a side stay in L2, so launches and the FP64 pipe bound these
+// kernels.  A Chebyshev step is one kernel: the stencil of d, the residual update, the recurrence
+// (d out of place, since neighbours read it) and the x update; S = diag(A)^{-1} is one number, so
+// it is folded into the coefficients.  From a zero guess the first step works on b directly
+// (d_0 = c0 S b is never stored), and the restriction residual is formed in shared memory by the
+// restriction itself.  Stencil coefficients are moved into registers (in_register): an FP64 FMA
+// with a constant operand issues slower, and a five-point stencil skips its zero corners.
+// Separate operator and update kernels -> these: order-4 smoothing of 511 x 511 from a nonzero guess
+// 46.2 -> 30.8 us (of which about 15 us FP64 issue), a symmetric order-2 cycle on 63 x 63
+// 96.6 -> 40.6 us (27 -> 11 launches, and the dense coarse product 45.9 us -> a few).
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+
+namespace chebmg {
+
+namespace {
+
+constexpr int kBX = 32, kBY = 8;
+
+// A kernel parameter as a register operand the compiler cannot fold back.  Call it with whole warps.
+__device__ __forceinline__ double in_register(double v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ float in_register(float v) { return v; }
+
+// Which of the nine entries a stencil uses: all, or centre and edges.
+template <bool NINE>
+__device__ __forceinline__ constexpr bool used(int q) {
+  return NINE || q == 4 || (q & 1);
+}
+template <typename T, bool NINE>
+__device__ __forceinline__ void load_stencil(const Stencil9<T>& p, T (&c)[9]) {
+#pragma unroll
+  for (int q = 0; q < 9; ++q) c[q] = used<NINE>(q) ? in_register(p.c[q]) : T(0);
+}
+
+// sum_q c[q] u(neighbour q) at (i, j), zero outside the grid; uc = u(i, j).  The terms cancel, so
+// the caller adds its residual to the finished sum rather than starting the chain with it (which
+// saves one operation and was measured four times less exact).
+template <typename T, bool NINE>
+__device__ __forceinline__ T stencil_sum(const Arith<T>& ar, const T* u, int mx, int my, int i, int j,
+                                         const T (&c)[9], T& uc) {
+  const T* p = u + (int64_t)j * mx + i;
+  T v[9];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    if (!used<NINE>(q)) continue;
+    const int a = q / 3 - 1, b = q % 3 - 1;
+    const bool in = (a == 0 || (a < 0 ? j > 0 : j + 1 < my)) && (b == 0 || (b < 0 ? i > 0 : i + 1 < mx));
+    v[q] = in ? p[a * mx + b] : T(0);
+  }
+  T acc = ar.mul(c[NINE ? 0 : 1], v[NINE ? 0 : 1]);
+#pragma unroll
+  for (int q = NINE ? 1 : 2; q < 9; ++q)
+    if (used<NINE>(q)) acc = fma(c[q], v[q], acc);
+  uc = v[4];
+  return acc;
+}
+
+struct Pt {
+  int i, j;
+  bool in;
+  int64_t g;
+};
+__device__ __forceinline__ Pt point(int mx, int my) {
+  Pt p;
+  p.i = blockIdx.x * kBX + threadIdx.x;
+  p.j = blockIdx.y * kBY + threadIdx.y;
+  p.in = p.i < mx && p.j < my;
+  p.g = (int64_t)p.j * mx + p.i;
+  return p;
+}
+
+// y = A u
+template <typename T, bool NINE>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_apply(int mx, int my, Stencil9<T> st, const T* __restrict__ u, T* __restrict__ y, int64_t ld) {
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);
+  pdl_wait();
+  const Pt p = point(mx, my);
+  if (!p.in) return;
+  const int64_t o = (int64_t)blockIdx.z * ld;   // right-hand side of a batch
+  T uc;
+  y[o + p.g] = stencil_sum<T, NINE>(ar, u + o, mx, my, p.i, p.j, c, uc);
+}
+
+// First step from a zero guess: with d_0 = c0 b (c0 includes S), r = b - A d_0 (st = -c0 A),
+// d = c1 d_0 + c2 r, x = w0 d_0 + w1 d.  last: r and d are not stored.
+template <typename T, bool NINE>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_first(int mx, int my, Stencil9<T> st, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ r,
+           T* __restrict__ d, T c0, T c1, T c2, T w0, T w1, int last, int64_t ld) {
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);
+  pdl_wait();
+  const Pt p = point(mx, my);
+  if (!p.in) return;
+  const int64_t o = (int64_t)blockIdx.z * ld;
+  const T b0 = b[o + p.g];
+  T uc;
+  const T rv = ar.add(stencil_sum<T, NINE>(ar, b + o, mx, my, p.i, p.j, c, uc), b0);
+  const T d0 = c0 * b0, dn = c1 * d0 + c2 * rv;
+  x[o + p.g] = w0 * d0 + w1 * dn;
+  if (last) return;
+  r[o + p.g] = rv;
+  d[o + p.g] = dn;
+}
+
+// One step: r -= A d (st = -A), d' = c1 d + c2 r (c2 includes S), then x = or += w0 d + w1 d'.
+// last: r and d' are not stored.  rin is r, or the residual to start from (r_out = rin - A d).
+template <typename T, bool NINE>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_step(int mx, int my, Stencil9<T> st, const T* __restrict__ d, T* __restrict__ dn, const T* rin, T* r, T* x, T c1,
+          T c2, int xmode, T w0, T w1, int last, int64_t ld) {
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);
+  pdl_wait();
+  const Pt p = point(mx, my);
+  if (!p.in) return;
+  const int64_t o = (int64_t)blockIdx.z * ld + p.g;
+  const T r0 = rin[o], x0 = xmode == SX_ADD ? x[o] : T(0);
+  T dc;
+  const T rv = ar.add(stencil_sum<T, NINE>(ar, d + (int64_t)blockIdx.z * ld, mx, my, p.i, p.j, c, dc), r0);
+  const T v = c1 * dc + c2 * rv;
+  if (xmode != SX_NONE) x[o] = (x0 + w0 * dc) + w1 * v;
+  if (last) return;
+  r[o] = rv;
+  dn[o] = v;
+}
+
+// r = b - A x (st = -A), and d = c0 r where d is given (c0 includes S).
+template <typename T, bool NINE>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_resid(int mx, int my, Stencil9<T> st, const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r,
+           T* __restrict__ d, T c0, int64_t ld) {
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);
+  pdl_wait();
+  const Pt p = point(mx, my);
+  if (!p.in) return;
+  const int64_t o = (int64_t)blockIdx.z * ld;
+  T xc;
+  const T b0 = b[o + p.g];
+  const T rv = ar.add(stencil_sum<T, NINE>(ar, x + o, mx, my, p.i, p.j, c, xc), b0);
+  r[o + p.g] = rv;
+  if (d) d[o + p.g] = c0 * rv;
+}
+
+// rc = P^T (b - A x) for coarsening by two (st = -A): a block forms the residual of the fine points
+// under its tile of coarse points in shared memory (one row and column shared with the next tile).
+constexpr int kTX = 16, kTY = 8;
+template <typename T, bool NINE>
+__global__ void __launch_bounds__(kTX * kTY)
+k_fd_resid_restrict(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* __restrict__ b,
+                    const T* __restrict__ x, T* __restrict__ rc, int64_t ldf, int64_t ldc) {
+  constexpr int FX = 2 * kTX + 1, FY = 2 * kTY + 1;
+  __shared__ T sr[FY][FX + 1];
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);
+  pdl_wait();
+  b += (int64_t)blockIdx.z * ldf;
+  x += (int64_t)blockIdx.z * ldf;
+  rc += (int64_t)blockIdx.z * ldc;
+  const int I0 = blockIdx.x * kTX, J0 = blockIdx.y * kTY;
+  for (int q = threadIdx.x; q < FX * FY; q += kTX * kTY) {
+    const int fi = q % FX, fj = q / FX, i = 2 * I0 + fi, j = 2 * J0 + fj;
+    T v = T(0), xc;
+    if (i < mx && j < my) v = ar.add(stencil_sum<T, NINE>(ar, x, mx, my, i, j, c, xc), b[(int64_t)j * mx + i]);
+    sr[fj][fi] = v;
+  }
+  __syncthreads();
+  const int tx = threadIdx.x % kTX, ty = threadIdx.x / kTX, I = I0 + tx, J = J0 + ty;
+  if (I >= mcx || J >= mcy) return;
+  T acc = T(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const T* row = sr[2 * ty + a] + 2 * tx;
+    const T v = T(0.5) * (row[0] + row[2]) + row[1];
+    acc += (a == 1 ? T(1) : T(0.5)) * v;
+  }
+  rc[(int64_t)J * mcx + I] = acc;
+}
+
+// rc(I,J) = sum_{|a|,|b| < c} w_a w_b rf(c(I+1)-1+b, c(J+1)-1+a), w_d = (c - |d|)/c.  C: the factor
+// when known at compile time (2), else 0.
+template <typename T, int C>
+__global__ void __launch_bounds__(256)
+k_fd_restrict(int mfx, int mfy, int mcx, int mcy, int cr, const T* __restrict__ rf, T* __restrict__ rc, int64_t ldf,
+              int64_t ldc) {
+  pdl_wait();
+  rf += (int64_t)blockIdx.z * ldf;
+  rc += (int64_t)blockIdx.z * ldc;
+  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+  const int Jc = blockIdx.y * blockDim.y + threadIdx.y;
+  if (I >= mcx || Jc >= mcy) return;
+  const int c = C ? C : cr;
+  const int fi = c * (I + 1) - 1, fj = c * (Jc + 1) - 1;
+  const T inv_c = C == 2 ? T(0.5) : T(1) / T(c);
+  T acc = 0;
+#pragma unroll
+  for (int a = -(c - 1); a <= c - 1; ++a) {
+    const int jj = fj + a;
+    if (jj < 0 || jj >= mfy) continue;
+    const T wa = T(c - (a < 0 ? -a : a)) * inv_c;
+    T row = 0;
+#pragma unroll
+    for (int b = -(c - 1); b <= c - 1; ++b) {
+      const int ii = fi + b;
+      if (ii < 0 || ii >= mfx) continue;
+      row += T(c - (b < 0 ? -b : b)) * inv_c * rf[(size_t)jj * mfx + ii];
+    }
+    acc += wa * row;
+  }
+  rc[(size_t)Jc * mcx + I] = acc;
+}
+
+// zf (+)= P zc, bilinear.
+template <typename T, int C>
+__global__ void __launch_bounds__(256)
+k_fd_prolong(int mfx, int mfy, int mcx, int mcy, int cr, const T* __restrict__ zc, T* __restrict__ zf, int accumulate,
+             int64_t ldf, int64_t ldc) {
+  pdl_wait();
+  zf += (int64_t)blockIdx.z * ldf;
+  zc += (int64_t)blockIdx.z * ldc;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= mfx || j >= mfy) return;
+  const int c = C ? C : cr;
+  const T inv_c = C == 2 ? T(0.5) : T(1) / T(c);
+  const int I0 = (i + 1) / c - 1, J0 = (j + 1) / c - 1;
+  const int di = i - (c * (I0 + 1) - 1), dj = j - (c * (J0 + 1) - 1);
+  const T wi[2] = {T(c - di) * inv_c, T(di) * inv_c};
+  const T wj[2] = {T(c - dj) * inv_c, T(dj) * inv_c};
+  T acc = 0;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int Jc = J0 + a;
+    if (Jc < 0 || Jc >= mcy || (a == 1 && dj == 0)) continue;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int I = I0 + b;
+      if (I < 0 || I >= mcx || (b == 1 && di == 0)) continue;
+      acc += wj[a] * wi[b] * zc[(size_t)Jc * mcx + I];
+    }
+  }
+  T* dst = &zf[(size_t)j * mfx + i];
+  *dst = accumulate ? *dst + acc : acc;
+}
+
+// y = M x for a dense row-major n x n matrix, a warp per row (coalesced reads, one shuffle sum); a
+// block's rows are read once for every right-hand side it covers.  (A thread per row read the matrix
+// uncoalesced and summed n products in one chain: 45.9 us at n = 225.)
+constexpr int kDenseWarps = 4;
+__global__ void __launch_bounds__(32 * kDenseWarps)
+k_dense_matvec(int n, const double* __restrict__ M, const double* __restrict__ x, double* __restrict__ y, int nb,
+               int64_t ld) {
+  pdl_wait();
+  const int lane = threadIdx.x & 31, i = blockIdx.x * kDenseWarps + (threadIdx.x >> 5);
+  if (i >= n) return;
+  const double* row = M + (size_t)i * n;
+  for (int q = blockIdx.y; q < nb; q += gridDim.y) {
+    const double* xq = x + (int64_t)q * ld;
+    double a0 = 0.0, a1 = 0.0;
+    int j = lane;
+    for (; j + 32 < n; j += 64) {
+      a0 = fma(row[j], xq[j], a0);
+      a1 = fma(row[j + 32], xq[j + 32], a1);
+    }
+    if (j < n) a0 = fma(row[j], xq[j], a0);
+    a0 += a1;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) a0 += __shfl_down_sync(0xffffffffu, a0, s);
+    if (lane == 0) y[(int64_t)q * ld + i] = a0;
+  }
+}
+
+template <typename T>
+bool nine(const Stencil9<T>& st) {
+  return st.c[0] != T(0) || st.c[2] != T(0) || st.c[6] != T(0) || st.c[8] != T(0);
+}
+template <typename T>
+Stencil9<T> scaled(const Stencil9<double>& st, double f) {
+  Stencil9<T> o;
+  for (int q = 0; q < 9; ++q) o.c[q] = (T)(f * st.c[q]);
+  return o;
+}
+dim3 grid_of(int mx, int my, int nb) { return dim3((mx + kBX - 1) / kBX, (my + kBY - 1) / kBY, nb); }
+
+}  // namespace
+
+// Launches K<T, true> or K<T, false> by the stencil's corners.
+#define FD_LAUNCH(K, st, grid, block, ...)                                    \
+  do {                                                                        \
+    if (nine(st)) launch_dep(K<T, true>, grid, block, 0, s, __VA_ARGS__);       \
+    else launch_dep(K<T, false>, grid, block, 0, s, __VA_ARGS__);               \
+  } while (0)
+
+template <typename T>
+void fd_apply(int mx, int my, const Stencil9<double>& st, const T* u, T* y, cudaStream_t s, int nb, int64_t ld) {
+  const Stencil9<T> a = scaled<T>(st, 1.0);
+  FD_LAUNCH(k_fd_apply, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, u, y, ld);
+}
+
+template <typename T>
+void fd_first(int mx, int my, const Stencil9<double>& st, const T* b, T* x, T* r, T* d, double c0, double c1, double c2,
+              double w0, double w1, bool last, cudaStream_t s, int nb, int64_t ld) {
+  const double S = 1.0 / st.c[4];
+  const Stencil9<T> a = scaled<T>(st, -c0 * S);
+  FD_LAUNCH(k_fd_first, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, b, x, r, d, (T)(c0 * S), (T)c1, (T)(c2 * S),
+            (T)w0, (T)w1, last ? 1 : 0, ld);
+}
+
+template <typename T>
+void fd_step(int mx, int my, const Stencil9<double>& st, const T* d, T* dn, const T* rin, T* r, T* x, double c1,
+             double c2, int xmode, double w0, double w1, bool last, cudaStream_t s, int nb, int64_t ld) {
+  const Stencil9<T> a = scaled<T>(st, -1.0);
+  FD_LAUNCH(k_fd_step, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, d, dn, rin, r, x, (T)c1,
+            (T)(c2 / st.c[4]), xmode, (T)w0, (T)w1, last ? 1 : 0, ld);
+}
+
+template <typename T>
+void fd_resid(int mx, int my, const Stencil9<double>& st, const T* b, const T* x, T* r, T* d, double c0, cudaStream_t s,
+              int nb, int64_t ld) {
+  const Stencil9<T> a = scaled<T>(st, -1.0);
+  FD_LAUNCH(k_fd_resid, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, b, x, r, d, (T)(c0 / st.c[4]), ld);
+}
+
+template <typename T>
+void fd_resid_restrict(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* b, const T* x, T* rc,
+                       cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
+  const Stencil9<T> a = scaled<T>(st, -1.0);
+  const dim3 grid((mcx + kTX - 1) / kTX, (mcy + kTY - 1) / kTY, nb);
+  FD_LAUNCH(k_fd_resid_restrict, a, grid, dim3(kTX * kTY), mx, my, mcx, mcy, a, b, x, rc, ldf, ldc);
+}
+
+template <typename T>
+void fd_restrict(int mfx, int mfy, int mcx, int mcy, int c, const T* rf, T* rc, cudaStream_t s, int nb,
+                 int64_t ldf, int64_t ldc) {
+  const dim3 bs(16, 16), gs((mcx + 15) / 16, (mcy + 15) / 16, nb);
+  if (c == 2) launch_dep(k_fd_restrict<T, 2>, gs, bs, 0, s, mfx, mfy, mcx, mcy, c, rf, rc, ldf, ldc);
+  else launch_dep(k_fd_restrict<T, 0>, gs, bs, 0, s, mfx, mfy, mcx, mcy, c, rf, rc, ldf, ldc);
+}
+
+template <typename T>
+void fd_prolong(int mfx, int mfy, int mcx, int mcy, int c, const T* zc, T* zf, int accumulate,
+                cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
+  const dim3 bs(32, 8), gs((mfx + 31) / 32, (mfy + 7) / 8, nb);
+  if (c == 2) launch_dep(k_fd_prolong<T, 2>, gs, bs, 0, s, mfx, mfy, mcx, mcy, c, zc, zf, accumulate, ldf, ldc);
+  else launch_dep(k_fd_prolong<T, 0>, gs, bs, 0, s, mfx, mfy, mcx, mcy, c, zc, zf, accumulate, ldf, ldc);
+}
+
+void dense_matvec(int n, const double* M, const double* x, double* y, cudaStream_t s, int nb, int64_t ld) {
+  // rows of a few right-hand sides per block: enough blocks to fill the GPU for small n
+  const unsigned by = (unsigned)(nb < 16 ? nb : 16);
+  launch_dep(k_dense_matvec, dim3((n + kDenseWarps - 1) / kDenseWarps, by), dim3(32 * kDenseWarps), 0, s, n, M, x, y,
+             nb, ld);
+}
+
+#define FD_INST(T)                                                                                               \
+  template void fd_apply<T>(int, int, const Stencil9<double>&, const T*, T*, cudaStream_t, int, int64_t);        \
+  template void fd_first<T>(int, int, const Stencil9<double>&, const T*, T*, T*, T*, double, double, double,     \
+                            double, double, bool, cudaStream_t, int, int64_t);                                   \
+  template void fd_step<T>(int, int, const Stencil9<double>&, const T*, T*, const T*, T*, T*, double, double,    \
+                           int, double, double, bool, cudaStream_t, int, int64_t);                               \
+  template void fd_resid<T>(int, int, const Stencil9<double>&, const T*, const T*, T*, T*, double, cudaStream_t, \
+                            int, int64_t);                                                                       \
+  template void fd_resid_restrict<T>(int, int, int, int, const Stencil9<double>&, const T*, const T*, T*,        \
+                                     cudaStream_t, int, int64_t, int64_t);                                       \
+  template void fd_restrict<T>(int, int, int, int, int, const T*, T*, cudaStream_t, int, int64_t, int64_t);      \
+  template void fd_prolong<T>(int, int, int, int, int, const T*, T*, int, cudaStream_t, int, int64_t, int64_t);
+
+FD_INST(float)
+FD_INST(double)
+
+}  // namespace chebmg

@@ -3,8 +3,7 @@
 // SEM operator (Sec. 1, Eq. 1.3): per element w_m = sum_n G_mn (Dhat_n u),
 // y_e = sum_m Dhat_m^T w_m, then direct-stiffness summation into the global
 // vector by atomics, skipping Dirichlet nodes.  p-multigrid transfers
-// (Sec. 4.1) apply J x J x J per element.  FD (Sec. 3): a constant 3x3
-// stencil per level (five-point on the finest, Galerkin nine-point below).
+// (Sec. 4.1) apply J x J x J per element.  (FD kernels: fd.cu.)
 // Chebyshev recurrences: Algorithms 1 and 2 split into an operator pass and
 // an elementwise pass (the elementwise kernels are in chebyshev.cu).
 #include <cuda_runtime.h>
@@ -405,128 +404,6 @@ void sem_prolong(int Qf, int Qc, int64_t E, const uint32_t* gidf, const uint32_t
                  const T* zc, T* zf, int accumulate, cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
   launch_dep(k_sem_prolong<T>, dim3((unsigned)E, nb), dim3(kTransferThreads), transfer_smem<T>(Qf, Qc), s, Qf, Qc,
              gidf, gidc, J, zc, zf, accumulate, ldf, ldc);
-}
-
-// ===========================================================================
-// FD kernels
-// ===========================================================================
-template <typename T>
-__global__ void k_fd_apply(int mx, int my, Stencil9<T> st, const T* __restrict__ u, T* __restrict__ y,
-                           int64_t ld) {
-  pdl_wait();
-  u += (int64_t)blockIdx.z * ld;   // right-hand side of a batch
-  y += (int64_t)blockIdx.z * ld;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= mx || j >= my) return;
-  T acc = 0;
-#pragma unroll
-  for (int a = -1; a <= 1; ++a) {
-    const int jj = j + a;
-    if (jj < 0 || jj >= my) continue;
-#pragma unroll
-    for (int b = -1; b <= 1; ++b) {
-      const int ii = i + b;
-      if (ii < 0 || ii >= mx) continue;
-      acc += st.c[(a + 1) * 3 + (b + 1)] * u[(size_t)jj * mx + ii];
-    }
-  }
-  y[(size_t)j * mx + i] = acc;
-}
-
-template <typename T>
-void fd_apply(int mx, int my, const Stencil9<T>& st, const T* u, T* y, cudaStream_t s, int nb, int64_t ld) {
-  dim3 bs(32, 8);
-  dim3 gs((mx + 31) / 32, (my + 7) / 8, nb);
-  launch_dep(k_fd_apply<T>, gs, bs, 0, s, mx, my, st, u, y, ld);
-}
-
-// rc(I,J) = sum_{|a|,|b| < c} w_a w_b rf(c(I+1)-1+b, c(J+1)-1+a), w_d = (c - |d|)/c
-template <typename T>
-__global__ void k_fd_restrict(int mfx, int mfy, int mcx, int mcy, int c, const T* __restrict__ rf,
-                              T* __restrict__ rc, int64_t ldf, int64_t ldc) {
-  pdl_wait();
-  rf += (int64_t)blockIdx.z * ldf;
-  rc += (int64_t)blockIdx.z * ldc;
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const int Jc = blockIdx.y * blockDim.y + threadIdx.y;
-  if (I >= mcx || Jc >= mcy) return;
-  const int fi = c * (I + 1) - 1, fj = c * (Jc + 1) - 1;
-  const T inv_c = T(1) / T(c);
-  T acc = 0;
-  for (int a = -(c - 1); a <= c - 1; ++a) {
-    const int jj = fj + a;
-    if (jj < 0 || jj >= mfy) continue;
-    const T wa = T(c - (a < 0 ? -a : a)) * inv_c;
-    T row = 0;
-    for (int b = -(c - 1); b <= c - 1; ++b) {
-      const int ii = fi + b;
-      if (ii < 0 || ii >= mfx) continue;
-      row += T(c - (b < 0 ? -b : b)) * inv_c * rf[(size_t)jj * mfx + ii];
-    }
-    acc += wa * row;
-  }
-  rc[(size_t)Jc * mcx + I] = acc;
-}
-
-template <typename T>
-__global__ void k_fd_prolong(int mfx, int mfy, int mcx, int mcy, int c, const T* __restrict__ zc,
-                             T* __restrict__ zf, int accumulate, int64_t ldf, int64_t ldc) {
-  pdl_wait();
-  zf += (int64_t)blockIdx.z * ldf;
-  zc += (int64_t)blockIdx.z * ldc;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= mfx || j >= mfy) return;
-  const T inv_c = T(1) / T(c);
-  const int I0 = (i + 1) / c - 1, J0 = (j + 1) / c - 1;
-  const int di = i - (c * (I0 + 1) - 1), dj = j - (c * (J0 + 1) - 1);
-  T wi[2] = {T(c - di) * inv_c, T(di) * inv_c};
-  T wj[2] = {T(c - dj) * inv_c, T(dj) * inv_c};
-  T acc = 0;
-  for (int a = 0; a < 2; ++a) {
-    const int Jc = J0 + a;
-    if (Jc < 0 || Jc >= mcy || wj[a] == T(0)) continue;
-    for (int b = 0; b < 2; ++b) {
-      const int I = I0 + b;
-      if (I < 0 || I >= mcx || wi[b] == T(0)) continue;
-      acc += wj[a] * wi[b] * zc[(size_t)Jc * mcx + I];
-    }
-  }
-  T* dst = &zf[(size_t)j * mfx + i];
-  *dst = accumulate ? *dst + acc : acc;
-}
-
-template <typename T>
-void fd_restrict(int mfx, int mfy, int mcx, int mcy, int c, const T* rf, T* rc, cudaStream_t s, int nb,
-                 int64_t ldf, int64_t ldc) {
-  dim3 bs(16, 16);
-  dim3 gs((mcx + 15) / 16, (mcy + 15) / 16, nb);
-  launch_dep(k_fd_restrict<T>, gs, bs, 0, s, mfx, mfy, mcx, mcy, c, rf, rc, ldf, ldc);
-}
-
-template <typename T>
-void fd_prolong(int mfx, int mfy, int mcx, int mcy, int c, const T* zc, T* zf, int accumulate,
-                cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
-  dim3 bs(32, 8);
-  dim3 gs((mfx + 31) / 32, (mfy + 7) / 8, nb);
-  launch_dep(k_fd_prolong<T>, gs, bs, 0, s, mfx, mfy, mcx, mcy, c, zc, zf, accumulate, ldf, ldc);
-}
-
-__global__ void k_dense_matvec(int n, const double* __restrict__ M, const double* __restrict__ x,
-                               double* __restrict__ y, int64_t ld) {
-  pdl_wait();
-  x += (int64_t)blockIdx.y * ld;
-  y += (int64_t)blockIdx.y * ld;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double acc = 0.0;
-  for (int j = 0; j < n; ++j) acc += M[(size_t)i * n + j] * x[j];
-  y[i] = acc;
-}
-
-void dense_matvec(int n, const double* M, const double* x, double* y, cudaStream_t s, int nb, int64_t ld) {
-  launch_dep(k_dense_matvec, dim3((n + 127) / 128, nb), dim3(128), 0, s, n, M, x, y, ld);
 }
 
 // p[0 .. bytes) = 0, 16-byte stores over the aligned body: the zeroing of a work vector as a
@@ -1388,11 +1265,7 @@ void scale(int64_t n, double a, const double* x, double* y, cudaStream_t s) {
   template void sem_restrict<T>(int, int, int64_t, const uint32_t*, const uint32_t*, const T*, const T*,  \
                                 T*, cudaStream_t, int, int64_t, int64_t);                              \
   template void sem_prolong<T>(int, int, int64_t, const uint32_t*, const uint32_t*, const T*, const T*,   \
-                               T*, int, cudaStream_t, int, int64_t, int64_t);                          \
-  template void fd_apply<T>(int, int, const Stencil9<T>&, const T*, T*, cudaStream_t, int, int64_t);    \
-  template void fd_restrict<T>(int, int, int, int, int, const T*, T*, cudaStream_t, int, int64_t, int64_t); \
-  template void fd_prolong<T>(int, int, int, int, int, const T*, T*, int, cudaStream_t, int, int64_t,     \
-                              int64_t);
+                               T*, int, cudaStream_t, int, int64_t, int64_t);
 
 CHEBMG_INST(float)
 CHEBMG_INST(double)
