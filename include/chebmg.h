@@ -150,8 +150,8 @@ int chebmg_coarse_info(const chebmg_ctx* ctx, int* degree, double* lmax);
 /* Kernels of the SEM coarse CG (same method, same status words):
  *   CHEBMG_COARSE_GRID    one persistent cooperative launch over up to one block per SM;
  *                         products exchange rows through global memory as 64-bit words that
- *                         carry the value and its exchange tag together (no separate flag),
- *                         grid-wide reductions on an arrival counter (any coarse mesh);
+ *                         carry the value and its exchange tag together (no separate flag); any
+ *                         coarse mesh, on box lattices with the vector staged in shared memory;
  *   CHEBMG_COARSE_CLUSTER one thread-block cluster (up to 16 CTAs): box lattices at N = 1 with
  *                         the FP32 preconditioner; the operator's FP32 copy and the exchanged
  *                         vectors in shared memory, halos through distributed shared memory,
@@ -159,7 +159,7 @@ int chebmg_coarse_info(const chebmg_ctx* ctx, int* degree, double* lmax);
  *   CHEBMG_COARSE_HOST    host-driven loop of kernels (cooperative launch unavailable). */
 enum { CHEBMG_COARSE_HOST = 0, CHEBMG_COARSE_GRID = 1, CHEBMG_COARSE_CLUSTER = 2 };
 /* Kernel chosen at setup (timed together with the degree), its thread blocks and the rows
- * each block owns (grid: a power of two times 256; cluster: planes x lattice plane). */
+ * each block owns (grid: a power of two; cluster: planes x lattice plane). */
 int chebmg_coarse_shape(const chebmg_ctx* ctx, int* kernel, int* blocks, int* rows_per_block);
 /* Overrides the coarse kernel (GRID or CLUSTER); EINVAL where it does not apply. */
 int chebmg_set_coarse_kernel(chebmg_ctx* ctx, int kernel);

@@ -144,6 +144,8 @@ struct chebmg_ctx {
   float* coarse_invDf = nullptr;
   bool coarse_pf32 = false;     // coarse CG preconditioner in FP32
   int coarse_rows_per_block = 0;
+  int coarse_lat = 0;           // rows per block of the lattice form of the grid-wide kernel; 0: not used
+  unsigned long long* cred = nullptr;   // its tagged partial sums, two parities
   // the outer Krylov product of the finest level: 0 FP64, 1 FP64-class arithmetic on FP32 pairs
   int outer_op = 0;
   void* G_x2 = nullptr;         // level-0 geometric factors as FP32 pairs
@@ -568,12 +570,25 @@ void prolong_to(chebmg_ctx* c, int j, const T* zc, T* zf, int accumulate) {
   check_launch();
 }
 
+// Partial sums of the lattice coarse kernel: as many blocks as there can be SMs, and a phantom one.
+constexpr int kCoarseRedBlocks = 1024;
+size_t coarse_red_bytes() { return sizeof(unsigned long long) * 2 * kCoarseRedWords * (kCoarseRedBlocks + 1); }
+
 // Shape of the persistent coarse kernel: at least rpt_min rows per thread.
 void set_coarse_shape(chebmg_ctx* c, int rpt_min) {
   int grid = 0, rb = 0;
   coarse_pcg_shape(c->L.back().n, rpt_min, &grid, &rb);
   c->coarse_grid = grid;
   c->coarse_rows_per_block = rb;
+}
+
+// Block sizes the lattice form can run with here, smallest first.
+std::vector<int> coarse_lat_blocks(const chebmg_ctx* c) {
+  std::vector<int> v;
+  if (c->lat_val && c->cred)
+    for (int b : {64, 128, 256, 512, 1024})
+      if (coarse_lat_fits(c->L.back().n, c->cc_nx, b)) v.push_back(b);
+  return v;
 }
 
 CoarseCG coarse_args(chebmg_ctx* c, const double* b, double* x) {
@@ -606,6 +621,8 @@ CoarseCG coarse_args(chebmg_ctx* c, const double* b, double* x) {
     a.lat_nx = c->cc_nx;
     a.lat_nxy = c->cc_nx * c->cc_ny;
   }
+  a.lat_block = c->lat_val ? c->coarse_lat : 0;
+  a.red = c->cred;
   a.exf[0] = c->cexf[0];
   a.exf[1] = c->cexf[1];
   a.exd[0] = c->cexd[0];
@@ -619,6 +636,7 @@ CoarseCG coarse_args(chebmg_ctx* c, const double* b, double* x) {
       CK(cudaMemsetAsync(c->cexf[q], 0, sizeof(unsigned long long) * a.n, c->s));
       CK(cudaMemsetAsync(c->cexd[q], 0, sizeof(unsigned long long) * 2 * a.n, c->s));
     }
+    if (c->cred) CK(cudaMemsetAsync(c->cred, 0, coarse_red_bytes(), c->s));
     c->coarse_gen = 0;
   }
   a.gen0 = (unsigned)c->coarse_gen;
@@ -959,6 +977,10 @@ void common_alloc(chebmg_ctx* c) {
     c->cctl = c->dstat + 4;   // zeroed above
     c->hcctl = c->hdstat + 4;
     c->cpart = dalloc<double>(c, 6 * std::max(1, grid));   // two generations of 3 partials per block
+    if (c->lat_val) {
+      c->cred = reinterpret_cast<unsigned long long*>(dalloc<unsigned char>(c, (int64_t)coarse_red_bytes()));
+      CK(cudaMemsetAsync(c->cred, 0, coarse_red_bytes(), c->s));
+    }
     for (int q = 0; q < 2; ++q) {   // tag 0 (zeroed words) is never used
       c->cexf[q] = dalloc<unsigned long long>(c, nc);
       c->cexd[q] = dalloc<unsigned long long>(c, 2 * nc);
@@ -1074,43 +1096,61 @@ void autotune_coarse_degree(chebmg_ctx* c) {
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   float best = 1e30f;
-  int best_m = 1, best_rpt = 1, last_rb = -1, best_kernel = 0;
-  const bool try_cluster = c->cc_ok && c->coarse_pf32;
-  for (int rpt = 1; rpt <= 2 * kCoarseMaxRowsPerThread; rpt *= 2) {
-    const bool cluster = rpt > kCoarseMaxRowsPerThread;   // last round: the cluster kernel
-    if (cluster && !try_cluster) break;
-    c->coarse_kernel = cluster ? 1 : 0;
-    if (!cluster) {
-      set_coarse_shape(c, rpt);
-      if (c->coarse_grid <= 0 || c->coarse_rows_per_block == last_rb) continue;
-      last_rb = c->coarse_rows_per_block;
+  int best_m = 1, best_rpt = 1, best_lat = 0, best_kernel = 0;
+  // one shape (or kernel) with every degree
+  auto try_degrees = [&](int rpt) {
+    for (int m : {1, 2, 4, 8, 12, 16, 24, 32}) {
+      c->coarse_degree = m;
+      float t_min = 1e30f;
+      bool ok = true;
+      for (int rep = 0; rep < 2 && ok; ++rep) {
+        CK(cudaEventRecord(e0, c->s));
+        if (coarse_solve64(c, b, x) != CHEBMG_OK) ok = false;
+        CK(cudaEventRecord(e1, c->s));
+        CK(cudaEventSynchronize(e1));
+        read_scal(c);
+        if (c->hcctl[2] != CS_OK) ok = false;
+        float ms = 0.f;
+        CK(cudaEventElapsedTime(&ms, e0, e1));
+        t_min = std::min(t_min, ms);
+      }
+      if (ok && t_min < best) {
+        best = t_min;
+        best_m = m;
+        best_rpt = rpt;
+        best_lat = c->coarse_lat;
+        best_kernel = c->coarse_kernel;
+      }
     }
-  for (int m : {1, 2, 4, 8, 12, 16, 24, 32}) {
-    c->coarse_degree = m;
-    float t_min = 1e30f;
-    bool ok = true;
-    for (int rep = 0; rep < 2 && ok; ++rep) {
-      CK(cudaEventRecord(e0, c->s));
-      if (coarse_solve64(c, b, x) != CHEBMG_OK) ok = false;
-      CK(cudaEventRecord(e1, c->s));
-      CK(cudaEventSynchronize(e1));
-      read_scal(c);
-      if (c->hcctl[2] != CS_OK) ok = false;
-      float ms = 0.f;
-      CK(cudaEventElapsedTime(&ms, e0, e1));
-      t_min = std::min(t_min, ms);
-    }
-    if (ok && t_min < best) {
-      best = t_min;
-      best_m = m;
-      best_rpt = rpt;
-      best_kernel = c->coarse_kernel;
-    }
+  };
+  // grid-wide: the lattice form where it runs (it beat the general one at every size measured), else
+  // the general one at several rows per thread
+  c->coarse_kernel = 0;
+  const std::vector<int> lat = coarse_lat_blocks(c);
+  for (int blk : lat) {
+    c->coarse_lat = blk;
+    try_degrees(1);
   }
+  int last_rb = -1;
+  for (int rpt = 1; lat.empty() && rpt <= kCoarseMaxRowsPerThread; rpt *= 2) {
+    c->coarse_lat = 0;
+    set_coarse_shape(c, rpt);
+    if (c->coarse_grid <= 0 || c->coarse_rows_per_block == last_rb) continue;
+    last_rb = c->coarse_rows_per_block;
+    try_degrees(rpt);
   }
+  const int grid_lat = best_lat, grid_rpt = best_rpt;
+  if (c->cc_ok && c->coarse_pf32) {
+    c->coarse_kernel = 1;
+    try_degrees(best_rpt);
+  }
+  // the grid-wide shape stays the best grid-wide one (the kernel can be selected by hand)
+  best_lat = grid_lat;
+  best_rpt = grid_rpt;
+  c->coarse_lat = best_lat;
   c->coarse_degree = best_m;
   c->coarse_kernel = best_kernel;
-  set_coarse_shape(c, best_kernel == 1 ? 1 : best_rpt);
+  set_coarse_shape(c, best_rpt);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   CK(cudaMemsetAsync(c->cctl + 4, 0, sizeof(unsigned), c->s));
@@ -2515,8 +2555,9 @@ int chebmg_coarse_shape(const chebmg_ctx* c, int* kernel, int* blocks, int* rows
   const bool cluster = sem && c->coarse_kernel == 1 && c->cc_ok && c->coarse_pf32;
   const bool grid = sem && !cluster && c->coop_ok;
   *kernel = cluster ? CHEBMG_COARSE_CLUSTER : grid ? CHEBMG_COARSE_GRID : CHEBMG_COARSE_HOST;
-  *blocks = cluster ? c->cc_ctas : grid ? c->coarse_grid : 0;
-  *rows_per_block = cluster ? c->cc_rmax : grid ? c->coarse_rows_per_block : 0;
+  const int lat = c->coarse_lat;
+  *blocks = cluster ? c->cc_ctas : !grid ? 0 : lat ? (int)((c->L.back().n + lat - 1) / lat) : c->coarse_grid;
+  *rows_per_block = cluster ? c->cc_rmax : !grid ? 0 : lat ? lat : c->coarse_rows_per_block;
   return CHEBMG_OK;
 }
 

@@ -393,6 +393,10 @@ struct CoarseCG {
   unsigned long long* exf[2];   // [n] FP32 values
   unsigned long long* exd[2];   // [2 n] FP64 values
   unsigned gen0;
+  // coarse_lat.cu (lat_block > 0): rows, and threads, per block; the blocks' partial sums as tagged
+  // words, 6 per block and reduction parity (one block more than can run: the self-test's phantom).
+  int lat_block;
+  unsigned long long* red;
 };
 // Step coefficients of the coarse CG's polynomial preconditioner (Algorithm 2, beta = 1):
 // step i (1 <= i < degree) updates d = c1[i] d + c2[i] S r.  The coarse kernels fill this table
@@ -473,6 +477,13 @@ bool coarse_pcg_launch(const CoarseCG& a, int grid, cudaStream_t s, cudaError_t*
 // Grid size (blocks) and rows per block for a coarse problem of n rows, at least rpt_min rows
 // per thread (a power of two up to kCoarseMaxRowsPerThread); grid 0 = not possible.
 void coarse_pcg_shape(int64_t n, int rpt_min, int* grid, int* rows_per_block);
+
+// The same CG on a box lattice with the exchanged vector staged in shared memory (coarse_lat.cu):
+// one row per thread, lat_block rows per block.  coarse_lat_fits: whether that block size can run
+// (64 .. 1024 threads, one block per SM, shared memory, loads per thread).
+constexpr int kCoarseRedWords = 6;
+bool coarse_lat_fits(int64_t n, int nx, int lat_block);
+bool coarse_lat_launch(const CoarseCG& a, cudaStream_t s, cudaError_t* err);
 
 // ---- coarse CG on one thread-block cluster (coarse_cluster.cu; box lattice at N = 1) ----
 // Forward half of the 27-point lattice stencil, slot k -> offset (dx, dy, dz): slot 0 the

@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "coarse_util.cuh"
 #include "common.cuh"
 
 namespace chebmg {
@@ -738,13 +739,6 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
 __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-constexpr uint64_t kWaitNs = 1000000000ull;   // every wait gives up after about a second
-
 // Spins until *p >= target (acquire); false after kWaitNs, with the timeout recorded.
 __device__ __forceinline__ bool wait_at_least(const unsigned* p, unsigned target, unsigned* ctl) {
   if (ld_acquire(p) >= target) return true;
@@ -794,22 +788,6 @@ __device__ __forceinline__ bool allreduce3(unsigned* ctl, unsigned& gen, unsigne
   c = C;
   return ok;
 }
-// ---- tagged-word exchange ----
-__device__ __forceinline__ void st_tagged(unsigned long long* p, unsigned long long w) {
-  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
-__device__ __forceinline__ void st_tagged2(unsigned long long* p, unsigned long long w0, unsigned long long w1) {
-  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(w0), "l"(w1) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_tagged(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-  return w;
-}
-__device__ __forceinline__ void ld_tagged2(const unsigned long long* p, unsigned long long& w0,
-                                           unsigned long long& w1) {
-  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");
-}
 // Column index load that the compiler may not merge with an earlier one (keeps the reload
 // loop from holding all column indices in registers).
 __device__ __forceinline__ int ld_col(const int* p) {
@@ -817,52 +795,6 @@ __device__ __forceinline__ int ld_col(const int* p) {
   asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
-
-// One exchanged value: FP32 in one tagged word, FP64 as two (high and low halves, loaded
-// and stored together; each half carries the tag, so a torn pair is never accepted).
-template <typename V>
-struct Tagged;
-template <>
-struct Tagged<float> {
-  struct W {
-    unsigned long long w;
-  };
-  static __device__ __forceinline__ unsigned long long* buf(const CoarseCG& a, unsigned gx) {
-    return a.exf[gx & 1u];
-  }
-  static __device__ __forceinline__ void store(unsigned long long* b, int64_t g, unsigned tag, float v) {
-    st_tagged(b + g, ((unsigned long long)tag << 32) | __float_as_uint(v));
-  }
-  static __device__ __forceinline__ W load(const unsigned long long* b, int64_t g) { return {ld_tagged(b + g)}; }
-  static __device__ __forceinline__ bool ready(const W& w, unsigned tag) { return (unsigned)(w.w >> 32) == tag; }
-  static __device__ __forceinline__ float value(const W& w) { return __uint_as_float((unsigned)w.w); }
-  static __device__ __forceinline__ float coef(const CoarseCG& a, int64_t i) { return __ldg(&a.valf[i]); }
-};
-template <>
-struct Tagged<double> {
-  struct W {
-    unsigned long long hi, lo;
-  };
-  static __device__ __forceinline__ unsigned long long* buf(const CoarseCG& a, unsigned gx) {
-    return a.exd[gx & 1u];
-  }
-  static __device__ __forceinline__ void store(unsigned long long* b, int64_t g, unsigned tag, double v) {
-    const unsigned long long t = (unsigned long long)tag << 32;
-    st_tagged2(b + 2 * g, t | (unsigned)__double2hiint(v), t | (unsigned)__double2loint(v));
-  }
-  static __device__ __forceinline__ W load(const unsigned long long* b, int64_t g) {
-    W w;
-    ld_tagged2(b + 2 * g, w.hi, w.lo);
-    return w;
-  }
-  static __device__ __forceinline__ bool ready(const W& w, unsigned tag) {
-    return (unsigned)(w.hi >> 32) == tag && (unsigned)(w.lo >> 32) == tag;
-  }
-  static __device__ __forceinline__ double value(const W& w) {
-    return __hiloint2double((int)(unsigned)w.hi, (int)(unsigned)w.lo);
-  }
-  static __device__ __forceinline__ double coef(const CoarseCG& a, int64_t i) { return __ldg(&a.val[i]); }
-};
 
 // Publishes this block's rows under exchange gx.  No barrier first: every product ends with
 // a block barrier, so this block has finished reading the buffer it overwrites (two exchanges
@@ -1185,6 +1117,7 @@ void coarse_pcg_shape(int64_t n, int rpt_min, int* grid, int* rows_per_block) {
 }
 
 bool coarse_pcg_launch(const CoarseCG& a, int grid, cudaStream_t s, cudaError_t* err) {
+  if (a.lat_block > 0) return coarse_lat_launch(a, s, err);
   CoarseCG arg = a;
   void* params[] = {&arg};
   const int rpt = a.rows_per_block / kCoarseThreads;
