@@ -64,6 +64,7 @@ k_adj_delta(int64_t n, int64_t ld, double beta, double c1, const double* __restr
 // out = a x + b y  (out may alias x or y)
 __global__ void __launch_bounds__(kThreads)
 k_lincomb(int64_t n, int64_t ld, double a, const double* x, double b, const double* y, double* out) {
+  pdl_wait();
   const int64_t o = (int64_t)blockIdx.y * ld;
   ROWS_LOOP(n) out[o + g] = a * x[o + g] + (y ? b * y[o + g] : 0.0);
 }
@@ -155,8 +156,7 @@ void adj_delta(int64_t n, int64_t ld, int nb, double beta, double c1, const doub
 
 void lincomb(int64_t n, int64_t ld, int nb, double a, const double* x, double b, const double* y, double* out,
              cudaStream_t s) {
-  k_lincomb<<<dim3(blocks_for(n), nb), kThreads, 0, s>>>(n, ld, a, x, b, y, out);
-  g_launches.fetch_add(1, std::memory_order_relaxed);
+  launch_dep(k_lincomb, dim3(blocks_for(n), nb), dim3(kThreads), 0, s, n, ld, a, x, b, y, out);
 }
 
 void scale_rows(int64_t n, int64_t ld, int nb, const double* coef, const double* x, double* out, cudaStream_t s) {

@@ -194,6 +194,7 @@ struct chebmg_ctx {
     std::vector<double*> Et;                // e_0 .. e_steps
     double *W = nullptr, *Z = nullptr, *EB = nullptr, *ZB = nullptr, *WB = nullptr;
     double *part = nullptr, *acc = nullptr, *rows = nullptr, *coef = nullptr;
+    double* fdpart = nullptr;               // FD: partial sums of one smoother call's dots
   } gw;
   // ---- GMRES workspace ----
   struct GmresWork {
@@ -1767,6 +1768,7 @@ void grad_alloc(chebmg_ctx* c, int nb, int kmax, int steps) {
   for (double** p : {&g.W, &g.Z, &g.EB, &g.ZB, &g.WB}) take(*p, v0);
   take(g.part, adj_dot_scratch(c->L[0].n, nb));
   take(g.acc, kmax + nl);
+  if (c->type == TYPE_FD) take(g.fdpart, fd_adj_partials(c->L[0].mx, c->L[0].my, nb, kmax));
   take(g.rows, 2 * (int64_t)nb);
   take(g.coef, nb);
   g.nb = nb;
@@ -1794,11 +1796,78 @@ int vcycle_store(chebmg_ctx* c, int j, const double* b, double* x) {
   if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
   prolong_to<double>(c, j, vec<double>(C, VX), x, 1);
   if (c->post > 0) {
-    CK(cudaMemcpyAsync(c->gw.lv[j][GW_XM], x, sizeof(double) * span(c, L), cudaMemcpyDeviceToDevice, c->s));
+    cast<double, double>(L.n, x, c->gw.lv[j][GW_XM], c->s, c->nb, ldv(c, L), ldv(c, L));
     smooth<double>(c, j, b, x, c->post, false);
   }
   check_launch();
   return rc;
+}
+
+// smooth_adj on an FD level: the forward recomputation writes each d_i and r_i where the backward
+// steps read them (S is one number there, so S r_i is not stored), a kernel per step either way.
+// set_bbar: bbar is overwritten.
+void smooth_adj_fd(chebmg_ctx* c, int j, const double* b, const double* x0, int order, const double* xbar,
+                   double* bbar, bool set_bbar, double* x0bar) {
+  auto& g = c->gw;
+  Level& L = c->L[j];
+  const int nb = c->nb;
+  const int64_t ld = ldv(c, L);
+  const double S = 1.0 / L.st[4], lam = L.lmax * c->lscale;
+  const std::vector<double>& beta = c->beta_ovr;
+  const Stencil9<double> st = stencil(L);
+  const Recurrence q = recurrence(c, L, order);
+  // from a zero guess r_0 = b and d_0 = c0 S b, of which only b is needed
+  std::vector<const double*> D(order), R(order);
+  std::vector<double> coef(2 * order, 1.0);
+  for (int i = 0; i < order; ++i) {
+    D[i] = g.D[i];
+    R[i] = g.SR[i];
+  }
+  int i0 = 1;
+  if (x0) {
+    fd_resid<double>(L.mx, L.my, st, b, x0, g.SR[0], g.D[0], q.c0, c->s, nb, ld);
+  } else {
+    D[0] = R[0] = b;
+    coef[0] = q.c0 * S;
+    if (order > 1)
+      fd_first<double>(L.mx, L.my, st, b, nullptr, g.SR[1], g.D[1], q.c0, q.c1[1], q.c2[1], 0.0, 0.0, false, c->s, nb,
+                       ld);
+    i0 = 2;
+  }
+  for (int i = i0; i < order; ++i)
+    fd_step<double>(L.mx, L.my, st, D[i - 1], g.D[i], R[i - 1], g.SR[i], nullptr, q.c1[i], q.c2[i], SX_NONE, 0.0, 0.0,
+                    false, c->s, nb, ld);
+  fd_adj_dots(L.mx, L.my, order, D.data(), xbar, g.fdpart, c->s, nb, ld);
+  double *rho[2] = {g.lv[j][GW_RHO], g.lv[j][GW_YA]}, *del[2] = {g.lv[j][GW_DEL], g.lv[j][GW_XS]};
+  for (int i = order - 1; i >= 0; --i) {
+    const int n = order - 1 - i, in = n & 1, out = in ^ 1;
+    FdAdjStep a{};
+    if (n > 0) {
+      a.rho = rho[in];
+      a.del = del[in];
+    }
+    a.xbar = xbar;
+    a.r = R[i];
+    // d rho / d delta is c2_i / lambda (c0 for i = 0); its derivative in lambda is minus itself / lambda
+    a.k = i > 0 ? q.c2[i] : q.c0;
+    coef[order + i] = -a.k * S / lam;
+    a.bk = beta[order - 1];
+    a.last = i == 0;
+    if (!a.last) {
+      a.beta = beta[i - 1];
+      a.c1 = q.c1[i];
+    }
+    a.rho_out = rho[out];
+    a.del_out = del[out];
+    a.bbar = bbar;
+    a.set_bbar = set_bbar;
+    a.x0bar = x0 ? x0bar : nullptr;
+    a.part = g.fdpart;
+    a.dot = order + i;
+    fd_adj_step(L.mx, L.my, st, a, c->s, nb, ld);
+  }
+  fd_adj_finish(L.mx, L.my, nb, order, coef.data(), g.fdpart, g.acc, g.kmax + j, c->s);
+  check_launch();
 }
 
 // Adjoint of one Algorithm-2 smoother call on level j (inputs b and x0, x0 = null for a zero
@@ -1873,8 +1942,10 @@ int vcycle_adj(chebmg_ctx* c, int j, const double* b, const double* xbar, double
   const int nb = c->nb;
   const int64_t n = L.n, ld = ldv(c, L), sp = span(c, L);
   double* x0bar = g.lv[j][GW_X0B];
-  zero<double>(c, bbar, sp);
-  if (c->post > 0) smooth_adj(c, j, b, g.lv[j][GW_XM], c->post, xbar, bbar, x0bar);
+  const bool fd = L.type == TYPE_FD;
+  if (!fd) zero<double>(c, bbar, sp);
+  if (c->post > 0 && fd) smooth_adj_fd(c, j, b, g.lv[j][GW_XM], c->post, xbar, bbar, true, x0bar);
+  else if (c->post > 0) smooth_adj(c, j, b, g.lv[j][GW_XM], c->post, xbar, bbar, x0bar);
   else CK(cudaMemcpyAsync(x0bar, xbar, sizeof(double) * sp, cudaMemcpyDeviceToDevice, c->s));
   // x_mid = x_pre + P x_c
   restrict_to<double>(c, j, x0bar, g.lv[j + 1][GW_XB]);
@@ -1883,6 +1954,12 @@ int vcycle_adj(chebmg_ctx* c, int j, const double* b, const double* xbar, double
   // r_c = P^T (b - A x_pre)
   double* rb = g.lv[j][GW_RB];
   prolong_to<double>(c, j, g.lv[j + 1][GW_BB], rb, 0);
+  if (fd) {
+    fd_adj_mid(L.mx, L.my, stencil(L), rb, bbar, c->post == 0, x0bar, c->s, nb, ld);
+    if (c->pre > 0) smooth_adj_fd(c, j, b, nullptr, c->pre, x0bar, bbar, false, nullptr);
+    check_launch();
+    return rc;
+  }
   lincomb(n, ld, nb, 1.0, bbar, 1.0, rb, bbar, c->s);
   double* ya = g.lv[j][GW_YA];
   zero<double>(c, ya, sp);
@@ -1917,6 +1994,7 @@ int cycle_error_grad(chebmg_ctx* c, int nrhs, const double* E0, int steps, const
   c->beta_ovr.assign(betas, betas + nbeta);
   c->lscale = scale;
   BatchScope bs(c, nrhs);
+  const PdlScope pdl_(true);   // never captured: the kernels launch as a dependent chain
   Level& L = c->L[0];
   const int64_t n = L.n, ld = ldv(c, L), sp = span(c, L);
   const double* S = static_cast<const double*>(L.invD[CHEBMG_F64]);
@@ -1925,7 +2003,7 @@ int cycle_error_grad(chebmg_ctx* c, int nrhs, const double* E0, int steps, const
   dot_rows(n, ld, nrhs, g.Et[0], g.Et[0], g.part, g.rows, c->s);
   int rc = CHEBMG_OK;
   for (int t = 0; t < steps; ++t) {
-    zero<double>(c, g.W, sp);
+    if (L.type == TYPE_SEM) zero<double>(c, g.W, sp);
     apply_into<double>(c, 0, g.Et[t], g.W);
     rc = vcycle_store(c, 0, g.W, g.Z);
     if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
@@ -1951,14 +2029,14 @@ int cycle_error_grad(chebmg_ctx* c, int nrhs, const double* E0, int steps, const
   CK(cudaMemsetAsync(g.acc, 0, sizeof(double) * (g.kmax + c->L.size()), c->s));
   for (int t = steps - 1; t >= 0; --t) {
     lincomb(n, ld, nrhs, -1.0, g.EB, 0.0, nullptr, g.ZB, c->s);
-    zero<double>(c, g.W, sp);
+    if (L.type == TYPE_SEM) zero<double>(c, g.W, sp);
     apply_into<double>(c, 0, g.Et[t], g.W);
     rc = vcycle_store(c, 0, g.W, g.Z);                  // recomputed forward state of cycle t
     if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
     rc = vcycle_adj(c, 0, g.W, g.ZB, g.WB);
     if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
     double* ya = g.lv[0][GW_YA];
-    zero<double>(c, ya, sp);
+    if (L.type == TYPE_SEM) zero<double>(c, ya, sp);
     apply_into<double>(c, 0, g.WB, ya);
     lincomb(n, ld, nrhs, 1.0, g.EB, 1.0, ya, g.EB, c->s);
   }

@@ -279,6 +279,31 @@ void fd_restrict(int mfx, int mfy, int mcx, int mcy, int c, const T* rf, T* rc, 
 template <typename T>
 void fd_prolong(int mfx, int mfy, int mcx, int mcy, int c, const T* zc, T* zf, int accumulate,
                 cudaStream_t s, int nb = 1, int64_t ldf = 0, int64_t ldc = 0);
+// Adjoint of one FD smoother application (the recurrences at the top of adjoint.cu), a kernel per
+// step.  `part` holds the partial sums of 2 order dots: first <xbar, d_i>, then <delta, r_i>.
+struct FdAdjStep {
+  const double *rho, *del;      // null on the first step: rho = 0, delta = bk xbar
+  const double *xbar, *r;
+  double k;                     // rho' = rho + k S delta
+  double bk, beta, c1;          // delta' = beta xbar + c1 delta - A rho'
+  double *rho_out, *del_out;    // not rho and del themselves
+  bool last;                    // instead: bbar = (set_bbar) or += rho', x0bar = xbar - A rho' unless null
+  double* bbar;
+  bool set_bbar;
+  double* x0bar;
+  double* part;
+  int dot;                      // index of this step's <delta, r>
+};
+int64_t fd_adj_partials(int mx, int my, int nb, int order);
+void fd_adj_step(int mx, int my, const Stencil9<double>& st, const FdAdjStep& a, cudaStream_t s, int nb, int64_t ld);
+void fd_adj_dots(int mx, int my, int nv, const double* const* d, const double* xbar, double* part, cudaStream_t s,
+                 int nb, int64_t ld);
+// acc[i] += coef[i] <xbar, d_i>, acc[lslot] += sum_i coef[order + i] <delta, r_i>  (order <= 64)
+void fd_adj_finish(int mx, int my, int nb, int order, const double* coef, const double* part, double* acc, int lslot,
+                   cudaStream_t s);
+// bbar = (set_bbar) or += rb, x0bar -= A rb
+void fd_adj_mid(int mx, int my, const Stencil9<double>& st, const double* rb, double* bbar, bool set_bbar,
+                double* x0bar, cudaStream_t s, int nb, int64_t ld);
 void dense_matvec(int n, const double* M, const double* x, double* y, cudaStream_t s, int nb = 1, int64_t ld = 0);
 
 // ---- Chebyshev recurrences (Algorithms 1 and 2), elementwise over n ----

@@ -90,7 +90,7 @@ k_fd_apply(int mx, int my, Stencil9<T> st, const T* __restrict__ u, T* __restric
 }
 
 // First step from a zero guess: with d_0 = c0 b (c0 includes S), r = b - A d_0 (st = -c0 A),
-// d = c1 d_0 + c2 r, x = w0 d_0 + w1 d.  last: r and d are not stored.
+// d = c1 d_0 + c2 r, x = w0 d_0 + w1 d (unless x is null).  last: r and d are not stored.
 template <typename T, bool NINE>
 __global__ void __launch_bounds__(kBX * kBY)
 k_fd_first(int mx, int my, Stencil9<T> st, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ r,
@@ -106,7 +106,7 @@ k_fd_first(int mx, int my, Stencil9<T> st, const T* __restrict__ b, T* __restric
   T uc;
   const T rv = ar.add(stencil_sum<T, NINE>(ar, b + o, mx, my, p.i, p.j, c, uc), b0);
   const T d0 = c0 * b0, dn = c1 * d0 + c2 * rv;
-  x[o + p.g] = w0 * d0 + w1 * dn;
+  if (x) x[o + p.g] = w0 * d0 + w1 * dn;
   if (last) return;
   r[o + p.g] = rv;
   d[o + p.g] = dn;
@@ -283,6 +283,156 @@ k_dense_matvec(int n, const double* __restrict__ M, const double* __restrict__ x
   }
 }
 
+// ---- adjoint of a smoother application (recurrences at the top of adjoint.cu) ----
+__device__ __forceinline__ double block_dot(double v) {   // sum over the block, result in thread (0, 0)
+  __shared__ double sh[kBY];
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+  if (threadIdx.x == 0) sh[threadIdx.y] = v;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    v = 0.0;
+#pragma unroll
+    for (int q = 0; q < kBY; ++q) v += sh[q];
+  }
+  return v;
+}
+__device__ __forceinline__ int64_t part_index(int dot) {   // partials of one dot: [right-hand side][block]
+  const int64_t nblk = (int64_t)gridDim.x * gridDim.y;
+  return ((int64_t)dot * gridDim.z + blockIdx.z) * nblk + (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
+}
+
+// One step: rho' = rho + k delta (with FIRST: rho = 0 and delta = bk xbar), the partial <delta, r>, then
+//   a middle step: delta' = beta xbar + c1 delta - A rho';
+//   the last (LAST): bbar = or += rho', and x0bar = xbar - A rho' where x0bar is given.
+// st = -A.  rho' of the tile and its rim is formed in shared memory, so A needs no pass of its own.
+template <bool NINE, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_adj_step(int mx, int my, Stencil9<double> st, const double* __restrict__ rho, const double* __restrict__ del,
+              const double* __restrict__ xbar, const double* __restrict__ r, double k, double bk, double beta,
+              double c1, double* __restrict__ rho_out, double* __restrict__ del_out, double* bbar, int set_bbar,
+              double* __restrict__ x0bar, double* __restrict__ part, int dot, int64_t ld) {
+  __shared__ double s[kBY + 2][kBX + 2];
+  double c[9];
+  const Arith<double> ar;
+  load_stencil<double, NINE>(st, c);
+  k = in_register(k);
+  pdl_wait();
+  const int64_t o = (int64_t)blockIdx.z * ld;
+  const int i0 = blockIdx.x * kBX - 1, j0 = blockIdx.y * kBY - 1;
+  const int tid = threadIdx.y * kBX + threadIdx.x;
+  for (int q = tid; q < (kBX + 2) * (kBY + 2); q += kBX * kBY) {
+    const int sj = q / (kBX + 2), si = q - sj * (kBX + 2), i = i0 + si, j = j0 + sj;
+    double v = 0.0;
+    if (i >= 0 && i < mx && j >= 0 && j < my) {
+      const int64_t g = o + (int64_t)j * mx + i;
+      v = FIRST ? ar.mul(k, bk * xbar[g]) : fma(k, del[g], rho[g]);
+    }
+    s[sj][si] = v;
+  }
+  const Pt p = point(mx, my);
+  double xb = 0.0, dv = 0.0, rv = 0.0;
+  if (p.in) {
+    xb = xbar[o + p.g];
+    dv = FIRST ? bk * xb : del[o + p.g];
+    rv = r[o + p.g];
+  }
+  __syncthreads();
+  if (p.in) {
+    const int si = threadIdx.x + 1, sj = threadIdx.y + 1;
+    double acc = 0.0;
+    if (!LAST || x0bar) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q)
+        if (used<NINE>(q)) acc = fma(c[q], s[sj + q / 3 - 1][si + q % 3 - 1], acc);
+    }
+    const double rn = s[sj][si];
+    if constexpr (LAST) {
+      bbar[o + p.g] = set_bbar ? rn : bbar[o + p.g] + rn;
+      if (x0bar) x0bar[o + p.g] = xb + acc;
+    } else {
+      rho_out[o + p.g] = rn;
+      del_out[o + p.g] = fma(beta, xb, fma(c1, dv, acc));
+    }
+  }
+  const double t = block_dot(dv * rv);
+  if (tid == 0) part[part_index(dot)] = t;
+}
+
+// Partial <xbar, d_i> for up to kAdjDots vectors.
+constexpr int kAdjDots = 8;
+struct AdjVecs {
+  const double* p[kAdjDots];
+};
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_adj_dots(int mx, int my, int nv, AdjVecs d, const double* __restrict__ xbar, double* __restrict__ part, int dot0,
+              int64_t ld) {
+  pdl_wait();
+  const Pt p = point(mx, my);
+  const int64_t o = (int64_t)blockIdx.z * ld + p.g;
+  const double xb = p.in ? xbar[o] : 0.0;
+#pragma unroll
+  for (int v = 0; v < kAdjDots; ++v) {
+    if (v >= nv) break;
+    const double t = block_dot(p.in ? xb * d.p[v][o] : 0.0);
+    if (threadIdx.x == 0 && threadIdx.y == 0) part[part_index(dot0 + v)] = t;
+    __syncthreads();
+  }
+}
+
+// acc[i] += coef[i] * dot i for i < K (block i), acc[lslot] += sum_i coef[K + i] * dot (K + i) (block
+// K); a dot is the sum of its `count` partials, in fixed order.
+constexpr int kAdjMaxOrder = 64;
+struct AdjCoef {
+  double c[2 * kAdjMaxOrder];
+};
+__global__ void __launch_bounds__(256)
+k_fd_adj_finish(int K, int64_t count, const double* __restrict__ part, const __grid_constant__ AdjCoef coef,
+                double* __restrict__ acc, int lslot) {
+  pdl_wait();
+  __shared__ double sh[8];
+  const bool lam = (int)blockIdx.x == K;
+  const int d0 = blockIdx.x, nd = lam ? K : 1;
+  double s = 0.0;
+  for (int d = 0; d < nd; ++d) {
+    double t0 = 0.0, t1 = 0.0;
+    const double* p = part + (int64_t)(d0 + d) * count;
+    int64_t q = threadIdx.x;
+    for (; q + 256 < count; q += 512) {
+      t0 += p[q];
+      t1 += p[q + 256];
+    }
+    if (q < count) t0 += p[q];
+    s += coef.c[d0 + d] * (t0 + t1);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) s += sh[q];
+    acc[lam ? lslot : d0] += s;
+  }
+}
+
+// bbar = or += rb, x0bar -= A rb (st = -A)
+template <bool NINE>
+__global__ void __launch_bounds__(kBX * kBY)
+k_fd_adj_mid(int mx, int my, Stencil9<double> st, const double* __restrict__ rb, double* __restrict__ bbar,
+             int set_bbar, double* __restrict__ x0bar, int64_t ld) {
+  double c[9];
+  const Arith<double> ar;
+  load_stencil<double, NINE>(st, c);
+  pdl_wait();
+  const Pt p = point(mx, my);
+  if (!p.in) return;
+  const int64_t o = (int64_t)blockIdx.z * ld;
+  double uc;
+  const double acc = stencil_sum<double, NINE>(ar, rb + o, mx, my, p.i, p.j, c, uc);
+  x0bar[o + p.g] += acc;
+  bbar[o + p.g] = set_bbar ? uc : bbar[o + p.g] + uc;
+}
+
 template <typename T>
 bool nine(const Stencil9<T>& st) {
   return st.c[0] != T(0) || st.c[2] != T(0) || st.c[6] != T(0) || st.c[8] != T(0);
@@ -363,6 +513,59 @@ void dense_matvec(int n, const double* M, const double* x, double* y, cudaStream
   const unsigned by = (unsigned)(nb < 16 ? nb : 16);
   launch_dep(k_dense_matvec, dim3((n + kDenseWarps - 1) / kDenseWarps, by), dim3(32 * kDenseWarps), 0, s, n, M, x, y,
              nb, ld);
+}
+
+int64_t fd_adj_partials(int mx, int my, int nb, int order) {
+  const dim3 g = grid_of(mx, my, nb);
+  return 2 * (int64_t)order * g.x * g.y * g.z;
+}
+
+void fd_adj_step(int mx, int my, const Stencil9<double>& st, const FdAdjStep& a, cudaStream_t s, int nb, int64_t ld) {
+  const Stencil9<double> m = scaled<double>(st, -1.0);
+  const dim3 grid = grid_of(mx, my, nb), block(kBX, kBY);
+  const double k = a.k / st.c[4];   // S folded in
+  auto go = [&](auto kernel) {
+    launch_dep(kernel, grid, block, 0, s, mx, my, m, a.rho, a.del, a.xbar, a.r, k, a.bk, a.beta, a.c1, a.rho_out,
+               a.del_out, a.bbar, a.set_bbar ? 1 : 0, a.x0bar, a.part, a.dot, ld);
+  };
+  const bool first = a.rho == nullptr;
+  if (nine(m)) {
+    if (first && a.last) go(k_fd_adj_step<true, true, true>);
+    else if (first) go(k_fd_adj_step<true, true, false>);
+    else if (a.last) go(k_fd_adj_step<true, false, true>);
+    else go(k_fd_adj_step<true, false, false>);
+  } else {
+    if (first && a.last) go(k_fd_adj_step<false, true, true>);
+    else if (first) go(k_fd_adj_step<false, true, false>);
+    else if (a.last) go(k_fd_adj_step<false, false, true>);
+    else go(k_fd_adj_step<false, false, false>);
+  }
+}
+
+void fd_adj_dots(int mx, int my, int nv, const double* const* d, const double* xbar, double* part, cudaStream_t s,
+                 int nb, int64_t ld) {
+  for (int v0 = 0; v0 < nv; v0 += kAdjDots) {
+    AdjVecs a{};
+    const int n = nv - v0 < kAdjDots ? nv - v0 : kAdjDots;
+    for (int v = 0; v < n; ++v) a.p[v] = d[v0 + v];
+    launch_dep(k_fd_adj_dots, grid_of(mx, my, nb), dim3(kBX, kBY), 0, s, mx, my, n, a, xbar, part, v0, ld);
+  }
+}
+
+void fd_adj_finish(int mx, int my, int nb, int order, const double* coef, const double* part, double* acc, int lslot,
+                   cudaStream_t s) {
+  AdjCoef c{};
+  for (int q = 0; q < 2 * order; ++q) c.c[q] = coef[q];
+  const dim3 g = grid_of(mx, my, nb);
+  launch_dep(k_fd_adj_finish, dim3(order + 1), dim3(256), 0, s, order, (int64_t)g.x * g.y * g.z, part, c, acc, lslot);
+}
+
+void fd_adj_mid(int mx, int my, const Stencil9<double>& st, const double* rb, double* bbar, bool set_bbar,
+                double* x0bar, cudaStream_t s, int nb, int64_t ld) {
+  const Stencil9<double> m = scaled<double>(st, -1.0);
+  const dim3 grid = grid_of(mx, my, nb), block(kBX, kBY);
+  if (nine(m)) launch_dep(k_fd_adj_mid<true>, grid, block, 0, s, mx, my, m, rb, bbar, set_bbar ? 1 : 0, x0bar, ld);
+  else launch_dep(k_fd_adj_mid<false>, grid, block, 0, s, mx, my, m, rb, bbar, set_bbar ? 1 : 0, x0bar, ld);
 }
 
 #define FD_INST(T)                                                                                               \
