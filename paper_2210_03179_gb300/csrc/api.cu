@@ -2407,10 +2407,18 @@ void upload_sem_levels(chebmg_ctx* c, std::vector<SemHostLevel>& H, bool boxed) 
     L.G[CHEBMG_F64] = upload<double>(c, h.G);
     L.invD[CHEBMG_F64] = upload<double>(c, invd);
     L.D[CHEBMG_F64] = upload<double>(c, h.Dm);
-    if (h.N == 7) CK(sem_ax8_set_D(h.Dm.data()));
+    if (h.N == 7) {
+      CK(sem_ax8_set_D(h.Dm.data()));
+      CK(cudaStreamSynchronize(nullptr));   // the uploads above went through the default stream
+      permute_g8<double>(L.E, static_cast<double*>(L.G[CHEBMG_F64]), c->s);
+    }
     if (sem_axl_supported(h.NQ)) CK(sem_axl_set_D(h.NQ, h.Dm.data()));
     if (smoothed32) {
       L.G[CHEBMG_F32] = upload<float>(c, h.G);
+      if (h.N == 7) {
+        CK(cudaStreamSynchronize(nullptr));
+        permute_g8<float>(L.E, static_cast<float*>(L.G[CHEBMG_F32]), c->s);
+      }
       L.invD[CHEBMG_F32] = upload<float>(c, invd);
       L.D[CHEBMG_F32] = upload<float>(c, h.Dm);
     }

@@ -23,8 +23,8 @@ __device__ double g_eo_d[64];
 template <typename T, int EB_ = 2>
 struct Ax8 {
   static constexpr int EB = EB_;                       // elements per block
-  static constexpr int R = sizeof(T) == 4 ? 12 : 10;   // padded row stride (16-B aligned rows)
-  static constexpr int P = sizeof(T) == 4 ? 104 : 88;  // padded plane stride (bank spread)
+  static constexpr int R = 12;    // padded row stride (16-B aligned rows)
+  static constexpr int P = 100;   // padded plane stride (see line_of)
   static constexpr int STAGE = 8 * P;
   static constexpr int GELEM = 6 * 512;
   static size_t smem_bytes() { return sizeof(T) * (size_t)EB * (GELEM + 3 * STAGE); }

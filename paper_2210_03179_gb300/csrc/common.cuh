@@ -134,6 +134,11 @@ void sem_prolong(int Qf, int Qc, int64_t E, const uint32_t* gidf, const uint32_t
                  const T* J, const T* zc, T* zf, int accumulate, cudaStream_t s, int nb = 1, int64_t ldf = 0,
                  int64_t ldc = 0);
 
+// Order-7 geometric factors, E x [6][512] with a plane's 64 points as [j][i] -> in the order of the
+// operator's threads (line_of in ax8_util.cuh), in place; every order-7 kernel reads them so.
+template <typename T>
+void permute_g8(int64_t E, T* G, cudaStream_t s);
+
 // Order-7 element operator (line passes, even-odd D, TMA-staged geometric factors).
 // sem_ax8_set_D uploads the even-odd blocks of the 8x8 GLL derivative matrix (row-major).
 cudaError_t sem_ax8_set_D(const double* D);

@@ -44,7 +44,7 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   T* sS = sR + EB * C::STAGE;
 
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t e0 = (int64_t)blockIdx.x * EB;
   const int nvalid = (int)((E - e0) < EB ? (E - e0) : EB);
   const bool valid = le < nvalid;
@@ -110,7 +110,7 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   const T* gG = sG + le * C::GELEM;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const int p = k * 64 + b * 8 + a;
+    const int p = k * 64 + t;
     const int q = k * P + b * R + a;
     const T ur = sr[q], us = ss[q], utk = ut[k];
     const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
@@ -165,7 +165,7 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   T* sR = sU + EB_ * C::STAGE;
   T* sS = sR + EB_ * C::STAGE;
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t e = (int64_t)blockIdx.x * EB_ + le;
   const bool valid = e < E;
   T* su = sU + le * C::STAGE;
@@ -199,7 +199,7 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   const T* gG = G + (valid ? e : 0) * C::GELEM;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const int p = k * 64 + b * 8 + a;
+    const int p = k * 64 + t;
     const int q = k * P + b * R + a;
     const T ur = sr[q], us = ss[q], utk = ut[k];
     const T g00 = __ldg(gG + p), g01 = __ldg(gG + 512 + p), g02 = __ldg(gG + 1024 + p);
@@ -259,7 +259,7 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   T* sR = sU + EB * C::STAGE;
   T* sS = sR + EB * C::STAGE;
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t nbatch = (E + EB - 1) / EB;
   int64_t batch = blockIdx.x;
   if (batch >= nbatch) return;
@@ -341,7 +341,7 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     const T* gG = sG + buf * EB * C::GELEM + le * C::GELEM;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int p = k * 64 + b * 8 + a;
+      const int p = k * 64 + t;
       const int q = k * P + b * R + a;
       const T ur = sr[q], us = ss[q], utk = ut[k];
       const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
@@ -405,7 +405,7 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   T* sR = sU + EB * C::STAGE;
   T* sS = sR + EB * C::STAGE;
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t e0 = (int64_t)blockIdx.x * EB;
   const int nvalid = (int)((E - e0) < EB ? (E - e0) : EB);
   const bool valid = le < nvalid;
@@ -475,7 +475,7 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     const T* gG = sG + le * C::GELEM;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int p = k * 64 + b * 8 + a;
+      const int p = k * 64 + t;
       const int qq = k * P + b * R + a;
       const T ur = sr[qq], us = ss[qq], utk = ut[k];
       const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
@@ -536,14 +536,14 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   T* sR = sU + EB * C::STAGE;
   T* sS = sR + EB * C::STAGE;
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t e = (int64_t)blockIdx.x * EB + le;
   const bool valid = e < E;
   const int q0 = blockIdx.y * rb;
   const int q1 = q0 + rb < nb ? q0 + rb : nb;
   T gr[6][8];
   {
-    const T* gG = G + (valid ? e : 0) * C::GELEM + b * 8 + a;
+    const T* gG = G + (valid ? e : 0) * C::GELEM + t;
 #pragma unroll
     for (int c = 0; c < 6; ++c)
 #pragma unroll
@@ -641,7 +641,7 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sStage = sG + EB * C::GELEM;   // [2 right-hand sides][3 stages][EB][STAGE]
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t e0 = (int64_t)blockIdx.x * EB;
   const int nvalid = (int)((E - e0) < EB ? (E - e0) : EB);
   const bool valid = le < nvalid;
@@ -722,7 +722,7 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
     const T* gG = sG + le * C::GELEM;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int p = k * 64 + b * 8 + a;
+      const int p = k * 64 + t;
       const int qq = k * P + b * R + a;
       const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
       const T g11 = gG[1536 + p], g12 = gG[2048 + p], g22 = gG[2560 + p];
@@ -776,7 +776,25 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   }
 }
 
+// Four planes of 64 points per block (E x 48 planes).
+template <typename T>
+__global__ void __launch_bounds__(256) k_permute_g8(T* __restrict__ G) {
+  const int t = threadIdx.x & 63;
+  T* plane = G + ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 6)) * 64;
+  const T v = plane[line_of(t) * 8 + (t & 7)];
+  __syncthreads();
+  plane[t] = v;
+}
+
 }  // namespace
+
+template <typename T>
+void permute_g8(int64_t E, T* G, cudaStream_t s) {
+  k_permute_g8<T><<<(unsigned)(E * 12), 256, 0, s>>>(G);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+}
+template void permute_g8<float>(int64_t, float*, cudaStream_t);
+template void permute_g8<double>(int64_t, double*, cudaStream_t);
 
 cudaError_t sem_ax8_set_D(const double* D) {
   // symmetrised even-odd blocks of D and D^T (D[7-i][7-l] = -D[i][l] exactly)

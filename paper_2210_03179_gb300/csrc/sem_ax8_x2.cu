@@ -21,7 +21,7 @@ namespace {
 // even-odd blocks as FP32 pairs: [0] E of D, [1] O of D, [2] E of D^T, [3] O of D^T
 __constant__ f32x2 c_eo_x2[4][4][4];
 
-constexpr int kR = 10, kP = 88, kStage = 8 * kP, kGElem = 6 * 512;   // same strides as FP64
+constexpr int kR = 9, kP = 76, kStage = 8 * kP, kGElem = 6 * 512;   // fewest bank conflicts for 8-byte values
 
 template <int W>
 __device__ __forceinline__ void line8_x2(const f32x2 (&u)[8], f32x2 (&o)[8]) {
@@ -61,7 +61,7 @@ k_sem_ax8_x2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const f32
   f32x2* sS = sR + EB * kStage;
 
   const int tid = threadIdx.x;
-  const int le = tid >> 6, t = tid & 63, a = t & 7, b = t >> 3;
+  const int le = tid >> 6, t = tid & 63, a = t & 7, b = line_of(t);
   const int64_t e0 = (int64_t)blockIdx.x * EB;
   const int nvalid = (int)((E - e0) < EB ? (E - e0) : EB);
   const bool valid = le < nvalid;
@@ -140,7 +140,7 @@ k_sem_ax8_x2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const f32
     const f32x2* gG = sG + le * kGElem;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const int p = k * 64 + b * 8 + a;
+      const int p = k * 64 + t;
       const int qq = k * kP + b * kR + a;
       const f32x2 ur = sr[qq], us = ss[qq], utk = ut[k];
       const f32x2 g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];

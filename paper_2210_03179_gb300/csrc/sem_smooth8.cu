@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
   }
 
   // ---------------- compute warps ----------------
-  const int le = tid >> 6, tt = tid & 63, ca = tt & 7, cb = tt >> 3;
+  const int le = tid >> 6, tt = tid & 63, ca = tt & 7, cb = line_of(tt);
   T* Y = static_cast<T*>(a.y);
   T* su = sU + le * C::STAGE;
   T* sr = sR + le * C::STAGE;
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
         T wt[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int p = k * 64 + cb * 8 + ca;
+          const int p = k * 64 + tt;
           const int qq = k * P + cb * R + ca;
           const T ur = sr[qq], us = ss[qq], utk = ut[k];
           const T g00 = gG[p], g01 = gG[512 + p], g02 = gG[1024 + p];
