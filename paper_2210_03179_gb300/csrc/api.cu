@@ -761,6 +761,14 @@ int coarse_solve64_batched(chebmg_ctx* c, const double* b, double* x) {
     a.pf32 = c->coarse_pf32 ? 1 : 0;
     a.valf = c->ell_valf;
     a.invDf = c->coarse_invDf;
+    a.lat_nx = a.lat_nxy = 0;
+    if (c->lat_val) {
+      a.nslot = 27;
+      a.val = c->lat_val;
+      a.valf = c->lat_valf;
+      a.lat_nx = c->cc_nx;
+      a.lat_nxy = c->cc_nx * c->cc_ny;
+    }
     if (!coarse_block_launch(a, c->nb, c->s)) throw Error(CHEBMG_ECUDA, "batched coarse launch failed");
     check_launch();
     return CHEBMG_OK;

@@ -43,42 +43,6 @@ size_t lat_smem(int block, int nx) {
   return 2 * w * (sizeof(double) + sizeof(float)) + 2 * 3 * sizeof(double) * (size_t)block;
 }
 
-__device__ __forceinline__ double wsum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Block sums of three values, in every thread, fixed order; one warp adds through shared memory (few
-// FP64 instructions).  `buf` alternates between calls, so no barrier is needed before the writes.
-__device__ __forceinline__ void block_sum3(double* buf, double* res, double& a, double& b, double& c) {
-  const int T = blockDim.x;
-  buf[threadIdx.x] = a;
-  buf[T + threadIdx.x] = b;
-  buf[2 * T + threadIdx.x] = c;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-    for (int q = threadIdx.x; q < T; q += 32) {
-      t0 += buf[q];
-      t1 += buf[T + q];
-      t2 += buf[2 * T + q];
-    }
-    t0 = wsum(t0);
-    t1 = wsum(t1);
-    t2 = wsum(t2);
-    if (threadIdx.x == 0) {
-      res[0] = t0;
-      res[1] = t1;
-      res[2] = t2;
-    }
-  }
-  __syncthreads();
-  a = res[0];
-  b = res[1];
-  c = res[2];
-}
-
 // M: band words a thread loads per product (at most); MAXT: threads per block (at most).  Up to 256
 // threads the coefficients stay in registers.
 template <bool PF32, int M, int MAXT>

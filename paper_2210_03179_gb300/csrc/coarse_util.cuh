@@ -1,5 +1,5 @@
-// Helpers shared by the persistent coarse CG kernels (kernels.cu, coarse_lat.cu): the clock of their
-// bounded waits and the tagged-word exchange.
+// Helpers shared by the coarse CG kernels (kernels.cu, coarse_lat.cu, batched.cu): the clock of their
+// bounded waits, the tagged-word exchange and block sums.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -78,6 +78,43 @@ struct Tagged<double> {
   }
   static __device__ __forceinline__ double coef(const CoarseCG& a, int64_t i) { return __ldg(&a.val[i]); }
 };
+
+__device__ __forceinline__ double warp_total(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Block sums of three values, in every thread, fixed order; one warp adds through shared memory (few
+// FP64 instructions).  buf: 3 blockDim.x values.  buf and res alternate between calls, so no
+// barrier is needed before the writes.
+__device__ __forceinline__ void block_sum3(double* buf, double* res, double& a, double& b, double& c) {
+  const int T = blockDim.x;
+  buf[threadIdx.x] = a;
+  buf[T + threadIdx.x] = b;
+  buf[2 * T + threadIdx.x] = c;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+    for (int q = threadIdx.x; q < T; q += 32) {
+      t0 += buf[q];
+      t1 += buf[T + q];
+      t2 += buf[2 * T + q];
+    }
+    t0 = warp_total(t0);
+    t1 = warp_total(t1);
+    t2 = warp_total(t2);
+    if (threadIdx.x == 0) {
+      res[0] = t0;
+      res[1] = t1;
+      res[2] = t2;
+    }
+  }
+  __syncthreads();
+  a = res[0];
+  b = res[1];
+  c = res[2];
+}
 
 }  // namespace
 }  // namespace chebmg
