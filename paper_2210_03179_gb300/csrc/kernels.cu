@@ -128,7 +128,7 @@ static void launch_sem_ax(int64_t E, const uint32_t* gid, const T* G, const T* D
 // factors of the t-line (24 values) and D (16) are loaded into registers before the gather
 // (and, under programmatic dependent launch, before waiting for the kernel that wrote u).
 // IMPLICIT: global ids from the box lattice (ids and Dirichlet flags computed, no map read).
-constexpr int kAx4Threads = 256;                 // 16 elements per block
+constexpr int kAx4Threads = 64;                  // 4 elements per block: small levels spread over the SMs
 constexpr int kAx4Plane = 20;                    // padded k-plane stride: conflict-free s lines
 
 template <typename T, bool IMPLICIT>

@@ -7,16 +7,16 @@
 // for every FMA and is bound by them).  The derivative matrix is centro-antisymmetric,
 // D[Q-1-i][Q-1-l] = -D[i][l]: sums and differences of mirrored points halve the multiplications
 // (h = Q / 2 of each; odd Q has a middle point that joins the even half and a middle row of
-// differences alone).  FP32 keeps the factors of a thread's t-line in registers, all loads in
-// flight before the gather; FP64, bound by its FP64 pipe, reads them where they are used.
+// differences alone).
 // Strides R (rows) and P (planes) are those with the fewest bank conflicts over the passes.
 //
 // Measured, one thread per point -> line passes, with the zeroing of the output (6 to 12 us):
 // FP32 order 9 on 23^3 elements 215.5 -> 116.9 us and on 13^3 44.9 -> 24.6, order 8 on 25^3
 // 242.5 -> 92.3, order 5 on 38^3 164.8 -> 91.3, order 2 on 42^3 26.7 -> 22.5; FP64 order 9 on 23^3
 // 1555 -> 1334, order 5 on 38^3 932 -> 874, order 2 on 42^3 109.7 -> 102.4.  Then, with the FP64
-// coefficients in shared memory: order 9 1334 -> 1216 us, order 5 874 -> 833; and with three blocks of
-// the FP32 order-9 form per SM (80 registers, a little spilling): 116.9 -> 105.0 and 24.6 -> 20.0 us.
+// coefficients in shared memory: order 9 1334 -> 1216 us, order 5 874 -> 833; and with the FP32 factors
+// read where they are used instead of held in registers (twice the elements in flight per SM): order
+// 9 116.9 -> 87.2 us on 23^3 and 18.9 -> 13.4 on 12^3, order 8 90.3 -> 75.2, order 5 87.5 -> 83.1.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -76,9 +76,13 @@ template <typename T, int Q>
 struct AxL {
   static constexpr bool F = sizeof(T) == 4;
   static constexpr int QQ = Q * Q, NP = Q * Q * Q;
-  // elements per block: nearly whole warps (FP64 pays for every idle lane of its last warp)
-  static constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : Q == 9 ? 3 : F ? 2 : 5;
-  static constexpr int MINB = Q == 9 ? 2 : Q == 10 && F ? 3 : 1;   // blocks per SM to fit registers for
+  // FP32 reads the factors where they are used, with small blocks and many of them per SM; at order 6
+  // holding them in registers was faster (87.2 against 91.3 us on 33^3 elements)
+  static constexpr bool GREG = F && (Q == 7 || Q == 3);
+  // elements per block: FP64 nearly whole warps (it pays for every idle lane of its last warp)
+  static constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : F ? 1 : Q == 9 ? 3 : 5;
+  // blocks per SM to fit registers for
+  static constexpr int MINB = F ? (Q == 10 ? 9 : Q == 9 ? 10 : Q == 6 ? 4 : Q == 5 ? 8 : 1) : (Q == 9 ? 2 : 1);
   static constexpr int THREADS = (EB * QQ + 31) / 32 * 32;
   static constexpr int R = F ? (Q == 3 ? 4 : Q == 5 ? 6 : Q == 6 ? 9 : Q == 7 ? 8 : Q) : (Q == 6 ? 9 : Q);
   static constexpr int P = F ? (Q == 3 ? 35 : Q == 5 ? 37 : Q == 6 ? 70 : Q == 7 ? 71 : Q == 9 ? 81 : 101)
@@ -149,7 +153,7 @@ k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   T* sr = su + C::STAGE;
   T* ss = sr + C::STAGE;
   const T* Ge = G + (valid ? e : 0) * (6 * NP) + t;
-  constexpr bool GREG = sizeof(T) == 4;
+  constexpr bool GREG = C::GREG;
   T gr[GREG ? 6 : 1][GREG ? Q : 1];
   if constexpr (GREG) {
 #pragma unroll
