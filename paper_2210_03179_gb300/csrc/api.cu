@@ -73,7 +73,7 @@ namespace chebmg {
 const double* beta_row(int k) { return (k >= 1 && k <= 16) ? kBeta[k - 1] : nullptr; }
 void set_last_error(const char* msg) { g_last_error = msg; }
 
-enum { VB = 0, VX = 1, VR = 2, VD = 3, VY = 4, NV = 5 };
+enum { VB = 0, VX = 1, VR = 2, VD = 3, VY = 4, VP = 5, NV = 6 };   // VP (FD): the pre-smoother's iterate
 enum { TYPE_SEM = 0, TYPE_FD = 1 };
 
 struct Level {
@@ -290,7 +290,7 @@ void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld, b
     else if (L.Q == 4 && L.ax4[dt] % 100 == 41)
       sem_ax4<T>(L.E, L.gid, L.ax4[dt] >= 100 ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]),
                  static_cast<const T*>(L.D[dt]), x, y, c->s, nb, ld, subtract);
-    else if (sem_axl_supported(L.Q))
+    else if (sem_axl_chosen<T>(L.Q, L.E * nb))
       sem_axl<T>(L.Q, L.E, L.gid, L.boxed ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]), x, y, c->s, nb, ld,
                  subtract);
     else
@@ -317,7 +317,7 @@ void apply_subtract(chebmg_ctx* c, int j, const T* x, T* r) {
 template <typename T>
 void zero(chebmg_ctx* c, T* p, int64_t n) {
   // inside a chain of programmatic dependent launches a zeroing kernel keeps the chain going
-  if (pdl_on(c->s)) zero_bytes(p, (int64_t)sizeof(T) * n, c->s);
+  if (g_pdl) zero_bytes(p, (int64_t)sizeof(T) * n, c->s);
   else CK(cudaMemsetAsync(p, 0, sizeof(T) * (size_t)n, c->s));
 }
 
@@ -461,7 +461,7 @@ void smooth_sem(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero, 
   const int64_t n = L.n, ld = ldv(c, L);
   const int nb = c->nb;
   // one right-hand side: the step kernels launch as programmatic dependents of each other
-  const PdlScope pdl_(g_pdl || nb == 1);
+  const PdlScope pdl_(g_pdl || nb == 1, c->s);
   T* r = vec<T>(L, VR);
   T* d = vec<T>(L, VD);
   const T* S = invD_of<T>(L);
@@ -486,13 +486,14 @@ void smooth_sem(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero, 
   check_launch();
 }
 
-// smooth() on an FD level: one kernel per step, d alternating between VD and VY.
+// smooth() on an FD level: one kernel per step, d alternating between VD and VY.  have_r: r = b - A x and
+// d = c0 S r are in VR and VD already.
 template <typename T>
-void smooth_fd(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero) {
+void smooth_fd(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero, bool have_r = false) {
   Level& L = c->L[j];
   const int64_t n = L.n, ld = ldv(c, L);
   const int nb = c->nb;
-  const PdlScope pdl_(g_pdl || nb == 1);
+  const PdlScope pdl_(g_pdl || nb == 1, c->s);
   T *r = vec<T>(L, VR), *d = vec<T>(L, VD), *dn = vec<T>(L, VY);
   const Stencil9<double> st = stencil(L);
   const Recurrence q = recurrence(c, L, order);
@@ -509,7 +510,7 @@ void smooth_fd(chebmg_ctx* c, int j, const T* b, T* x, int order, bool x_zero) {
   } else if (x_zero) {
     smooth_begin<T>(n, b, x, r, d, invD_of<T>(L), q.c0, order == 1, q.w[0], nullptr, c->s, nb, ld);
   } else {
-    fd_resid<T>(L.mx, L.my, st, b, x, r, d, q.c0, c->s, nb, ld);
+    if (!have_r) fd_resid<T>(L.mx, L.my, st, b, x, r, d, q.c0, c->s, nb, ld);
     if (order == 1) axpy<T>(n, q.w[0], d, x, c->s, nb, ld);
   }
   for (; i < order; ++i) {
@@ -810,19 +811,50 @@ void apply_outer(chebmg_ctx* c, const double* p, double* q) {
   apply_into<double>(c, 0, p, q);
 }
 
-// VB of level j + 1 = P^T (b - A x), r = b - A x already in VR where have_r.
 template <typename T>
-void residual_restrict(chebmg_ctx* c, int j, const T* b, const T* x, bool have_r) {
+int vcycle_level(chebmg_ctx* c, int j, const T* b, T* x);
+
+// x = V-cycle(b) from FD level j.  xm, if given, keeps the iterate before the post-smoother;
+// `coarser` runs level j + 1.
+template <typename T, typename F>
+int vcycle_fd(chebmg_ctx* c, int j, const T* b, T* x, T* xm, F&& coarser) {
   Level& L = c->L[j];
   Level& C = c->L[j + 1];
-  T *r = vec<T>(L, VR), *rc = vec<T>(C, VB);
-  if (!have_r && L.c_next == 2) {
-    fd_resid_restrict<T>(L.mx, L.my, C.mx, C.my, stencil(L), b, x, rc, c->s, c->nb, ldv(c, L), ldv(c, C));
-    check_launch();
-    return;
+  const int nb = c->nb;
+  const int64_t ldf = ldv(c, L), ldc = ldv(c, C);
+  const Stencil9<double> st = stencil(L);
+  const PdlScope pdl_(g_pdl || nb == 1, c->s);
+  const bool two = L.c_next == 2;
+  T *xp = two ? vec<T>(L, VP) : x, *r = vec<T>(L, VR), *rc = vec<T>(C, VB), *zc = vec<T>(C, VX);
+  if (two && (c->pre == 1 || c->pre == 2)) {
+    const Recurrence q = recurrence(c, L, c->pre);
+    fd_smooth_restrict<T>(L.mx, L.my, C.mx, C.my, st, b, xp, rc, c->pre, q.c0, c->pre == 2 ? q.c1[1] : 0.0,
+                          c->pre == 2 ? q.c2[1] : 0.0, q.w[0], c->pre == 2 ? q.w[1] : 0.0, c->s, nb, ldf, ldc);
+  } else {
+    if (c->pre > 0) smooth_fd<T>(c, j, b, xp, c->pre, true);
+    else zero<T>(c, xp, span(c, L));
+    if (two) {
+      fd_resid_restrict<T>(L.mx, L.my, C.mx, C.my, st, b, xp, rc, c->s, nb, ldf, ldc);
+    } else {
+      fd_resid<T>(L.mx, L.my, st, b, xp, r, static_cast<T*>(nullptr), 0.0, c->s, nb, ldf);
+      restrict_to<T>(c, j, r, rc);
+    }
   }
-  if (!have_r) fd_resid<T>(L.mx, L.my, stencil(L), b, x, r, static_cast<T*>(nullptr), 0.0, c->s, c->nb, ldv(c, L));
-  restrict_to<T>(c, j, r, rc);
+  check_launch();
+  const int rcode = coarser(rc, zc);
+  if (rcode != CHEBMG_OK && rcode != CHEBMG_ENOTCONV) return rcode;
+  if (two) {
+    const bool post = c->post > 0;
+    const double c0 = post ? recurrence(c, L, c->post).c0 : 0.0;
+    fd_prolong_resid<T>(L.mx, L.my, C.mx, C.my, st, xp, zc, b, x, xm, post ? r : nullptr,
+                        post ? vec<T>(L, VD) : nullptr, c0, c->s, nb, ldf, ldc);
+  } else {
+    prolong_to<T>(c, j, zc, x, 1);
+    if (xm) cast<T, T>(L.n, x, xm, c->s, nb, ldf, ldf);
+  }
+  if (c->post > 0) smooth_fd<T>(c, j, b, x, c->post, false, two);
+  check_launch();
+  return rcode;
 }
 
 // z = V-cycle(b) from level j (Eq. 2.2), in precision T.
@@ -831,22 +863,22 @@ int vcycle_level(chebmg_ctx* c, int j, const T* b, T* x) {
   if (j == (int)c->L.size() - 1) return coarse<T>(c, b, x);
   Level& L = c->L[j];
   Level& C = c->L[j + 1];
+  if (L.type == TYPE_FD)
+    return vcycle_fd<T>(c, j, b, x, static_cast<T*>(nullptr),
+                        [&](const T* rc, T* zc) { return vcycle_level<T>(c, j + 1, rc, zc); });
   // the fused kernel computes the restriction residual in the same launch as the pre-smoother; the
-  // separate SEM kernels leave r = b, from which one more product subtracts A x; the FD restriction
-  // by two forms the residual itself
-  const bool sem = L.type == TYPE_SEM;
+  // separate kernels leave r = b, from which one more product subtracts A x
   T* r = vec<T>(L, VR);
   bool have_r = false;
   if (c->pre > 0) {
     have_r = smooth_fused<T>(c, j, b, x, c->pre, true, true);
-    if (!have_r && sem) smooth_sem<T>(c, j, b, x, c->pre, true, true);
-    else if (!have_r) smooth_fd<T>(c, j, b, x, c->pre, true);
+    if (!have_r) smooth_sem<T>(c, j, b, x, c->pre, true, true);
   } else {
     zero<T>(c, x, span(c, L));
-    if (sem) cast<T, T>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
+    cast<T, T>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
   }
-  if (!have_r && sem) apply_subtract<T>(c, j, x, r);
-  residual_restrict<T>(c, j, b, x, sem);
+  if (!have_r) apply_subtract<T>(c, j, x, r);
+  restrict_to<T>(c, j, r, vec<T>(C, VB));
   int rc = vcycle_level<T>(c, j + 1, vec<T>(C, VB), vec<T>(C, VX));
   if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
   prolong_to<T>(c, j, vec<T>(C, VX), x, 1);
@@ -941,9 +973,10 @@ double lanczos(chebmg_ctx* c, int j, int steps) {
 }
 
 void alloc_vectors(chebmg_ctx* c, Level& L, bool with32) {
-  for (int w = 0; w < NV; ++w) L.v[CHEBMG_F64][w] = dalloc<double>(c, L.ld);
+  const int nv = L.type == TYPE_FD ? NV : VP;
+  for (int w = 0; w < nv; ++w) L.v[CHEBMG_F64][w] = dalloc<double>(c, L.ld);
   if (with32)
-    for (int w = 0; w < NV; ++w) L.v[CHEBMG_F32][w] = dalloc<float>(c, L.ld);
+    for (int w = 0; w < nv; ++w) L.v[CHEBMG_F32][w] = dalloc<float>(c, L.ld);
 }
 
 void common_alloc(chebmg_ctx* c) {
@@ -1791,15 +1824,15 @@ int vcycle_store(chebmg_ctx* c, int j, const double* b, double* x) {
   if (j == last) return coarse<double>(c, b, x);
   Level& L = c->L[j];
   Level& C = c->L[j + 1];
+  if (L.type == TYPE_FD)
+    return vcycle_fd<double>(c, j, b, x, c->post > 0 ? c->gw.lv[j][GW_XM] : nullptr,
+                             [&](const double* rc, double* zc) { return vcycle_store(c, j + 1, rc, zc); });
   if (c->pre > 0) smooth<double>(c, j, b, x, c->pre, true);
   else zero<double>(c, x, span(c, L));
-  const bool sem = L.type == TYPE_SEM;
-  if (sem) {
-    double* r = vec<double>(L, VR);
-    cast<double, double>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
-    apply_subtract<double>(c, j, x, r);
-  }
-  residual_restrict<double>(c, j, b, x, sem);
+  double* r = vec<double>(L, VR);
+  cast<double, double>(L.n, b, r, c->s, c->nb, ldv(c, L), ldv(c, L));
+  apply_subtract<double>(c, j, x, r);
+  restrict_to<double>(c, j, r, vec<double>(C, VB));
   const int rc = vcycle_store(c, j + 1, vec<double>(C, VB), vec<double>(C, VX));
   if (rc != CHEBMG_OK && rc != CHEBMG_ENOTCONV) return rc;
   prolong_to<double>(c, j, vec<double>(C, VX), x, 1);
@@ -2002,7 +2035,7 @@ int cycle_error_grad(chebmg_ctx* c, int nrhs, const double* E0, int steps, const
   c->beta_ovr.assign(betas, betas + nbeta);
   c->lscale = scale;
   BatchScope bs(c, nrhs);
-  const PdlScope pdl_(true);   // never captured: the kernels launch as a dependent chain
+  const PdlScope pdl_(true, c->s);   // never captured: the kernels launch as a dependent chain
   Level& L = c->L[0];
   const int64_t n = L.n, ld = ldv(c, L), sp = span(c, L);
   const double* S = static_cast<const double*>(L.invD[CHEBMG_F64]);
@@ -2869,7 +2902,7 @@ int chebmg_set_outer_operator(chebmg_ctx* c, int kind) {
 int chebmg_apply_outer(chebmg_ctx* c, const double* x, double* y) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     if (!x || !y) throw Error(CHEBMG_EINVAL, "NULL vector");
     zero<double>(c, y, c->L[0].n);
     apply_outer(c, x, y);
@@ -2881,7 +2914,7 @@ int chebmg_apply_outer(chebmg_ctx* c, const double* x, double* y) {
 int chebmg_apply_A(chebmg_ctx* c, int level, int dtype, const void* x, void* y) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     Level& L = level_checked(c, level);
     check_dtype(c, dtype);
     if (!x || !y) throw Error(CHEBMG_EINVAL, "NULL vector");
@@ -2912,7 +2945,7 @@ int chebmg_inv_diagonal(chebmg_ctx* c, int level, int dtype, void* out) {
 int chebmg_smooth(chebmg_ctx* c, int level, int dtype, const void* b, void* x, int order, int x_is_zero) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     Level& L = level_checked(c, level);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "the coarsest level is not smoothed");
@@ -2931,7 +2964,7 @@ int chebmg_smooth(chebmg_ctx* c, int level, int dtype, const void* b, void* x, i
 int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* rc) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     level_checked(c, level);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
@@ -2945,7 +2978,7 @@ int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* r
 int chebmg_prolong(chebmg_ctx* c, int level, int dtype, const void* zc, void* zf, int accumulate) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     level_checked(c, level);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
@@ -2979,7 +3012,7 @@ int chebmg_coarse_solve(chebmg_ctx* c, const double* r, double* z, int* iters) {
 int chebmg_vcycle(chebmg_ctx* c, const double* r, double* z) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     if (!r || !z) throw Error(CHEBMG_EINVAL, "NULL vector");
     reset_coarse_sticky(c);
     int rc = vcycle_top(c, r, z);
@@ -2994,7 +3027,7 @@ int chebmg_pcg_solve(chebmg_ctx* c, const double* b, double* u, double rtol, int
                      double* relres, double* history) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1);   // the solve's kernels launch as programmatic dependents
+    const PdlScope pdl_(c->nb == 1, c->s);   // the solve's kernels launch as programmatic dependents
     if (!b || !u || maxit < 0 || !(rtol > 0.0)) throw Error(CHEBMG_EINVAL, "bad solve arguments");
     Level& L = c->L[0];
     const int64_t n = L.n;
@@ -3270,7 +3303,7 @@ int chebmg_gmres_solve(chebmg_ctx* c, const double* b, double* u, double rtol, i
     enter(c);
     if (!b || !u || maxit < 0 || !(rtol > 0.0) || restart < 1 || restart + 1 > gmres_max_basis())
       throw Error(CHEBMG_EINVAL, "bad GMRES arguments");
-    const PdlScope pdl_(c->nb == 1);
+    const PdlScope pdl_(c->nb == 1, c->s);
     return gmres_solve(c, b, u, rtol, restart, maxit, iters, relres, history);
   });
 }

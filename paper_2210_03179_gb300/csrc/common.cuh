@@ -20,21 +20,21 @@ extern std::atomic<int64_t> g_launches;
 // operations are visible -- before its first global memory access.  Launches into a stream
 // that is being captured are ordinary launches.
 extern thread_local bool g_pdl;
+// A scope belongs to one stream and does not outlast a call, so the stream's capture status is
+// looked up once here instead of at every launch.
 struct PdlScope {
   bool old;
-  explicit PdlScope(bool on) : old(g_pdl) { g_pdl = on; }
+  PdlScope(bool on, cudaStream_t s) : old(g_pdl) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    g_pdl = on && cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+  }
   ~PdlScope() { g_pdl = old; }
   PdlScope(const PdlScope&) = delete;
   PdlScope& operator=(const PdlScope&) = delete;
 };
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-inline bool pdl_on(cudaStream_t s) {
-  if (!g_pdl) return false;
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
-}
 // Launches kernel k (which must begin with pdl_wait()) as a programmatic dependent when
-// pdl_on(s), else as an ordinary launch; counts the launch.
+// g_pdl is set, else as an ordinary launch; counts the launch.
 template <typename... KArgs, typename... Args>
 inline void launch_dep(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -46,7 +46,7 @@ inline void launch_dep(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = pdl_on(s) ? 1 : 0;
+  cfg.numAttrs = g_pdl ? 1 : 0;
   cudaLaunchKernelEx(&cfg, k, static_cast<Args&&>(args)...);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
@@ -155,6 +155,8 @@ void sem_ax4(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, con
 // Orders 2, 4, 5, 6, 8 and 9 (Q = 3, 5, 6, 7, 9, 10) by line passes (sem_axl.cu); ids from the box
 // lattice when lat is given, else from gid.  sem_axl_set_D uploads the order's derivative matrix.
 bool sem_axl_supported(int Q);
+template <typename T>
+bool sem_axl_chosen(int Q, int64_t elements);   // else sem_ax
 cudaError_t sem_axl_set_D(int Q, const double* D);
 template <typename T>
 void sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
@@ -278,6 +280,16 @@ void fd_resid(int mx, int my, const Stencil9<double>& st, const T* b, const T* x
 template <typename T>
 void fd_resid_restrict(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* b, const T* x, T* rc,
                        cudaStream_t s, int nb, int64_t ldf, int64_t ldc);
+// A smoother of order 1 or 2 from a zero guess (as fd_first; order 1: x = w0 c0 S b) and the restriction
+// of its residual in one: x and rc = P^T (b - A x), coarsening by two.
+template <typename T>
+void fd_smooth_restrict(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* b, T* x, T* rc, int order,
+                        double c0, double c1, double c2, double w0, double w1, cudaStream_t s, int nb, int64_t ldf,
+                        int64_t ldc);
+// x = xp + P xc (coarsening by two, x not xp), xm = x if given, and if r is given r = b - A x, d = c0 S r.
+template <typename T>
+void fd_prolong_resid(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* xp, const T* xc, const T* b,
+                      T* x, T* xm, T* r, T* d, double c0, cudaStream_t s, int nb, int64_t ldf, int64_t ldc);
 template <typename T>
 void fd_restrict(int mfx, int mfy, int mcx, int mcy, int c, const T* rf, T* rc, cudaStream_t s, int nb = 1,
                  int64_t ldf = 0, int64_t ldc = 0);

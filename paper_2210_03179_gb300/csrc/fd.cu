@@ -11,7 +11,7 @@
 // with a constant operand issues slower, and a five-point stencil skips its zero corners.
 // Separate operator and update kernels -> these: order-4 smoothing of 511 x 511 from a nonzero guess
 // 46.2 -> 30.8 us (of which about 15 us FP64 issue), a symmetric order-2 cycle on 63 x 63
-// 96.6 -> 40.6 us (27 -> 11 launches, and the dense coarse product 45.9 us -> a few).
+// 96.6 -> 32.1 us (27 -> 7 launches, the dense coarse product 45.9 us -> a few, small blocks).
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -20,7 +20,7 @@ namespace chebmg {
 
 namespace {
 
-constexpr int kBX = 32, kBY = 8;
+constexpr int kBX = 32, kBY = 8;   // threads of a block over the grid (kBY: at most)
 
 // A kernel parameter as a register operand the compiler cannot fold back.  Call it with whole warps.
 __device__ __forceinline__ double in_register(double v) { return __shfl_sync(0xffffffffu, v, 0); }
@@ -68,7 +68,7 @@ struct Pt {
 __device__ __forceinline__ Pt point(int mx, int my) {
   Pt p;
   p.i = blockIdx.x * kBX + threadIdx.x;
-  p.j = blockIdx.y * kBY + threadIdx.y;
+  p.j = blockIdx.y * blockDim.y + threadIdx.y;
   p.in = p.i < mx && p.j < my;
   p.g = (int64_t)p.j * mx + p.i;
   return p;
@@ -156,12 +156,13 @@ k_fd_resid(int mx, int my, Stencil9<T> st, const T* __restrict__ b, const T* __r
 
 // rc = P^T (b - A x) for coarsening by two (st = -A): a block forms the residual of the fine points
 // under its tile of coarse points in shared memory (one row and column shared with the next tile).
-constexpr int kTX = 16, kTY = 8;
-template <typename T, bool NINE>
-__global__ void __launch_bounds__(kTX * kTY)
+// TY coarse rows per block: 8, or 2 where 8 leave SMs idle (a block's points are FP64 work in series).
+constexpr int kTX = 16, kRestrictThreads = 256;
+template <typename T, bool NINE, int TY>
+__global__ void __launch_bounds__(kRestrictThreads)
 k_fd_resid_restrict(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* __restrict__ b,
                     const T* __restrict__ x, T* __restrict__ rc, int64_t ldf, int64_t ldc) {
-  constexpr int FX = 2 * kTX + 1, FY = 2 * kTY + 1;
+  constexpr int FX = 2 * kTX + 1, FY = 2 * TY + 1;
   __shared__ T sr[FY][FX + 1];
   T c[9];
   const Arith<T> ar;
@@ -170,8 +171,8 @@ k_fd_resid_restrict(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* _
   b += (int64_t)blockIdx.z * ldf;
   x += (int64_t)blockIdx.z * ldf;
   rc += (int64_t)blockIdx.z * ldc;
-  const int I0 = blockIdx.x * kTX, J0 = blockIdx.y * kTY;
-  for (int q = threadIdx.x; q < FX * FY; q += kTX * kTY) {
+  const int I0 = blockIdx.x * kTX, J0 = blockIdx.y * TY;
+  for (int q = threadIdx.x; q < FX * FY; q += kRestrictThreads) {
     const int fi = q % FX, fj = q / FX, i = 2 * I0 + fi, j = 2 * J0 + fj;
     T v = T(0), xc;
     if (i < mx && j < my) v = ar.add(stencil_sum<T, NINE>(ar, x, mx, my, i, j, c, xc), b[(int64_t)j * mx + i]);
@@ -179,7 +180,7 @@ k_fd_resid_restrict(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* _
   }
   __syncthreads();
   const int tx = threadIdx.x % kTX, ty = threadIdx.x / kTX, I = I0 + tx, J = J0 + ty;
-  if (I >= mcx || J >= mcy) return;
+  if (ty >= TY || I >= mcx || J >= mcy) return;
   T acc = T(0);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -188,6 +189,125 @@ k_fd_resid_restrict(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* _
     acc += (a == 1 ? T(1) : T(0.5)) * v;
   }
   rc[(int64_t)J * mcx + I] = acc;
+}
+
+// Orders 1 and 2 from a zero guess with the restriction of their residual: x depends on b alone, so a
+// block forms x on the fine points under its coarse tile and a rim of one, the residual there, and
+// restricts it; it writes the x it owns.  One launch instead of two, x not read back.
+template <typename T, bool NINE, int TY>
+__global__ void __launch_bounds__(kRestrictThreads)
+k_fd_smooth_restrict(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* __restrict__ b, T* __restrict__ x,
+                     T* __restrict__ rc, int order, T c0, T c1, T c2, T w0, T w1, int64_t ldf, int64_t ldc) {
+  constexpr int FX = 2 * kTX + 1, FY = 2 * TY + 1;
+  __shared__ T sx[FY + 2][FX + 2];
+  __shared__ T sr[FY][FX + 1];
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);    // -A
+  pdl_wait();
+  b += (int64_t)blockIdx.z * ldf;
+  x += (int64_t)blockIdx.z * ldf;
+  rc += (int64_t)blockIdx.z * ldc;
+  const int I0 = blockIdx.x * kTX, J0 = blockIdx.y * TY;
+  const bool lastx = blockIdx.x + 1 == gridDim.x, lasty = blockIdx.y + 1 == gridDim.y;
+  for (int q = threadIdx.x; q < (FX + 2) * (FY + 2); q += kRestrictThreads) {
+    const int sj = q / (FX + 2), si = q - sj * (FX + 2), i = 2 * I0 + si - 1, j = 2 * J0 + sj - 1;
+    T v = T(0);
+    if (i >= 0 && i < mx && j >= 0 && j < my) {
+      const int64_t g = (int64_t)j * mx + i;
+      if (order == 1) {
+        v = w0 * (c0 * b[g]);
+      } else {
+        T b0;
+        const T s = stencil_sum<T, NINE>(ar, b, mx, my, i, j, c, b0);
+        const T rv = fma(c0, s, b0), d0 = c0 * b0, dn = c1 * d0 + c2 * rv;
+        v = w0 * d0 + w1 * dn;
+      }
+      if (si >= 1 && sj >= 1 && (si <= 2 * kTX || lastx) && (sj <= 2 * TY || lasty)) x[g] = v;
+    }
+    sx[sj][si] = v;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < FX * FY; q += kRestrictThreads) {
+    const int fj = q / FX, fi = q - fj * FX, i = 2 * I0 + fi, j = 2 * J0 + fj;
+    T v = T(0);
+    if (i < mx && j < my) {
+      T acc = ar.mul(c[4], sx[fj + 1][fi + 1]);
+#pragma unroll
+      for (int k = 0; k < 9; ++k)
+        if (k != 4 && used<NINE>(k)) acc = fma(c[k], sx[fj + k / 3][fi + k % 3], acc);
+      v = ar.add(acc, b[(int64_t)j * mx + i]);
+    }
+    sr[fj][fi] = v;
+  }
+  __syncthreads();
+  const int tx = threadIdx.x % kTX, ty = threadIdx.x / kTX, I = I0 + tx, J = J0 + ty;
+  if (ty >= TY || I >= mcx || J >= mcy) return;
+  T acc = T(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const T* row = sr[2 * ty + a] + 2 * tx;
+    const T v = T(0.5) * (row[0] + row[2]) + row[1];
+    acc += (a == 1 ? T(1) : T(0.5)) * v;
+  }
+  rc[(int64_t)J * mcx + I] = acc;
+}
+
+// (P xc)(i, j), coarsening by two: even points lie between two coarse ones.
+template <typename T>
+__device__ __forceinline__ T interpolate2(const T* __restrict__ xc, int mcx, int mcy, int i, int j) {
+  const int I = ((i + 1) >> 1) - 1, J = ((j + 1) >> 1) - 1;
+  const bool di = !(i & 1), dj = !(j & 1);
+  const bool i0 = I >= 0, i1 = di && I + 1 < mcx, j0 = J >= 0, j1 = dj && J + 1 < mcy;
+  const T* r0 = xc + (int64_t)J * mcx + I;
+  const T a = (i0 && j0 ? r0[0] : T(0)), b = (i1 && j0 ? r0[1] : T(0));
+  const T e = (i0 && j1 ? r0[mcx] : T(0)), f = (i1 && j1 ? r0[mcx + 1] : T(0));
+  T s = dj ? (a + e) : a;
+  if (di) s += dj ? (b + f) : b;
+  return s * ((di ? T(0.5) : T(1)) * (dj ? T(0.5) : T(1)));
+}
+
+// x = xp + P xc (xm = x if given); with r: r = b - A x (st = -A), d = c0 r.  Out of place, so that a
+// block can form x on its tile and a rim of one and take the residual at once.
+template <typename T, bool NINE, int BY>
+__global__ void __launch_bounds__(kBX * BY)
+k_fd_prolong_resid(int mx, int my, int mcx, int mcy, Stencil9<T> st, const T* __restrict__ xp,
+                   const T* __restrict__ xc, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ xm,
+                   T* __restrict__ r, T* __restrict__ d, T c0, int64_t ldf, int64_t ldc) {
+  __shared__ T s[BY + 2][kBX + 2];
+  T c[9];
+  const Arith<T> ar;
+  load_stencil<T, NINE>(st, c);
+  pdl_wait();
+  const int64_t o = (int64_t)blockIdx.z * ldf;
+  xc += (int64_t)blockIdx.z * ldc;
+  const Pt p = point(mx, my);
+  if (!r) {
+    if (p.in) x[o + p.g] = xp[o + p.g] + interpolate2(xc, mcx, mcy, p.i, p.j);
+    return;
+  }
+  const int i0 = blockIdx.x * kBX - 1, j0 = blockIdx.y * BY - 1;
+  const int tid = threadIdx.y * kBX + threadIdx.x;
+  for (int q = tid; q < (kBX + 2) * (BY + 2); q += kBX * BY) {
+    const int sj = q / (kBX + 2), si = q - sj * (kBX + 2), i = i0 + si, j = j0 + sj;
+    T v = T(0);
+    if (i >= 0 && i < mx && j >= 0 && j < my)
+      v = xp[o + (int64_t)j * mx + i] + interpolate2(xc, mcx, mcy, i, j);
+    s[sj][si] = v;
+  }
+  const T b0 = p.in ? b[o + p.g] : T(0);
+  __syncthreads();
+  if (!p.in) return;
+  const int si = threadIdx.x + 1, sj = threadIdx.y + 1;
+  T acc = ar.mul(c[4], s[sj][si]);
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    if (k != 4 && used<NINE>(k)) acc = fma(c[k], s[sj + k / 3 - 1][si + k % 3 - 1], acc);
+  const T rv = ar.add(acc, b0);
+  x[o + p.g] = s[sj][si];
+  if (xm) xm[o + p.g] = s[sj][si];
+  r[o + p.g] = rv;
+  d[o + p.g] = c0 * rv;
 }
 
 // rc(I,J) = sum_{|a|,|b| < c} w_a w_b rf(c(I+1)-1+b, c(J+1)-1+a), w_d = (c - |d|)/c.  C: the factor
@@ -443,21 +563,46 @@ Stencil9<T> scaled(const Stencil9<double>& st, double f) {
   for (int q = 0; q < 9; ++q) o.c[q] = (T)(f * st.c[q]);
   return o;
 }
-dim3 grid_of(int mx, int my, int nb) { return dim3((mx + kBX - 1) / kBX, (my + kBY - 1) / kBY, nb); }
+dim3 grid_of(int mx, int my, int nb, int by = kBY) { return dim3((mx + kBX - 1) / kBX, (my + by - 1) / by, nb); }
+// Rows per block: `many`, or `few` where that leaves SMs without a block -- small grids are bound by the
+// FP64 work that the busiest SM does in series.  A symmetric order-2 cycle, tall blocks alone -> this:
+// 63 x 63 40.7 -> 32.1 us, 127 x 127 54.5 -> 42.8, 511 x 511 (its coarse levels) 103.0 -> 90.5.
+int rows_for(int mx, int my, int nb, int bx, int many, int few) {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  return (int64_t)((mx + bx - 1) / bx) * ((my + many - 1) / many) * nb < sms ? few : many;
+}
 
 }  // namespace
 
-// Launches K<T, true> or K<T, false> by the stencil's corners.
-#define FD_LAUNCH(K, st, grid, block, ...)                                    \
-  do {                                                                        \
-    if (nine(st)) launch_dep(K<T, true>, grid, block, 0, s, __VA_ARGS__);       \
-    else launch_dep(K<T, false>, grid, block, 0, s, __VA_ARGS__);               \
+// Launches K<T, true> or K<T, false> by the stencil's corners, a thread per point.
+#define FD_LAUNCH(K, st, ...)                                                      \
+  do {                                                                             \
+    const int by_ = rows_for(mx, my, nb, kBX, kBY, 2);                              \
+    const dim3 grid_ = grid_of(mx, my, nb, by_), block_(kBX, by_);                   \
+    if (nine(st)) launch_dep(K<T, true>, grid_, block_, 0, s, __VA_ARGS__);          \
+    else launch_dep(K<T, false>, grid_, block_, 0, s, __VA_ARGS__);                  \
+  } while (0)
+// The same for the tiled kernels, with ROWS (of `few` or `many`) rows per block.
+#define FD_LAUNCH_TILED(K, st, rows, few, many, grid, block, ...)                       \
+  do {                                                                                  \
+    if (nine(st)) {                                                                     \
+      if (rows == few) launch_dep(K<T, true, few>, grid, block, 0, s, __VA_ARGS__);       \
+      else launch_dep(K<T, true, many>, grid, block, 0, s, __VA_ARGS__);                  \
+    } else {                                                                            \
+      if (rows == few) launch_dep(K<T, false, few>, grid, block, 0, s, __VA_ARGS__);      \
+      else launch_dep(K<T, false, many>, grid, block, 0, s, __VA_ARGS__);                 \
+    }                                                                                   \
   } while (0)
 
 template <typename T>
 void fd_apply(int mx, int my, const Stencil9<double>& st, const T* u, T* y, cudaStream_t s, int nb, int64_t ld) {
   const Stencil9<T> a = scaled<T>(st, 1.0);
-  FD_LAUNCH(k_fd_apply, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, u, y, ld);
+  FD_LAUNCH(k_fd_apply, a, mx, my, a, u, y, ld);
 }
 
 template <typename T>
@@ -465,7 +610,7 @@ void fd_first(int mx, int my, const Stencil9<double>& st, const T* b, T* x, T* r
               double w0, double w1, bool last, cudaStream_t s, int nb, int64_t ld) {
   const double S = 1.0 / st.c[4];
   const Stencil9<T> a = scaled<T>(st, -c0 * S);
-  FD_LAUNCH(k_fd_first, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, b, x, r, d, (T)(c0 * S), (T)c1, (T)(c2 * S),
+  FD_LAUNCH(k_fd_first, a, mx, my, a, b, x, r, d, (T)(c0 * S), (T)c1, (T)(c2 * S),
             (T)w0, (T)w1, last ? 1 : 0, ld);
 }
 
@@ -473,7 +618,7 @@ template <typename T>
 void fd_step(int mx, int my, const Stencil9<double>& st, const T* d, T* dn, const T* rin, T* r, T* x, double c1,
              double c2, int xmode, double w0, double w1, bool last, cudaStream_t s, int nb, int64_t ld) {
   const Stencil9<T> a = scaled<T>(st, -1.0);
-  FD_LAUNCH(k_fd_step, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, d, dn, rin, r, x, (T)c1,
+  FD_LAUNCH(k_fd_step, a, mx, my, a, d, dn, rin, r, x, (T)c1,
             (T)(c2 / st.c[4]), xmode, (T)w0, (T)w1, last ? 1 : 0, ld);
 }
 
@@ -481,15 +626,37 @@ template <typename T>
 void fd_resid(int mx, int my, const Stencil9<double>& st, const T* b, const T* x, T* r, T* d, double c0, cudaStream_t s,
               int nb, int64_t ld) {
   const Stencil9<T> a = scaled<T>(st, -1.0);
-  FD_LAUNCH(k_fd_resid, a, grid_of(mx, my, nb), dim3(kBX, kBY), mx, my, a, b, x, r, d, (T)(c0 / st.c[4]), ld);
+  FD_LAUNCH(k_fd_resid, a, mx, my, a, b, x, r, d, (T)(c0 / st.c[4]), ld);
 }
 
 template <typename T>
 void fd_resid_restrict(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* b, const T* x, T* rc,
                        cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
   const Stencil9<T> a = scaled<T>(st, -1.0);
-  const dim3 grid((mcx + kTX - 1) / kTX, (mcy + kTY - 1) / kTY, nb);
-  FD_LAUNCH(k_fd_resid_restrict, a, grid, dim3(kTX * kTY), mx, my, mcx, mcy, a, b, x, rc, ldf, ldc);
+  const int ty = rows_for(mcx, mcy, nb, kTX, 8, 2);
+  const dim3 grid((mcx + kTX - 1) / kTX, (mcy + ty - 1) / ty, nb);
+  FD_LAUNCH_TILED(k_fd_resid_restrict, a, ty, 2, 8, grid, dim3(kRestrictThreads), mx, my, mcx, mcy, a, b, x, rc, ldf, ldc);
+}
+
+template <typename T>
+void fd_smooth_restrict(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* b, T* x, T* rc, int order,
+                        double c0, double c1, double c2, double w0, double w1, cudaStream_t s, int nb, int64_t ldf,
+                        int64_t ldc) {
+  const double S = 1.0 / st.c[4];
+  const Stencil9<T> a = scaled<T>(st, -1.0);
+  const int ty = rows_for(mcx, mcy, nb, kTX, 8, 2);
+  const dim3 grid((mcx + kTX - 1) / kTX, (mcy + ty - 1) / ty, nb);
+  FD_LAUNCH_TILED(k_fd_smooth_restrict, a, ty, 2, 8, grid, dim3(kRestrictThreads), mx, my, mcx, mcy, a, b, x, rc, order, (T)(c0 * S), (T)c1,
+            (T)(c2 * S), (T)w0, (T)w1, ldf, ldc);
+}
+
+template <typename T>
+void fd_prolong_resid(int mx, int my, int mcx, int mcy, const Stencil9<double>& st, const T* xp, const T* xc, const T* b,
+                      T* x, T* xm, T* r, T* d, double c0, cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
+  const Stencil9<T> a = scaled<T>(st, -1.0);
+  const int by = rows_for(mx, my, nb, kBX, 8, 4);
+  FD_LAUNCH_TILED(k_fd_prolong_resid, a, by, 4, 8, grid_of(mx, my, nb, by), dim3(kBX, by), mx, my, mcx, mcy, a, xp, xc, b, x, xm, r, d,
+            (T)(c0 / st.c[4]), ldf, ldc);
 }
 
 template <typename T>
@@ -578,6 +745,11 @@ void fd_adj_mid(int mx, int my, const Stencil9<double>& st, const double* rb, do
                             int, int64_t);                                                                       \
   template void fd_resid_restrict<T>(int, int, int, int, const Stencil9<double>&, const T*, const T*, T*,        \
                                      cudaStream_t, int, int64_t, int64_t);                                       \
+  template void fd_smooth_restrict<T>(int, int, int, int, const Stencil9<double>&, const T*, T*, T*, int,        \
+                                      double, double, double, double, double, cudaStream_t, int, int64_t,        \
+                                      int64_t);                                                                  \
+  template void fd_prolong_resid<T>(int, int, int, int, const Stencil9<double>&, const T*, const T*, const T*,   \
+                                    T*, T*, T*, T*, double, cudaStream_t, int, int64_t, int64_t);                \
   template void fd_restrict<T>(int, int, int, int, int, const T*, T*, cudaStream_t, int, int64_t, int64_t);      \
   template void fd_prolong<T>(int, int, int, int, int, const T*, T*, int, cudaStream_t, int, int64_t, int64_t);
 

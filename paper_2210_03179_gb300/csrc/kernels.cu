@@ -35,8 +35,8 @@ constexpr int kVecThreads = 256;
 }  // namespace
 
 // ===========================================================================
-// SEM element operator, one thread per point: orders 1 and 3 (line passes in sem_axl.cu and
-// sem_ax8.cu for the others; order 3 has k_sem_ax4 below as well, autotuned)
+// SEM element operator, one thread per point: orders 1 and 3, and order 6 on a few elements (line
+// passes in sem_axl.cu and sem_ax8.cu otherwise; order 3 has k_sem_ax4 below as well, autotuned)
 // ===========================================================================
 template <int Q>
 struct SemShape {
@@ -284,6 +284,7 @@ void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const
   switch (Q) {
     case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); break;
     case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); break;
     default: break;
   }
 }

@@ -72,18 +72,18 @@ struct Coef<double, Q> : Arith<double> {
   }
 };
 
-template <typename T, int Q>
+// EB elements per block.
+template <typename T, int Q, int EB_>
 struct AxL {
   static constexpr bool F = sizeof(T) == 4;
-  static constexpr int QQ = Q * Q, NP = Q * Q * Q;
+  static constexpr int QQ = Q * Q, NP = Q * Q * Q, EB = EB_;
   // FP32 reads the factors where they are used, with small blocks and many of them per SM; at order 6
   // holding them in registers was faster (87.2 against 91.3 us on 33^3 elements)
   static constexpr bool GREG = F && (Q == 7 || Q == 3);
-  // elements per block: FP64 nearly whole warps (it pays for every idle lane of its last warp)
-  static constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : F ? 1 : Q == 9 ? 3 : 5;
-  // blocks per SM to fit registers for
-  static constexpr int MINB = F ? (Q == 10 ? 9 : Q == 9 ? 10 : Q == 6 ? 4 : Q == 5 ? 8 : 1) : (Q == 9 ? 2 : 1);
   static constexpr int THREADS = (EB * QQ + 31) / 32 * 32;
+  // blocks per SM to fit registers for
+  static constexpr int MINB = EB == 1 && !(F && Q >= 9) ? 1
+                              : F ? (Q == 10 ? 9 : Q == 9 ? 10 : Q == 6 ? 4 : Q == 5 ? 8 : 1) : (Q == 9 ? 2 : 1);
   static constexpr int R = F ? (Q == 3 ? 4 : Q == 5 ? 6 : Q == 6 ? 9 : Q == 7 ? 8 : Q) : (Q == 6 ? 9 : Q);
   static constexpr int P = F ? (Q == 3 ? 35 : Q == 5 ? 37 : Q == 6 ? 70 : Q == 7 ? 71 : Q == 9 ? 81 : 101)
                              : (Q == 3 ? 19 : Q == 5 ? 25 : Q == 6 ? 54 : Q == 7 ? 55 : Q == 9 ? 89 : 106);
@@ -134,11 +134,11 @@ __device__ __forceinline__ void line(const Coef<T, Q>& c, const T (&u)[Q], T (&o
   }
 }
 
-template <typename T, int Q, bool IMPLICIT>
-__global__ void __launch_bounds__(AxL<T, Q>::THREADS, AxL<T, Q>::MINB)
+template <typename T, int Q, int EB, bool IMPLICIT>
+__global__ void __launch_bounds__(AxL<T, Q, EB>::THREADS, AxL<T, Q, EB>::MINB)
 k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __restrict__ G,
           const T* __restrict__ u, T* __restrict__ y, int64_t ld, uint32_t neg) {
-  using C = AxL<T, Q>;
+  using C = AxL<T, Q, EB>;
   constexpr int R = C::R, P = C::P, QQ = C::QQ, NP = C::NP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) typename Coef<T, Q>::Shared sCoef;
@@ -250,19 +250,47 @@ k_sem_axl(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   }
 }
 
+template <typename T, int Q, int EB>
+void launch_eb(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
+               int nb, int64_t ld, uint32_t neg) {
+  using C = AxL<T, Q, EB>;
+  static bool configured = false;
+  if (!configured) {
+    cudaFuncSetAttribute(k_sem_axl<T, Q, EB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    cudaFuncSetAttribute(k_sem_axl<T, Q, EB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    configured = true;
+  }
+  const dim3 blocks((unsigned)((E + EB - 1) / EB), nb);
+  if (lat) launch_dep(k_sem_axl<T, Q, EB, true>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, *lat, G, u, y, ld, neg);
+  else launch_dep(k_sem_axl<T, Q, EB, false>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, Lattice{}, G, u, y, ld, neg);
+}
+
+// Elements per block: the number that fills whole warps best (FP64 issue is paid for every lane of a
+// warp), or one where that leaves SMs idle: the busiest SM then has fewer warps to issue for.  36
+// elements of order 9 in FP64: 72.1 us in blocks of five, 21.6 in blocks of one (24.6 with a thread
+// per point).
 template <typename T, int Q>
 void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s, int nb,
             int64_t ld, uint32_t neg) {
-  using C = AxL<T, Q>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_axl<T, Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    cudaFuncSetAttribute(k_sem_axl<T, Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    configured = true;
+  constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : sizeof(T) == 4 ? 1 : Q == 9 ? 3 : 5;
+  constexpr int SMALL = Q == 3 ? 3 : 1;
+  if constexpr (EB > SMALL) {
+    static int sms = 0;
+    if (sms == 0) {
+      int dev = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    }
+    auto warps = [&](int eb, int threads) {   // of the busiest SM
+      const int64_t blocks = (E + eb - 1) / eb * nb;
+      return (blocks + sms - 1) / sms * (threads / 32);
+    };
+    if (warps(SMALL, AxL<T, Q, SMALL>::THREADS) < warps(EB, AxL<T, Q, EB>::THREADS)) {
+      launch_eb<T, Q, SMALL>(E, gid, lat, G, u, y, s, nb, ld, neg);
+      return;
+    }
   }
-  const dim3 blocks((unsigned)((E + C::EB - 1) / C::EB), nb);
-  if (lat) launch_dep(k_sem_axl<T, Q, true>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, *lat, G, u, y, ld, neg);
-  else launch_dep(k_sem_axl<T, Q, false>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, Lattice{}, G, u, y, ld, neg);
+  launch_eb<T, Q, EB>(E, gid, lat, G, u, y, s, nb, ld, neg);
 }
 
 template <typename T>
@@ -283,6 +311,21 @@ void fill(const double* S, int Q, LineTab<T>& t) {   // S: symmetrised D, [Q][Q]
 }
 
 }  // namespace
+
+// FP64 order 6 on at most one element per SM: a thread per point has the shorter serial chains (36
+// elements 11.4 against 13.8 us; on 448 elements 21.7 against 17.1).
+template <typename T>
+bool sem_axl_chosen(int Q, int64_t elements) {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  return sem_axl_supported(Q) && !(sizeof(T) == 8 && Q == 7 && elements <= sms);
+}
+template bool sem_axl_chosen<float>(int, int64_t);
+template bool sem_axl_chosen<double>(int, int64_t);
 
 bool sem_axl_supported(int Q) { return Q == 3 || (Q >= 5 && Q <= 10 && Q != 8); }
 
