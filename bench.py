@@ -849,7 +849,7 @@ def main():
     roofline = {"bound": "hbm",
                 "kernel": ("fine FP32 Chebyshev step, fused: k_sem_smooth8 (one launch per smoother application)"
                            if fused32 else
-                           "fine FP32 Chebyshev step: k_sem_ax8p (element Ax + gather-scatter) + k_cheb4_step"),
+                           "fine FP32 Chebyshev step: k_sem_ax8p (element Ax + gather-scatter) + k_smooth_step"),
                 "achieved": achieved, "peak": hbm if hbm else 6800.0, "unit": "GB/s",
                 "frac": achieved / (hbm if hbm else 6800.0),
                 "peak_source": "of measured (MEASURED_PEAKS.json hbm_gbs)" if hbm else "of fallback",

@@ -584,12 +584,13 @@ void set_coarse_shape(chebmg_ctx* c, int rpt_min) {
   c->coarse_rows_per_block = rb;
 }
 
-// Block sizes the lattice form can run with here, smallest first.
+// Block sizes of the lattice form worth timing here: the two smallest that can run (at every size
+// measured one of them was the fastest; each costs a set of timed solves at setup).
 std::vector<int> coarse_lat_blocks(const chebmg_ctx* c) {
   std::vector<int> v;
   if (c->lat_val && c->cred)
     for (int b : {64, 128, 256, 512, 1024})
-      if (coarse_lat_fits(c->L.back().n, c->cc_nx, b)) v.push_back(b);
+      if (v.size() < 2 && coarse_lat_fits(c->L.back().n, c->cc_nx, b)) v.push_back(b);
   return v;
 }
 
@@ -1360,6 +1361,11 @@ void check_dtype(chebmg_ctx* c, int dtype) {
   if (dtype == CHEBMG_F32 && c->fp32) return;
   throw Error(CHEBMG_EINVAL, "dtype not available in this context");
 }
+
+// Transfer calls on levels below this size launch ordinarily: there the host's launch calls bound them, and
+// a memset and an ordinary launch are the cheaper pair (144 elements of order 7: 14.1 against 14.6 us for a
+// restriction and an interpolation; 26,880 elements: 57.2 against 50.0 us as a chain).
+constexpr int64_t kChainMinN = 100000;
 
 void enter(chebmg_ctx* c) {
   if (!c) throw Error(CHEBMG_EINVAL, "ctx is NULL");
@@ -2964,8 +2970,7 @@ int chebmg_smooth(chebmg_ctx* c, int level, int dtype, const void* b, void* x, i
 int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* rc) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1, c->s);
-    level_checked(c, level);
+    const PdlScope pdl_(c->nb == 1 && level_checked(c, level).n >= kChainMinN, c->s);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
     if (!rf || !rc) throw Error(CHEBMG_EINVAL, "NULL vector");
@@ -2978,8 +2983,7 @@ int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* r
 int chebmg_prolong(chebmg_ctx* c, int level, int dtype, const void* zc, void* zf, int accumulate) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1, c->s);
-    level_checked(c, level);
+    const PdlScope pdl_(c->nb == 1 && level_checked(c, level).n >= kChainMinN, c->s);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
     if (!zc || !zf) throw Error(CHEBMG_EINVAL, "NULL vector");
