@@ -35,8 +35,8 @@ constexpr int kVecThreads = 256;
 }  // namespace
 
 // ===========================================================================
-// SEM element operator, one thread per point: orders 1 and 3, and order 6 on a few elements (line
-// passes in sem_axl.cu and sem_ax8.cu otherwise; order 3 has k_sem_ax4 below as well, autotuned)
+// SEM element operator, one thread per point: orders 1 and 3, and in FP64 the orders of the line passes
+// (sem_axl.cu) on few elements; order 7 is in sem_ax8.cu, order 3 has k_sem_ax4 below as well, autotuned
 // ===========================================================================
 template <int Q>
 struct SemShape {
@@ -284,8 +284,14 @@ void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const
   switch (Q) {
     case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); break;
     case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    default: break;
+    default:
+      if constexpr (sizeof(T) == 8) {   // FP64 on few elements (sem_axl_chosen)
+        if (Q == 5) launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg);
+        else if (Q == 6) launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg);
+        else if (Q == 7) launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg);
+        else if (Q == 9) launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg);
+        else if (Q == 10) launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg);
+      }
   }
 }
 

@@ -266,9 +266,8 @@ void launch_eb(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, c
 }
 
 // Elements per block: the number that fills whole warps best (FP64 issue is paid for every lane of a
-// warp), or one where that leaves SMs idle: the busiest SM then has fewer warps to issue for.  36
-// elements of order 9 in FP64: 72.1 us in blocks of five, 21.6 in blocks of one (24.6 with a thread
-// per point).
+// warp), or one where that leaves SMs idle: the busiest SM then has fewer warps to issue for (36
+// elements of order 9 in FP64: 72.1 us in blocks of five, 21.6 in blocks of one).
 template <typename T, int Q>
 void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s, int nb,
             int64_t ld, uint32_t neg) {
@@ -312,8 +311,12 @@ void fill(const double* S, int Q, LineTab<T>& t) {   // S: symmetrised D, [Q][Q]
 
 }  // namespace
 
-// FP64 order 6 on at most one element per SM: a thread per point has the shorter serial chains (36
-// elements 11.4 against 13.8 us; on 448 elements 21.7 against 17.1).
+// FP64 on few elements: a thread per point has the shorter serial chains, and the line passes' fewer
+// operations count only once every SM has warps enough to keep FP64 issue busy.  Four products of a
+// smoother, thread per point against line passes: order 4 on 512 elements 41.5 / 47.3 us, on 640 61.2 /
+// 47.3; order 5 on 294 39.4 / 57.4, on 512 60.0 / 80.0, on 640 82.7 / 82.5; order 6 on 294 55.8 / 65.6, on
+// 448 76.3 / 79.5, on 640 114.8 / 98.2; order 8 on 150 68.2 / 85.6, on 180 114.2 / 105.0; order 9 on 150
+// 91.7 / 97.9, on 180 170.0 / 155.9.  Order 2: even at every size.
 template <typename T>
 bool sem_axl_chosen(int Q, int64_t elements) {
   static int sms = 0;
@@ -322,7 +325,8 @@ bool sem_axl_chosen(int Q, int64_t elements) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   }
-  return sem_axl_supported(Q) && !(sizeof(T) == 8 && Q == 7 && elements <= sms);
+  const int64_t few = sizeof(T) == 4 || Q == 3 ? 0 : Q >= 9 ? 1 : 4;   // elements per SM
+  return sem_axl_supported(Q) && elements > few * sms;
 }
 template bool sem_axl_chosen<float>(int, int64_t);
 template bool sem_axl_chosen<double>(int, int64_t);

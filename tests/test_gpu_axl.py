@@ -42,3 +42,24 @@ def test_operator(order, mesh, boxed):
         cm.chebmg_apply_A_batched(s.ctx, 0, dt, T(X, ty), Y)
         assert relerr(N(Y), ref) < TOL[dt]
     s.close()
+
+
+# FP64 takes the line passes above four elements per SM (one at orders 8 and 9) and a thread per point
+# up to there: both sides of the line on 152 SMs.
+@pytest.mark.parametrize("order,mesh", [(o, m) for o in (4, 5, 6) for m in ((19, 8, 4), (29, 7, 3))] +
+                         [(o, m) for o in (8, 9) for m in ((19, 4, 2), (17, 3, 3))])
+@pytest.mark.parametrize("boxed", [True, False])
+def test_operator_about_the_line(order, mesh, boxed):
+    v = W.sem_box_vertices(*mesh)
+    L = SemLevel(v, order)
+    kw = dict(orders=(order, 1), prec="fp64", lmax=[1.0])
+    if boxed:
+        s = cm.Solver("sem", verts=v, **kw)
+    else:
+        s = cm.Solver("sem_mesh", coords=L.coords.reshape(L.E, -1, 3), gid=L.gid.reshape(L.E, -1), n=L.n,
+                      dirichlet=L.dirichlet.copy(), **kw)
+    x = np.random.default_rng(order).uniform(-1, 1, L.n)
+    y = torch.full((L.n,), 3.0, dtype=torch.float64, device="cuda")
+    cm.chebmg_apply_A(s.ctx, 0, cm.CHEBMG_F64, T(x), y)
+    assert relerr(N(y), L.apply_A(x)) < TOL[cm.CHEBMG_F64]
+    s.close()
