@@ -277,14 +277,9 @@ int loads_of(int block, int nx) { return (3 * band_of(block, nx).bw + block - 1)
 }  // namespace
 
 bool coarse_lat_fits(int64_t n, int nx, int block) {
-  static int sms = -1, optin = 0;
-  if (sms < 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
-  return n < (int64_t)1 << 30 && (n + block - 1) / block <= sms && loads_of(block, nx) <= 8 &&
+  static PerDevice smem_max;
+  const int optin = smem_max([] { return device_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin); });
+  return n < (int64_t)1 << 30 && (n + block - 1) / block <= sm_count() && loads_of(block, nx) <= 8 &&
          lat_smem(block, nx) + 4096 <= (size_t)optin;
 }
 

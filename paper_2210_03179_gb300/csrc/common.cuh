@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "device.cuh"
 #include "setup_host.h"
 
 namespace chebmg {

@@ -568,13 +568,7 @@ dim3 grid_of(int mx, int my, int nb, int by = kBY) { return dim3((mx + kBX - 1) 
 // FP64 work that the busiest SM does in series.  A symmetric order-2 cycle, tall blocks alone -> this:
 // 63 x 63 40.7 -> 32.1 us, 127 x 127 54.5 -> 42.8, 511 x 511 (its coarse levels) 103.0 -> 90.5.
 int rows_for(int mx, int my, int nb, int bx, int many, int few) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
-  return (int64_t)((mx + bx - 1) / bx) * ((my + many - 1) / many) * nb < sms ? few : many;
+  return (int64_t)((mx + bx - 1) / bx) * ((my + many - 1) / many) * nb < sm_count() ? few : many;
 }
 
 }  // namespace

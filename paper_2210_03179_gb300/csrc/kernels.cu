@@ -1103,12 +1103,7 @@ static const void* coarse_kernel(int rpt) {
 }
 
 void coarse_pcg_shape(int64_t n, int rpt_min, int* grid, int* rows_per_block) {
-  static int sms = -1;
-  if (sms < 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
+  const int sms = sm_count() > 0 ? sm_count() : 1;
   const int64_t per_block_min = (n + sms - 1) / sms;
   int rpt = 1;
   while (rpt < rpt_min && rpt < kCoarseMaxRowsPerThread) rpt *= 2;

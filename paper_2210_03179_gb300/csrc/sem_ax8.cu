@@ -826,11 +826,8 @@ template <typename T, int EB, bool IM>
 static void launch_ax8(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
                        unsigned* err, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_ax8<T, EB, IM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes());
-    configured = true;
-  }
+  static PerDevice smem_set;
+  allow_smem(smem_set, (const void*)k_sem_ax8<T, EB, IM>, C::smem_bytes());
   const unsigned blocks = (unsigned)((E + EB - 1) / EB);
   launch_dep(k_sem_ax8<T, EB, IM>, dim3(blocks), dim3(64 * EB), C::smem_bytes(), s, E, gid, lat, G, u, y, err, neg);
 }
@@ -840,11 +837,8 @@ static void launch_ax8g(int64_t E, const uint32_t* gid, const Lattice& lat, cons
                         cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * 3 * C::STAGE;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_ax8g<T, EB, IM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
+  static PerDevice smem_set;
+  allow_smem(smem_set, (const void*)k_sem_ax8g<T, EB, IM>, smem);
   const unsigned blocks = (unsigned)((E + EB - 1) / EB);
   launch_dep(k_sem_ax8g<T, EB, IM>, dim3(blocks), dim3(64 * EB), smem, s, E, gid, lat, G, u, y, neg);
 }
@@ -854,15 +848,9 @@ static void launch_ax8p(int64_t E, const uint32_t* gid, const Lattice& lat, cons
                         unsigned* err, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * (NB * C::GELEM + 3 * C::STAGE);
-  static int grid = 0;
-  if (grid == 0) {
-    cudaFuncSetAttribute(k_sem_ax8p<T, EB, IM, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sem_ax8p<T, EB, IM, NB>, 64 * EB, smem);
-    grid = sms * (per_sm > 0 ? per_sm : 1);
-  }
+  static PerDevice smem_set, resident;
+  allow_smem(smem_set, (const void*)k_sem_ax8p<T, EB, IM, NB>, smem);
+  const int grid = resident_blocks(resident, (const void*)k_sem_ax8p<T, EB, IM, NB>, 64 * EB, smem);
   const int64_t nbatch = (E + EB - 1) / EB;
   const unsigned blocks = (unsigned)(nbatch < grid ? nbatch : grid);
   launch_dep(k_sem_ax8p<T, EB, IM, NB>, dim3(blocks), dim3(64 * EB), smem, s, E, gid, lat, G, u, y, err, neg);
@@ -872,12 +860,8 @@ template <typename T, int EB, bool IM>
 static void launch_ax8b(int64_t E, const uint32_t* gid, const Lattice& lat, const T* G, const T* u, T* y,
                         unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_ax8b<T, EB, IM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)C::smem_bytes());
-    configured = true;
-  }
+  static PerDevice smem_set;
+  allow_smem(smem_set, (const void*)k_sem_ax8b<T, EB, IM>, C::smem_bytes());
   if (rb < 1) rb = 1;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
   k_sem_ax8b<T, EB, IM><<<blocks, 64 * EB, C::smem_bytes(), s>>>(E, gid, lat, G, u, y, err, nb, ld, rb, neg);
@@ -889,11 +873,8 @@ static void launch_ax8b2(int64_t E, const uint32_t* gid, const Lattice& lat, con
                          unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * (C::GELEM + 6 * C::STAGE);
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_ax8b2<T, EB, IM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
+  static PerDevice smem_set;
+  allow_smem(smem_set, (const void*)k_sem_ax8b2<T, EB, IM>, smem);
   if (rb < 2) rb = 2;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
   k_sem_ax8b2<T, EB, IM><<<blocks, 64 * EB, smem, s>>>(E, gid, lat, G, u, y, err, nb, ld, rb, neg);
@@ -905,11 +886,8 @@ static void launch_ax8bg(int64_t E, const uint32_t* gid, const Lattice& lat, con
                          int64_t ld, int rb, cudaStream_t s, uint32_t neg) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * 3 * C::STAGE;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_ax8bg<T, EB, IM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
+  static PerDevice smem_set;
+  allow_smem(smem_set, (const void*)k_sem_ax8bg<T, EB, IM>, smem);
   if (rb < 1) rb = 1;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
   k_sem_ax8bg<T, EB, IM><<<blocks, 64 * EB, smem, s>>>(E, gid, lat, G, u, y, nb, ld, rb, neg);

@@ -188,11 +188,8 @@ size_t smem_x2(int eb) { return sizeof(f32x2) * (size_t)eb * (kGElem + 3 * kStag
 template <int EB, bool IM>
 void launch_x2(int64_t E, const uint32_t* gid, const Lattice& lat, const f32x2* G, const double* u, double* y,
                unsigned* err, int nb, int64_t ld, int rb, cudaStream_t s) {
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_ax8_x2<EB, IM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_x2(EB));
-    configured = true;
-  }
+  static PerDevice smem_set;
+  allow_smem(smem_set, (const void*)k_sem_ax8_x2<EB, IM>, smem_x2(EB));
   if (rb < 1) rb = 1;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), (unsigned)((nb + rb - 1) / rb));
   k_sem_ax8_x2<EB, IM><<<blocks, 64 * EB, smem_x2(EB), s>>>(E, gid, lat, G, u, y, err, nb, ld, rb);

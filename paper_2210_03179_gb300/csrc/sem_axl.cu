@@ -254,15 +254,15 @@ template <typename T, int Q, int EB>
 void launch_eb(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
                int nb, int64_t ld, uint32_t neg) {
   using C = AxL<T, Q, EB>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_sem_axl<T, Q, EB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    cudaFuncSetAttribute(k_sem_axl<T, Q, EB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    configured = true;
-  }
+  static PerDevice smem_lat, smem_map;
   const dim3 blocks((unsigned)((E + EB - 1) / EB), nb);
-  if (lat) launch_dep(k_sem_axl<T, Q, EB, true>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, *lat, G, u, y, ld, neg);
-  else launch_dep(k_sem_axl<T, Q, EB, false>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, Lattice{}, G, u, y, ld, neg);
+  if (lat) {
+    allow_smem(smem_lat, (const void*)k_sem_axl<T, Q, EB, true>, C::SMEM);
+    launch_dep(k_sem_axl<T, Q, EB, true>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, *lat, G, u, y, ld, neg);
+  } else {
+    allow_smem(smem_map, (const void*)k_sem_axl<T, Q, EB, false>, C::SMEM);
+    launch_dep(k_sem_axl<T, Q, EB, false>, blocks, dim3(C::THREADS), C::SMEM, s, E, gid, Lattice{}, G, u, y, ld, neg);
+  }
 }
 
 // Elements per block: the number that fills whole warps best (FP64 issue is paid for every lane of a
@@ -274,12 +274,7 @@ void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, cons
   constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : sizeof(T) == 4 ? 1 : Q == 9 ? 3 : 5;
   constexpr int SMALL = Q == 3 ? 3 : 1;
   if constexpr (EB > SMALL) {
-    static int sms = 0;
-    if (sms == 0) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
+    const int sms = sm_count() > 0 ? sm_count() : 1;
     auto warps = [&](int eb, int threads) {   // of the busiest SM
       const int64_t blocks = (E + eb - 1) / eb * nb;
       return (blocks + sms - 1) / sms * (threads / 32);
@@ -319,14 +314,8 @@ void fill(const double* S, int Q, LineTab<T>& t) {   // S: symmetrised D, [Q][Q]
 // 91.7 / 97.9, on 180 170.0 / 155.9.  Order 2: even at every size.
 template <typename T>
 bool sem_axl_chosen(int Q, int64_t elements) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  }
   const int64_t few = sizeof(T) == 4 || Q == 3 ? 0 : Q >= 9 ? 1 : 4;   // elements per SM
-  return sem_axl_supported(Q) && elements > few * sms;
+  return sem_axl_supported(Q) && elements > few * sm_count();
 }
 template bool sem_axl_chosen<float>(int, int64_t);
 template bool sem_axl_chosen<double>(int, int64_t);

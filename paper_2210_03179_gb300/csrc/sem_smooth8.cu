@@ -589,15 +589,9 @@ template <typename T, int EB>
 bool launch_fused(FusedSmooth& a, cudaStream_t s) {
   using C = Ax8<T, EB>;
   const size_t smem = sizeof(T) * (size_t)EB * (2 * C::GELEM + 3 * C::STAGE);
-  static int grid = 0;
-  if (grid == 0) {
-    cudaFuncSetAttribute(k_sem_smooth8<T, EB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sem_smooth8<T, EB>, 64 * EB + 32, smem);
-    grid = sms * (per_sm > 0 ? per_sm : 1);
-  }
+  static PerDevice smem_set, resident;
+  allow_smem(smem_set, (const void*)k_sem_smooth8<T, EB>, smem);
+  const int grid = resident_blocks(resident, (const void*)k_sem_smooth8<T, EB>, 64 * EB + 32, smem);
   cudaMemsetAsync(a.ctl, 0, sizeof(unsigned) * (size_t)fused_ctl_words(a.lat), s);
   const unsigned blocks = (unsigned)std::min<int64_t>(grid, std::max<int64_t>(a.total, 1));
   // cooperative: every block is resident, which the static schedule's waits rely on
