@@ -290,12 +290,12 @@ void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld, b
     else if (L.Q == 4 && L.ax4[dt] % 100 == 41)
       sem_ax4<T>(L.E, L.gid, L.ax4[dt] >= 100 ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]),
                  static_cast<const T*>(L.D[dt]), x, y, c->s, nb, ld, subtract);
-    else if (sem_axl_chosen<T>(L.Q, L.E * nb))
-      sem_axl<T>(L.Q, L.E, L.gid, L.boxed ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]), x, y, c->s, nb, ld,
-                 subtract);
-    else
-      sem_ax<T>(L.Q, L.E, L.gid, static_cast<const T*>(L.G[dt]), static_cast<const T*>(L.D[dt]), x, y, c->s, nb,
-                ld, subtract);
+    else if (!(sem_axl_chosen<T>(L.Q, L.E * nb)
+                   ? sem_axl<T>(L.Q, L.E, L.gid, L.boxed ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]), x, y,
+                                c->s, nb, ld, subtract)
+                   : sem_ax<T>(L.Q, L.E, L.gid, static_cast<const T*>(L.G[dt]), static_cast<const T*>(L.D[dt]), x, y,
+                               c->s, nb, ld, subtract)))
+      throw Error(CHEBMG_EINVAL, "no operator kernel for this order");
   } else {
     fd_apply<T>(L.mx, L.my, stencil(L), x, y, c->s, nb, ld);
   }

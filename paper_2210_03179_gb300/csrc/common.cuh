@@ -124,8 +124,10 @@ void zero_bytes(void* p, int64_t bytes, cudaStream_t s);
 // ---- SEM kernels (results accumulate into y: y += A u, or y -= A u when subtract is set) ----
 // Every operator, transfer and vector kernel also runs on a batch of nb right-hand sides:
 // vector b of the batch starts at offset b * ld (ld = 0 means n; per-node data shared).
+// sem_ax and sem_axl have kernels for some orders only and return false, having launched nothing, for
+// the others; sem_axl_chosen says which of the two an order takes here.
 template <typename T>
-void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
+bool sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
             cudaStream_t s, int nb = 1, int64_t ld = 0, bool subtract = false);
 template <typename T>
 void sem_restrict(int Qf, int Qc, int64_t E, const uint32_t* gidf, const uint32_t* gidc,
@@ -160,7 +162,7 @@ template <typename T>
 bool sem_axl_chosen(int Q, int64_t elements);   // else sem_ax
 cudaError_t sem_axl_set_D(int Q, const double* D);
 template <typename T>
-void sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
+bool sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
              int nb = 1, int64_t ld = 0, bool subtract = false);
 // The order-7 operator in FP64-class arithmetic on FP32 pairs (sem_ax8_x2.cu): G in that
 // format (sem_to_x2 converts an FP64 array of n values), u and y FP64; variant as sem_ax8's

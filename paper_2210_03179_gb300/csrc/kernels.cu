@@ -278,20 +278,24 @@ void sem_ax4(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, con
 }
 
 template <typename T>
-void sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
+bool sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const T* u, T* y,
             cudaStream_t s, int nb, int64_t ld, bool subtract) {
   const uint32_t neg = subtract ? kSignBit : 0u;
   switch (Q) {
-    case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); break;
-    case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); break;
+    case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+    case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
     default:
       if constexpr (sizeof(T) == 8) {   // FP64 on few elements (sem_axl_chosen)
-        if (Q == 5) launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg);
-        else if (Q == 6) launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg);
-        else if (Q == 7) launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg);
-        else if (Q == 9) launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg);
-        else if (Q == 10) launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg);
+        switch (Q) {
+          case 5: launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+          case 6: launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+          case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+          case 9: launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+          case 10: launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+          default: break;
+        }
       }
+      return false;
   }
 }
 
@@ -1196,7 +1200,7 @@ void scale(int64_t n, double a, const double* x, double* y, cudaStream_t s) {
 #define CHEBMG_INST(T)                                                                                \
   template void sem_ax4<T>(int64_t, const uint32_t*, const Lattice*, const T*, const T*, const T*, T*,           \
                            cudaStream_t, int, int64_t, bool);                                              \
-  template void sem_ax<T>(int, int64_t, const uint32_t*, const T*, const T*, const T*, T*, cudaStream_t, int,  \
+  template bool sem_ax<T>(int, int64_t, const uint32_t*, const T*, const T*, const T*, T*, cudaStream_t, int,  \
                           int64_t, bool);                                                             \
   template void sem_restrict<T>(int, int, int64_t, const uint32_t*, const uint32_t*, const T*, const T*,  \
                                 T*, cudaStream_t, int, int64_t, int64_t);                              \

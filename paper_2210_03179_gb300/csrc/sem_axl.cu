@@ -336,22 +336,22 @@ cudaError_t sem_axl_set_D(int Q, const double* D) {
 }
 
 template <typename T>
-void sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
+bool sem_axl(int Q, int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s,
              int nb, int64_t ld, bool subtract) {
   const uint32_t neg = subtract ? kSignBit : 0u;
   switch (Q) {
-    case 3: launch<T, 3>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
-    case 5: launch<T, 5>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
-    case 6: launch<T, 6>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
-    case 7: launch<T, 7>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
-    case 9: launch<T, 9>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
-    case 10: launch<T, 10>(E, gid, lat, G, u, y, s, nb, ld, neg); break;
-    default: break;
+    case 3: launch<T, 3>(E, gid, lat, G, u, y, s, nb, ld, neg); return true;
+    case 5: launch<T, 5>(E, gid, lat, G, u, y, s, nb, ld, neg); return true;
+    case 6: launch<T, 6>(E, gid, lat, G, u, y, s, nb, ld, neg); return true;
+    case 7: launch<T, 7>(E, gid, lat, G, u, y, s, nb, ld, neg); return true;
+    case 9: launch<T, 9>(E, gid, lat, G, u, y, s, nb, ld, neg); return true;
+    case 10: launch<T, 10>(E, gid, lat, G, u, y, s, nb, ld, neg); return true;
+    default: return false;
   }
 }
-template void sem_axl<float>(int, int64_t, const uint32_t*, const Lattice*, const float*, const float*, float*,
+template bool sem_axl<float>(int, int64_t, const uint32_t*, const Lattice*, const float*, const float*, float*,
                              cudaStream_t, int, int64_t, bool);
-template void sem_axl<double>(int, int64_t, const uint32_t*, const Lattice*, const double*, const double*, double*,
+template bool sem_axl<double>(int, int64_t, const uint32_t*, const Lattice*, const double*, const double*, double*,
                               cudaStream_t, int, int64_t, bool);
 
 }  // namespace chebmg
