@@ -532,6 +532,7 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
   const Coef8<T> cf(sCoef);
+  if constexpr (Coef8<T>::SHARED > 1) __syncthreads();   // the first line comes before the loop's first barrier
   T* sU = reinterpret_cast<T*>(smem_raw);
   T* sR = sU + EB * C::STAGE;
   T* sS = sR + EB * C::STAGE;
