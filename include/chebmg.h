@@ -163,6 +163,11 @@ enum { CHEBMG_COARSE_HOST = 0, CHEBMG_COARSE_GRID = 1, CHEBMG_COARSE_CLUSTER = 2
 int chebmg_coarse_shape(const chebmg_ctx* ctx, int* kernel, int* blocks, int* rows_per_block);
 /* Overrides the coarse kernel (GRID or CLUSTER); EINVAL where it does not apply. */
 int chebmg_set_coarse_kernel(chebmg_ctx* ctx, int kernel);
+/* Form of the grid-wide kernel: rows per block of the one with the vector in shared memory (box
+ * lattices; 64, 128, 256, 512 or 1024), 0 for the general one.  The setter selects GRID; EINVAL where
+ * that form or block size cannot run. */
+int chebmg_coarse_lattice(const chebmg_ctx* ctx, int* rows_per_block);
+int chebmg_set_coarse_lattice(chebmg_ctx* ctx, int rows_per_block);
 
 /* Arithmetic of the outer Krylov product q = A p on the finest level (chebmg_pcg_solve;
  * the operator of Sec. 1, Eq. 1.3):

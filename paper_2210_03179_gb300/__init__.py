@@ -98,6 +98,8 @@ _SIGNATURES = {
     "chebmg_coarse_info": (c_int, [c_void_p, POINTER(c_int), POINTER(c_double)]),
     "chebmg_coarse_shape": (c_int, [c_void_p, POINTER(c_int), POINTER(c_int), POINTER(c_int)]),
     "chebmg_set_coarse_kernel": (c_int, [c_void_p, c_int]),
+    "chebmg_coarse_lattice": (c_int, [c_void_p, POINTER(c_int)]),
+    "chebmg_set_coarse_lattice": (c_int, [c_void_p, c_int]),
     "chebmg_set_outer_operator": (c_int, [c_void_p, c_int]),
     "chebmg_apply_outer": (c_int, [c_void_p, c_void_p, c_void_p]),
     "chebmg_set_coarse_degree": (c_int, [c_void_p, c_int]),
@@ -294,6 +296,17 @@ def chebmg_coarse_shape(ctx):
 
 def chebmg_set_coarse_kernel(ctx, kernel: int) -> None:
     _check(lib().chebmg_set_coarse_kernel(ctx, int(kernel)), "chebmg_set_coarse_kernel")
+
+
+def chebmg_coarse_lattice(ctx) -> int:
+    """Rows per block of the coarse CG's shared-memory lattice form, 0 if the general form runs."""
+    r = c_int()
+    _check(lib().chebmg_coarse_lattice(ctx, byref(r)), "chebmg_coarse_lattice")
+    return r.value
+
+
+def chebmg_set_coarse_lattice(ctx, rows_per_block: int) -> None:
+    _check(lib().chebmg_set_coarse_lattice(ctx, int(rows_per_block)), "chebmg_set_coarse_lattice")
 
 
 def chebmg_set_outer_operator(ctx, kind: int) -> None:

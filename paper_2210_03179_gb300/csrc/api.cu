@@ -584,12 +584,13 @@ void set_coarse_shape(chebmg_ctx* c, int rpt_min) {
   c->coarse_rows_per_block = rb;
 }
 
+constexpr int kCoarseLatBlocks[] = {64, 128, 256, 512, 1024};
 // Block sizes of the lattice form worth timing here: the two smallest that can run (at every size
 // measured one of them was the fastest; each costs a set of timed solves at setup).
 std::vector<int> coarse_lat_blocks(const chebmg_ctx* c) {
   std::vector<int> v;
   if (c->lat_val && c->cred)
-    for (int b : {64, 128, 256, 512, 1024})
+    for (int b : kCoarseLatBlocks)
       if (v.size() < 2 && coarse_lat_fits(c->L.back().n, c->cc_nx, b)) v.push_back(b);
   return v;
 }
@@ -2707,6 +2708,29 @@ int chebmg_set_coarse_kernel(chebmg_ctx* c, int kernel) {
     } else {
       throw Error(CHEBMG_EINVAL, "bad coarse kernel");
     }
+    drop_graphs(c);
+    return CHEBMG_OK;
+  });
+}
+
+int chebmg_coarse_lattice(const chebmg_ctx* c, int* rows_per_block) {
+  if (!c || !rows_per_block) return CHEBMG_EINVAL;
+  *rows_per_block = c->coop_ok && c->lat_val ? c->coarse_lat : 0;
+  return CHEBMG_OK;
+}
+
+int chebmg_set_coarse_lattice(chebmg_ctx* c, int rows_per_block) {
+  return guard([&]() -> int {
+    enter(c);
+    if (!c->coop_ok || !c->ell_col) throw Error(CHEBMG_EINVAL, "no grid-wide persistent coarse kernel in this context");
+    if (rows_per_block != 0) {
+      bool size = false;
+      for (int b : kCoarseLatBlocks) size |= b == rows_per_block;
+      if (!size || !c->lat_val || !c->cred || !coarse_lat_fits(c->L.back().n, c->cc_nx, rows_per_block))
+        throw Error(CHEBMG_EINVAL, "the lattice coarse kernel cannot run with this block size");
+    }
+    c->coarse_lat = rows_per_block;
+    c->coarse_kernel = 0;
     drop_graphs(c);
     return CHEBMG_OK;
   });
