@@ -585,13 +585,25 @@ void set_coarse_shape(chebmg_ctx* c, int rpt_min) {
 }
 
 constexpr int kCoarseLatBlocks[] = {64, 128, 256, 512, 1024};
-// Block sizes of the lattice form worth timing here: the two smallest that can run (at every size
-// measured one of them was the fastest; each costs a set of timed solves at setup).
+// Block sizes of the lattice form worth timing here: the two smallest that can run and are no larger than
+// the general form's.  With larger ones fewer SMs work on the same products: on long boxes, whose bands
+// only blocks of 512 rows hold in few enough loads, the general form in blocks of 256 is faster.
+// Measured, us a coarse solve with the FP32 preconditioner, lattice blocks of 64 / 128 / 256 / 512 / 1024
+// rows and the general form:
+//   8^3        161 / 168 / 196 / 342 / 531   279      32^3      - / - / 413 / 723 / 1068   563
+//   16^3       244 / 240 / 275 / 443 / 694   373      36^3      - / - / - / 793 / 1156     982
+//   24^3         - / 317 / 341 / 601 / 900   465      150x30x8  - / - / - / 587 / 773      627
+//   200x4x4      - / - / 207 / 354 / 515     243      42^3      - / - / - / - / 1320       2512
+//   300x10x3     - / - / - / 372 / 527       243      600x6x6   - / - / - / - / 698        328
+// (the general form's blocks have 512 rows at 36^3 and 150x30x8, 1024 at 42^3, 256 at the others).  The
+// FP64 preconditioner has the same order everywhere, but for 12^3 and 20^3, where 128 rows beat 64 by 6%.
 std::vector<int> coarse_lat_blocks(const chebmg_ctx* c) {
   std::vector<int> v;
+  int grid = 0, general = 0;
+  coarse_pcg_shape(c->L.back().n, 1, &grid, &general);
   if (c->lat_val && c->cred)
     for (int b : kCoarseLatBlocks)
-      if (v.size() < 2 && coarse_lat_fits(c->L.back().n, c->cc_nx, b)) v.push_back(b);
+      if (v.size() < 2 && b <= general && coarse_lat_fits(c->L.back().n, c->cc_nx, b)) v.push_back(b);
   return v;
 }
 
@@ -1167,8 +1179,8 @@ void autotune_coarse_degree(chebmg_ctx* c) {
       }
     }
   };
-  // grid-wide: the lattice form where it runs (it beat the general one at every size measured), else
-  // the general one at several rows per thread
+  // grid-wide: the lattice form where it has a block size worth timing, else the general one at several
+  // rows per thread
   c->coarse_kernel = 0;
   const std::vector<int> lat = coarse_lat_blocks(c);
   for (int blk : lat) {
