@@ -32,14 +32,19 @@ struct Ax8 {
 
 // The line coefficients as a kernel uses them: FP32 constant-bank operands; FP64 in shared memory
 // (an FP64 FMA issues faster with register operands than with constant ones, see Fp64Unit), rows
-// loaded 16 bytes at a time where they are used.  Every thread of the block calls the constructor,
-// and a block barrier separates it from the first line8.
+// loaded 16 bytes at a time where they are used.  Every thread of the block (64 at least) calls the
+// constructor, which only fetches, and then stage(); a block barrier separates stage() from the first
+// line8.  A kernel that gathers first stages after it, so that the fetch is in flight with the gather:
+// on 8 to 64 elements a product took 0.1 to 1.0 us less (order-4 smoother from an iterate on 64
+// elements, best variant 68.3 -> 67.3 us, one element per block with bulk copies 72.6 -> 68.9), on 32^3
+// nothing changed.
 template <typename T>
 struct Coef8;
 template <>
 struct Coef8<float> : Arith<float> {
   static constexpr int SHARED = 1;
-  __device__ __forceinline__ explicit Coef8(float*) {}
+  __device__ __forceinline__ Coef8() {}
+  __device__ __forceinline__ void stage(float*) {}
   template <int W>
   __device__ __forceinline__ void row(int i, float (&v)[4]) const {
 #pragma unroll
@@ -50,8 +55,11 @@ template <>
 struct Coef8<double> : Arith<double> {
   static constexpr int SHARED = 64;
   const double* t;
-  __device__ __forceinline__ explicit Coef8(double* sh) : t(sh) {
-    for (int q = threadIdx.x; q < 64; q += blockDim.x) sh[q] = __ldg(&g_eo_d[q]);
+  double mine;
+  __device__ __forceinline__ Coef8() : t(nullptr), mine(threadIdx.x < 64 ? __ldg(&g_eo_d[threadIdx.x]) : 0.0) {}
+  __device__ __forceinline__ void stage(double* sh) {
+    t = sh;
+    if (threadIdx.x < 64) sh[threadIdx.x] = mine;
   }
   template <int W>
   __device__ __forceinline__ void row(int i, double (&v)[4]) const {

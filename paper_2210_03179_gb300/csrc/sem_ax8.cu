@@ -36,7 +36,7 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
   constexpr int EB = C::EB, R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
   __shared__ __align__(8) uint64_t bar;
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sU = sG + EB * C::GELEM;
@@ -76,9 +76,11 @@ k_sem_ax8(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __r
     col[k] = (g[k] & kGidDirichlet) ? T(0) : u[g[k] & kGidMask];
     su[k * P + b * R + a] = col[k];
   }
+  cf.stage(sCoef);
   T ut[8];
-  line8<T, 0>(cf, col, ut);
+  if constexpr (Coef8<T>::SHARED == 1) line8<T, 0>(cf, col, ut);
   __syncthreads();
+  if constexpr (Coef8<T>::SHARED > 1) line8<T, 0>(cf, col, ut);
   {
     T v[8], o[8];
     // r: thread (j = a, k = b) owns the row along i
@@ -160,7 +162,7 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
   T* sU = reinterpret_cast<T*>(smem_raw);
   T* sR = sU + EB_ * C::STAGE;
   T* sS = sR + EB_ * C::STAGE;
@@ -180,6 +182,7 @@ k_sem_ax8g(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
     col[k] = (g[k] & kGidDirichlet) ? T(0) : u[g[k] & kGidMask];
     su[k * P + b * R + a] = col[k];
   }
+  cf.stage(sCoef);
   __syncthreads();
   T ut[8];
   line8<T, 0>(cf, col, ut);
@@ -252,7 +255,8 @@ k_sem_ax8p(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
+  cf.stage(sCoef);
   __shared__ __align__(8) uint64_t bar[2];
   T* sG = reinterpret_cast<T*>(smem_raw);                 // [NB][EB * GELEM]
   T* sU = sG + NB * EB * C::GELEM;
@@ -398,7 +402,8 @@ k_sem_ax8b(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* __
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
+  cf.stage(sCoef);
   __shared__ __align__(8) uint64_t bar;
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sU = sG + EB * C::GELEM;
@@ -531,7 +536,8 @@ k_sem_ax8bg(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
+  cf.stage(sCoef);
   if constexpr (Coef8<T>::SHARED > 1) __syncthreads();   // the first line comes before the loop's first barrier
   T* sU = reinterpret_cast<T*>(smem_raw);
   T* sR = sU + EB * C::STAGE;
@@ -637,7 +643,8 @@ k_sem_ax8b2(int64_t E, const uint32_t* __restrict__ gid, Lattice lat, const T* _
   constexpr int R = C::R, P = C::P;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
+  cf.stage(sCoef);
   __shared__ __align__(8) uint64_t bar;
   T* sG = reinterpret_cast<T*>(smem_raw);
   T* sStage = sG + EB * C::GELEM;   // [2 right-hand sides][3 stages][EB][STAGE]

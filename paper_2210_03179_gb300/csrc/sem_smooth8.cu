@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(64 * EB + 32, 3) k_sem_smooth8(const __grid_co
   constexpr int R = C::R, P = C::P, NC = 64 * EB;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) T sCoef[Coef8<T>::SHARED];
-  const Coef8<T> cf(sCoef);
+  Coef8<T> cf;
+  cf.stage(sCoef);
   __shared__ __align__(8) uint64_t ready[2], done[2];
   __shared__ Item sh_item[2];
   T* sG = reinterpret_cast<T*>(smem_raw);   // [2][EB * GELEM], buffer = slot
