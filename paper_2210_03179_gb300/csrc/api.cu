@@ -1375,10 +1375,26 @@ void check_dtype(chebmg_ctx* c, int dtype) {
   throw Error(CHEBMG_EINVAL, "dtype not available in this context");
 }
 
-// Transfer calls on levels below this size launch ordinarily: there the host's launch calls bound them, and
-// a memset and an ordinary launch are the cheaper pair (144 elements of order 7: 14.1 against 14.6 us for a
-// restriction and an interpolation; 26,880 elements: 57.2 against 50.0 us as a chain).
-constexpr int64_t kChainMinN = 100000;
+// Whether a single operator or restriction call runs as a dependent chain (zeroing kernel, then the
+// kernel) or as a memset and an ordinary launch.  A chain costs the host about 0.6 us more a call; it hides
+// one to three us of a kernel's start.  In a loop of calls it therefore pays where the kernels, not the
+// host's launches, set the pace.  Measured, us a call, ordinary / chain, by nodes n of the finer level:
+//   operator     FP32 order 2: n = 729 5.9 / 6.2, 1,331 6.6 / 6.5; order 3: 1,000 5.8 / 6.5, 2,197 6.6 / 6.0;
+//                order 7: 3,375 7.2 / 6.5.  FD: 961 6.1 / 6.6, 3,969 6.9 / 6.5.  FP64 SEM: 125 8.3 / 6.3,
+//                343 9.9 / 6.6
+//   restriction  FP32 7 -> 3: 24,389 6.8 / 7.4, 46,656 7.5 / 7.4; 3 -> 1: 15,625 6.4 / 6.9, 29,791 7.6 / 7.4
+//                FP64 7 -> 3: 3,375 6.4 / 7.4, 10,648 9.1 / 7.4; 3 -> 1: 6,859 6.8 / 7.5, 15,625 7.5 / 7.4
+// Interpolations and FD restrictions are one kernel without a zeroing, and a chain was never slower there
+// (FP64 5 -> 3 at 68,921 nodes 8.2 / 5.8); nor in a smoother, whose kernels are all its own.
+constexpr int64_t kChainOperatorN = 1200, kChainRestrictN32 = 25000, kChainRestrictN64 = 5000,
+                  kChainRestrictLowN64 = 12000;   // orders up to 3: less FP64 work in an element
+bool chain_operator(const Level& L, int dtype) {
+  return (L.type == TYPE_SEM && dtype == CHEBMG_F64) || L.n >= kChainOperatorN;
+}
+bool chain_restrict(const Level& L, int dtype) {
+  return L.type == TYPE_FD ||
+         L.n >= (dtype != CHEBMG_F64 ? kChainRestrictN32 : L.Q <= 4 ? kChainRestrictLowN64 : kChainRestrictN64);
+}
 
 void enter(chebmg_ctx* c) {
   if (!c) throw Error(CHEBMG_EINVAL, "ctx is NULL");
@@ -2956,8 +2972,8 @@ int chebmg_apply_outer(chebmg_ctx* c, const double* x, double* y) {
 int chebmg_apply_A(chebmg_ctx* c, int level, int dtype, const void* x, void* y) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1, c->s);
     Level& L = level_checked(c, level);
+    const PdlScope pdl_(c->nb == 1 && chain_operator(L, dtype), c->s);
     check_dtype(c, dtype);
     if (!x || !y) throw Error(CHEBMG_EINVAL, "NULL vector");
     if (dtype == CHEBMG_F64) {
@@ -3006,7 +3022,7 @@ int chebmg_smooth(chebmg_ctx* c, int level, int dtype, const void* b, void* x, i
 int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* rc) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1 && level_checked(c, level).n >= kChainMinN, c->s);
+    const PdlScope pdl_(c->nb == 1 && chain_restrict(level_checked(c, level), dtype), c->s);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
     if (!rf || !rc) throw Error(CHEBMG_EINVAL, "NULL vector");
@@ -3019,7 +3035,8 @@ int chebmg_restrict(chebmg_ctx* c, int level, int dtype, const void* rf, void* r
 int chebmg_prolong(chebmg_ctx* c, int level, int dtype, const void* zc, void* zf, int accumulate) {
   return guard([&]() -> int {
     enter(c);
-    const PdlScope pdl_(c->nb == 1 && level_checked(c, level).n >= kChainMinN, c->s);
+    level_checked(c, level);
+    const PdlScope pdl_(c->nb == 1, c->s);
     check_dtype(c, dtype);
     if (level + 1 >= (int)c->L.size()) throw Error(CHEBMG_EINVAL, "no coarser level");
     if (!zc || !zf) throw Error(CHEBMG_EINVAL, "NULL vector");
