@@ -93,9 +93,11 @@ __device__ __forceinline__ void stage_J(T* sJ) {
 }
 
 template <int QF>
+constexpr int kElements = QF == 8 ? 2 : QF == 6 ? 7 : 16;        // elements per block: whole warps, nearly
+template <int QF, int EB_>
 struct Shape {
   static constexpr int T = QF * QF;                              // threads per element
-  static constexpr int EB = QF == 8 ? 2 : QF == 6 ? 7 : 16;      // elements per block
+  static constexpr int EB = EB_;
   static constexpr int THREADS = (EB * T + 31) / 32 * 32;
 };
 
@@ -136,11 +138,11 @@ __device__ __forceinline__ uint32_t column_id(const Lattice& L, ElemCoord c, int
 // its points below N in every direction, and a last element its end points too, which are
 // boundary points: the free fine values of an element are those with i, j, k < N, so the last
 // value of every line is zero.
-template <typename T, int QF, int QC>
-__global__ void __launch_bounds__(Shape<QF>::THREADS)
+template <typename T, int QF, int QC, int EB>
+__global__ void __launch_bounds__(Shape<QF, EB>::THREADS)
 k_restrict_box(int64_t E, Lattice Lf, Lattice Lc, BoxDiv bd, const T* __restrict__ rf, T* __restrict__ rc,
                int64_t ldf, int64_t ldc) {
-  using S = Shape<QF>;
+  using S = Shape<QF, EB>;
   constexpr int NF = QF - 1;
   constexpr int NT = S::T, PB = QF * QF + 8, PC = QC * QF + 4;      // padded planes
   constexpr int L1 = QF * QC, S1 = NT / L1 < 1 ? 1 : (NT / L1 > QC ? QC : NT / L1), O1 = QC / S1;
@@ -204,11 +206,11 @@ k_restrict_box(int64_t E, Lattice Lf, Lattice Lc, BoxDiv bd, const T* __restrict
 }
 
 // zf (+)= P zc at the owned fine copies (boundary nodes: zero when not accumulating)
-template <typename T, int QF, int QC>
-__global__ void __launch_bounds__(Shape<QF>::THREADS)
+template <typename T, int QF, int QC, int EB>
+__global__ void __launch_bounds__(Shape<QF, EB>::THREADS)
 k_prolong_box(int64_t E, Lattice Lf, Lattice Lc, BoxDiv bd, const T* __restrict__ zc, T* __restrict__ zf,
               int accumulate, int64_t ldf, int64_t ldc) {
-  using S = Shape<QF>;
+  using S = Shape<QF, EB>;
   constexpr int NF = QF - 1;
   constexpr int NT = S::T, PB = QC * QF + 4, PC = QF * QF + 8;
   constexpr int L1 = QC * QC, S1 = NT / L1 < 1 ? 1 : (NT / L1 > QF / 2 ? QF / 2 : NT / L1), O1 = (QF + S1 - 1) / S1;
@@ -321,19 +323,44 @@ bool transfer_box_supported(int Qf, int Qc) {
   return (Qf == 8 && Qc == 4) || (Qf == 4 && Qc == 2) || (Qf == 8 && Qc == 6) || (Qf == 6 && Qc == 4);
 }
 
+// Blocks of one element where full blocks leave SMs idle and the busiest SM then has fewer warps to issue
+// for.  Order 5 in FP64 alone: a full block's seven elements are FP64 work in series on one SM
+// (a single 5 -> 3 interpolation with the call's synchronisation on 64 to 392 elements 20.4 -> 18.2 us, a
+// restriction 20.8 -> 18.4; the lines meet at 456 elements).  Order 7 has two elements in a block, order 3 little work in each, and FP32 on so few elements is not
+// bound by its issue.
+template <int QF>
+bool single_elements(int64_t E, int nb) {
+  const int sms = sm_count() > 0 ? sm_count() : 1;
+  auto warps = [&](int eb, int threads) { return ((E + eb - 1) / eb * nb + sms - 1) / sms * (threads / 32); };
+  return warps(1, Shape<QF, 1>::THREADS) < warps(kElements<QF>, Shape<QF, kElements<QF>>::THREADS);
+}
+
+template <typename T, int QF, int QC, int EB>
+static void launch_restrict_eb(int64_t E, const Lattice& Lf, const Lattice& Lc, const T* rf, T* rc, cudaStream_t s,
+                               int nb, int64_t ldf, int64_t ldc) {
+  launch_dep(k_restrict_box<T, QF, QC, EB>, dim3((unsigned)((E + EB - 1) / EB), nb), dim3(Shape<QF, EB>::THREADS), 0,
+             s, E, Lf, Lc, box_div(Lf), rf, rc, ldf, ldc);
+}
+template <typename T, int QF, int QC, int EB>
+static void launch_prolong_eb(int64_t E, const Lattice& Lf, const Lattice& Lc, const T* zc, T* zf, int accumulate,
+                              cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
+  launch_dep(k_prolong_box<T, QF, QC, EB>, dim3((unsigned)((E + EB - 1) / EB), nb), dim3(Shape<QF, EB>::THREADS), 0,
+             s, E, Lf, Lc, box_div(Lf), zc, zf, accumulate, ldf, ldc);
+}
 template <typename T, int QF, int QC>
 static void launch_restrict(int64_t E, const Lattice& Lf, const Lattice& Lc, const T* rf, T* rc, cudaStream_t s, int nb,
                             int64_t ldf, int64_t ldc) {
-  using S = Shape<QF>;
-  launch_dep(k_restrict_box<T, QF, QC>, dim3((unsigned)((E + S::EB - 1) / S::EB), nb), dim3(S::THREADS), 0, s, E, Lf,
-             Lc, box_div(Lf), rf, rc, ldf, ldc);
+  if constexpr (sizeof(T) == 8 && QF == 6)
+    if (single_elements<QF>(E, nb)) return launch_restrict_eb<T, QF, QC, 1>(E, Lf, Lc, rf, rc, s, nb, ldf, ldc);
+  launch_restrict_eb<T, QF, QC, kElements<QF>>(E, Lf, Lc, rf, rc, s, nb, ldf, ldc);
 }
 template <typename T, int QF, int QC>
 static void launch_prolong(int64_t E, const Lattice& Lf, const Lattice& Lc, const T* zc, T* zf, int accumulate,
                            cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
-  using S = Shape<QF>;
-  launch_dep(k_prolong_box<T, QF, QC>, dim3((unsigned)((E + S::EB - 1) / S::EB), nb), dim3(S::THREADS), 0, s, E, Lf,
-             Lc, box_div(Lf), zc, zf, accumulate, ldf, ldc);
+  if constexpr (sizeof(T) == 8 && QF == 6)
+    if (single_elements<QF>(E, nb))
+      return launch_prolong_eb<T, QF, QC, 1>(E, Lf, Lc, zc, zf, accumulate, s, nb, ldf, ldc);
+  launch_prolong_eb<T, QF, QC, kElements<QF>>(E, Lf, Lc, zc, zf, accumulate, s, nb, ldf, ldc);
 }
 
 template <typename T>
