@@ -192,9 +192,9 @@ __global__ void k_cheb4_step(int64_t n, T* __restrict__ x, T* r, T* __restrict__
 
 // Zero guess: r = b (rin = b), d = c0 S b; or (from_r) from the residual r: d = c0 S r.  order1:
 // x = w d (x += w d from a residual) instead of storing d.  b_next leaves r = b_next for the
-// restriction residual.
+// restriction residual.  rin and x may be one buffer (a caller's b and x), rin and r as well.
 template <typename T, bool VEC>
-__global__ void k_smooth_begin(int64_t n, const T* rin, T* __restrict__ x, T* r, T* __restrict__ d,
+__global__ void k_smooth_begin(int64_t n, const T* rin, T* x, T* r, T* __restrict__ d,
                                const T* __restrict__ invD, T c0, T w, int from_r, int order1, const T* b_next, int64_t ld) {
   pdl_wait();
   { const int64_t off_ = (int64_t)blockIdx.y * ld; rin += off_; x += off_; r += off_; d += off_; if (b_next) b_next += off_; }
