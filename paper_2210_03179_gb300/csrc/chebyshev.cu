@@ -37,8 +37,9 @@ struct V16<double> {
   static constexpr int L = 2;
 };
 
-// 4th-kind init.  mode 2: d = c0 S b only; 1: x = 0, r = b, d = c0 S r; 0: r = b - y, y = 0,
-// d = c0 S r.  VEC: 16-byte accesses over the aligned body, scalar tail.
+// The adjoint's forward recurrence (SEM) and the context-free FD smoother: separate product vector y.
+// 4th-kind init: x = 0, r = b (x_is_zero) or r = b - y, y = 0; then d = c0 S r.  VEC: 16-byte accesses
+// over the aligned body, scalar tail.
 template <typename T, bool VEC>
 __global__ void k_cheb4_init(int64_t n, const T* __restrict__ b, T* __restrict__ x, T* __restrict__ r,
                              T* __restrict__ d, T* __restrict__ y, const T* __restrict__ invD, T c0,
@@ -56,12 +57,6 @@ __global__ void k_cheb4_init(int64_t n, const T* __restrict__ b, T* __restrict__
     VT rv, dv;
     T* rs = reinterpret_cast<T*>(&rv);
     T* ds = reinterpret_cast<T*>(&dv);
-    if (x_is_zero == 2) {   // x = 0 and r = b are left to the first step, which reads b
-#pragma unroll
-      for (int l = 0; l < L; ++l) ds[l] = c0 * ss[l] * bs[l];
-      reinterpret_cast<VT*>(d)[q] = dv;
-      continue;
-    }
     if (x_is_zero) {
 #pragma unroll
       for (int l = 0; l < L; ++l) rs[l] = bs[l];
@@ -80,10 +75,6 @@ __global__ void k_cheb4_init(int64_t n, const T* __restrict__ b, T* __restrict__
   }
   for (int64_t g = nv * L + tid; g < n; g += stride) {
     T rv;
-    if (x_is_zero == 2) {
-      d[g] = c0 * invD[g] * b[g];
-      continue;
-    }
     if (x_is_zero) {
       rv = b[g];
       x[g] = T(0);
@@ -97,20 +88,16 @@ __global__ void k_cheb4_init(int64_t n, const T* __restrict__ b, T* __restrict__
 }
 
 
-template <typename T, bool FIRST = false>
-__device__ __forceinline__ void cheb4_one(T& x, T& r, T& d, T& y, T s, T beta, T c1, T c2, T beta_next) {
+template <typename T>
+__device__ __forceinline__ void cheb4_one(T& x, T& r, T& d, T& y, T s, T beta, T c1, T c2) {
   const T dv = d;
   const T rv = r - y;
-  if (FIRST) x = beta * dv;    // first step from x = 0 (r holds b)
-  else x += beta * dv;
+  x += beta * dv;
   r = rv;
   d = c1 * dv + c2 * s * rv;
   y = T(0);
-  if (beta_next != T(0)) x += beta_next * d;   // last step: the final update x += beta_k d_k
 }
 
-// x += beta d; r -= y; d = c1 d + c2 S r; y = 0 -- 16-byte vector accesses over the aligned
-// body (every pointer comes from a 256-byte aligned allocation), scalar tail.
 // 16-byte global accesses with an L2 eviction hint.  The update streams x, r and S (evict
 // first) and keeps d and y in L2 (evict last): the next operator application gathers d and
 // accumulates into y, so they should still be there when it runs.
@@ -140,18 +127,15 @@ __device__ __forceinline__ void st16(VT* p, const VT& val, uint64_t pol) {
                : "memory");
 }
 
-// FIRST: the first step of a smoother application from x = 0, after an init that wrote only d:
-// r is read from b (rin) and x is not read (x = beta d), so the init writes neither x nor r.
-// (rin is r itself in the other steps, so neither is declared __restrict__.)
-template <typename T, bool VEC, bool FIRST = false>
-__global__ void k_cheb4_step(int64_t n, T* __restrict__ x, T* r, T* __restrict__ d,
-                             T* __restrict__ y, const T* __restrict__ invD, T beta, T c1, T c2, T beta_next,
-                             int64_t ld, const T* rin) {
+// x += beta d; r -= y; d = c1 d + c2 S r; y = 0.
+template <typename T, bool VEC>
+__global__ void k_cheb4_step(int64_t n, T* __restrict__ x, T* __restrict__ r, T* __restrict__ d,
+                             T* __restrict__ y, const T* __restrict__ invD, T beta, T c1, T c2, int64_t ld) {
   // Everything read here is the operator kernel's output or older: wait for that kernel before
   // the first load.  (Triggering the next kernel early as well, griddepcontrol.launch_dependents,
   // was measured slower: its waiting blocks cost this grid's last wave more than they saved.)
   pdl_wait();
-  { const int64_t off_ = (int64_t)blockIdx.y * ld; x += off_; r += off_; d += off_; y += off_; rin += off_; }
+  { const int64_t off_ = (int64_t)blockIdx.y * ld; x += off_; r += off_; d += off_; y += off_; }
   using VT = typename V16<T>::type;
   constexpr int L = V16<T>::L;
   const int64_t nv = VEC ? n / L : 0;
@@ -159,8 +143,7 @@ __global__ void k_cheb4_step(int64_t n, T* __restrict__ x, T* r, T* __restrict__
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const uint64_t first = l2_policy_first(), last = l2_policy_last();
   for (int64_t q = tid; q < nv; q += stride) {
-    VT xv = {}, rv = ld16(reinterpret_cast<const VT*>(rin) + q, first);
-    if (!FIRST) xv = ld16(reinterpret_cast<VT*>(x) + q, first);
+    VT xv = ld16(reinterpret_cast<VT*>(x) + q, first), rv = ld16(reinterpret_cast<VT*>(r) + q, first);
     VT dv = ld16(reinterpret_cast<VT*>(d) + q, last), yv = ld16(reinterpret_cast<VT*>(y) + q, last);
     const VT sv = ld16(reinterpret_cast<const VT*>(invD) + q, first);
     T* xs = reinterpret_cast<T*>(&xv);
@@ -169,18 +152,14 @@ __global__ void k_cheb4_step(int64_t n, T* __restrict__ x, T* r, T* __restrict__
     T* ys = reinterpret_cast<T*>(&yv);
     const T* ss = reinterpret_cast<const T*>(&sv);
 #pragma unroll
-    for (int l = 0; l < L; ++l) cheb4_one<T, FIRST>(xs[l], rs[l], ds[l], ys[l], ss[l], beta, c1, c2, beta_next);
+    for (int l = 0; l < L; ++l) cheb4_one<T>(xs[l], rs[l], ds[l], ys[l], ss[l], beta, c1, c2);
     st16(reinterpret_cast<VT*>(x) + q, xv, first);
     st16(reinterpret_cast<VT*>(r) + q, rv, first);
     st16(reinterpret_cast<VT*>(d) + q, dv, last);
     st16(reinterpret_cast<VT*>(y) + q, yv, last);
   }
-  for (int64_t g = nv * L + tid; g < n; g += stride) {
-    T xg = FIRST ? T(0) : x[g], rg = rin[g];
-    cheb4_one<T, FIRST>(xg, rg, d[g], y[g], invD[g], beta, c1, c2, beta_next);
-    x[g] = xg;
-    r[g] = rg;
-  }
+  for (int64_t g = nv * L + tid; g < n; g += stride)
+    cheb4_one<T>(x[g], r[g], d[g], y[g], invD[g], beta, c1, c2);
 }
 
 // ---- SEM smoothing: the operator subtracts A d from r in place ----
@@ -357,26 +336,17 @@ void cheb4_init(int64_t n, const T* b, T* x, T* r, T* d, T* y, const T* invD, do
     launch_dep(k_cheb4_init<T, false>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, b, x, r, d,
                y, invD, (T)c0, x_is_zero, ld);
 }
-template <typename T, bool FIRST>
-static void launch_cheb4_step(int64_t n, T* x, T* r, T* d, T* y, const T* invD, double beta, double c1, double c2,
-                              cudaStream_t s, int nb, int64_t ld, double beta_next, const T* rin) {
-  const uintptr_t align =
-      (uintptr_t)x | (uintptr_t)r | (uintptr_t)d | (uintptr_t)y | (uintptr_t)invD | (uintptr_t)rin;
-  if (align % 16 == 0 && (nb == 1 || (ld * sizeof(T)) % 16 == 0))
-    launch_dep(k_cheb4_step<T, true, FIRST>, dim3(grid_for(n / V16<T>::L + 1, kVecThreads), nb), dim3(kVecThreads),
-               0, s, n, x, r, d, y, invD, (T)beta, (T)c1, (T)c2, (T)beta_next, ld, rin);
-  else
-    launch_dep(k_cheb4_step<T, false, FIRST>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, x, r,
-               d, y, invD, (T)beta, (T)c1, (T)c2, (T)beta_next, ld, rin);
-}
 template <typename T>
 void cheb4_step(int64_t n, T* x, T* r, T* d, T* y, const T* invD, double beta, double c1, double c2,
-                cudaStream_t s, int nb, int64_t ld, double beta_next, const T* b_first) {
+                cudaStream_t s, int nb, int64_t ld) {
   if (!ld) ld = n;
-  if (b_first)
-    launch_cheb4_step<T, true>(n, x, r, d, y, invD, beta, c1, c2, s, nb, ld, beta_next, b_first);
+  const uintptr_t align = (uintptr_t)x | (uintptr_t)r | (uintptr_t)d | (uintptr_t)y | (uintptr_t)invD;
+  if (align % 16 == 0 && (nb == 1 || (ld * sizeof(T)) % 16 == 0))
+    launch_dep(k_cheb4_step<T, true>, dim3(grid_for(n / V16<T>::L + 1, kVecThreads), nb), dim3(kVecThreads), 0, s, n,
+               x, r, d, y, invD, (T)beta, (T)c1, (T)c2, ld);
   else
-    launch_cheb4_step<T, false>(n, x, r, d, y, invD, beta, c1, c2, s, nb, ld, beta_next, r);
+    launch_dep(k_cheb4_step<T, false>, dim3(grid_for(n, kVecThreads), nb), dim3(kVecThreads), 0, s, n, x, r, d, y,
+               invD, (T)beta, (T)c1, (T)c2, ld);
 }
 // Whether every pointer and the batch stride allow 16-byte accesses.
 template <typename T, typename... P>
@@ -455,13 +425,6 @@ void masked_copy(int64_t n, const double* in, const double* invD, double* out, c
 
 
 #define CHEBMG_CHEB_INST(T)                                                                                 \
-  template void cheb4_init<T>(int64_t, const T*, T*, T*, T*, T*, const T*, double, int, cudaStream_t, int,    \
-                              int64_t);                                                                 \
-  template void cheb4_step<T>(int64_t, T*, T*, T*, T*, const T*, double, double, double, cudaStream_t, int,   \
-                              int64_t, double, const T*);                                               \
-  template void cheb1_init<T>(int64_t, const T*, T*, T*, T*, T*, const T*, double, int, cudaStream_t, int,    \
-                              int64_t);                                                                 \
-  template void cheb1_step<T>(int64_t, T*, T*, T*, T*, const T*, double, double, cudaStream_t, int, int64_t); \
   template void smooth_begin<T>(int64_t, const T*, T*, T*, T*, const T*, double, bool, double, const T*,    \
                                 cudaStream_t, int, int64_t);                                            \
   template void smooth_begin_r<T>(int64_t, T*, T*, T*, const T*, double, bool, double, const T*, cudaStream_t, \
@@ -472,6 +435,14 @@ void masked_copy(int64_t n, const double* in, const double* invD, double* out, c
 
 CHEBMG_CHEB_INST(float)
 CHEBMG_CHEB_INST(double)
+template void cheb4_init<double>(int64_t, const double*, double*, double*, double*, double*, const double*, double, int,
+                                 cudaStream_t, int, int64_t);
+template void cheb4_step<double>(int64_t, double*, double*, double*, double*, const double*, double, double, double,
+                                 cudaStream_t, int, int64_t);
+template void cheb1_init<double>(int64_t, const double*, double*, double*, double*, double*, const double*, double, int,
+                                 cudaStream_t, int, int64_t);
+template void cheb1_step<double>(int64_t, double*, double*, double*, double*, const double*, double, double,
+                                 cudaStream_t, int, int64_t);
 template void cast<double, float>(int64_t, const double*, float*, cudaStream_t, int, int64_t, int64_t);
 template void cast<float, double>(int64_t, const float*, double*, cudaStream_t, int, int64_t, int64_t);
 template void cast<double, double>(int64_t, const double*, double*, cudaStream_t, int, int64_t, int64_t);

@@ -327,18 +327,16 @@ void fd_adj_mid(int mx, int my, const Stencil9<double>& st, const double* rb, do
 void dense_matvec(int n, const double* M, const double* x, double* y, cudaStream_t s, int nb = 1, int64_t ld = 0);
 
 // ---- Chebyshev recurrences (Algorithms 1 and 2), elementwise over n ----
-// 4th kind init: x_is_zero 1: x = 0, r = b; 0: r = b - y, y = 0; then d = c0 S r.  x_is_zero 2:
-// d = c0 S b only (x = 0 and r = b are left to the first cheb4_step, given b_first = b).
+// With a product vector y of its own, FP64 only: the adjoint's forward recurrence (SEM) and the context-free
+// FD smoother.
+// 4th kind init: x = 0, r = b (x_is_zero) or r = b - y, y = 0; then d = c0 S r.
 template <typename T>
 void cheb4_init(int64_t n, const T* b, T* x, T* r, T* d, T* y, const T* invD, double c0,
                 int x_is_zero, cudaStream_t s, int nb = 1, int64_t ld = 0);
-// 4th kind step: x += beta d; r -= y; d = c1 d + c2 S r; y = 0; then, if beta_next != 0 (the
-// last step), the final update x += beta_next d with the new d.  b_first: the first step from
-// x = 0 after cheb4_init with x_is_zero = 2 (d only): r = b_first - y and x = beta d.
+// 4th kind step: x += beta d; r -= y; d = c1 d + c2 S r; y = 0.
 template <typename T>
 void cheb4_step(int64_t n, T* x, T* r, T* d, T* y, const T* invD, double beta, double c1,
-                double c2, cudaStream_t s, int nb = 1, int64_t ld = 0, double beta_next = 0.0,
-                const T* b_first = nullptr);
+                double c2, cudaStream_t s, int nb = 1, int64_t ld = 0);
 // 1st kind init: r = S (b - y) (or S b), d = r / theta, y = 0 (x = 0 if x_is_zero).
 template <typename T>
 void cheb1_init(int64_t n, const T* b, T* x, T* r, T* d, T* y, const T* invD, double inv_theta,

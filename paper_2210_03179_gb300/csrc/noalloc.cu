@@ -138,7 +138,8 @@ extern "C" int chebmg_fd_smooth_noalloc(int m, double Lx, double Ly, int kind, i
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (!x_is_zero) fd_apply<double>(m, m, A, x, y, s);
 
-  // The same smoother arithmetic as chebmg_smooth on level 0 of an FD context.
+  // The smoother of chebmg_smooth on level 0 of an FD context, by separate operator and update kernels (its
+  // rounding differs).
   if (kind == CHEBMG_CHEB_1ST) {
     const double lmin = lmin_ratio * lmax;
     const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
