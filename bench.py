@@ -840,11 +840,13 @@ def main():
     step64 = smoother_step_time(s64, cm.CHEBMG_F64, False)
     E = NE ** 3
     L = E * (NORDER + 1) ** 3
-    alg_bytes32 = 4 * (6 * L + 7 * n)
+    fused32 = cm.chebmg_fused_smoother(s32.ctx, 0, cm.CHEBMG_F32)
+    # the factors, and the vectors read or written once each: r and d both ways, S, and x both ways every
+    # step (fused) or every other step (separate kernels)
+    alg_bytes32 = 4 * (6 * L + (7 if fused32 else 6) * n)
     pk = peaks()
     hbm = pk.get("hbm_gbs")
     achieved = alg_bytes32 / step32 / 1e9
-    fused32 = cm.chebmg_fused_smoother(s32.ctx, 0, cm.CHEBMG_F32)
     tile32 = cm.chebmg_tile_choice(s32.ctx, 0, cm.CHEBMG_F32)
     roofline = {"bound": "hbm",
                 "kernel": ("fine FP32 Chebyshev step, fused: k_sem_smooth8 (one launch per smoother application)"

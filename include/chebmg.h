@@ -187,6 +187,7 @@ int chebmg_set_outer_operator(chebmg_ctx* ctx, int kind);
 /* y = A x on the finest level with the context's outer operator (FP64 device vectors). */
 int chebmg_apply_outer(chebmg_ctx* ctx, const double* x, double* y);
 int chebmg_set_coarse_degree(chebmg_ctx* ctx, int degree);
+/* Overrides the autotuned operator variant of an order-7 or order-3 level (order 3: for batches too). */
 int chebmg_set_tile_choice(chebmg_ctx* ctx, int level, int dtype, int variant);
 
 /* Fused smoother on order-7 box-lattice levels (Algorithms 1 and 2 with the operator of

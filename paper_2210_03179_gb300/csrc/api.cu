@@ -94,6 +94,8 @@ struct Level {
   void* v[2][NV] = {{nullptr}};
   int eb[2] = {2, 2};   // variant of the order-7 operator, per dtype (autotuned)
   int ax4[2] = {41, 41};   // order-3 operator: 40 one thread per point, 41 line passes (+100 lattice ids)
+  int bax4[2] = {0, 0};    // the same for batches, 0: as ax4
+  bool ax4_set[2] = {false, false};   // ax4 was set by hand, for batches too
   int beb[2] = {2002, 2002};   // variant of the batched order-7 operator (autotuned per batch size)
   Lattice lat = {0, 0, 0, 0, 0, 0};
   bool boxed = true;    // SEM: the level carries the box lattice (lattice-indexed kernels usable)
@@ -282,13 +284,14 @@ void apply_into_ld(chebmg_ctx* c, int j, const T* x, T* y, int nb, int64_t ld, b
   Level& L = c->L[j];
   const int dt = dt_of<T>();
   if (L.type == TYPE_SEM) {
+    const int ax4 = L.Q != 4 ? 0 : nb > 1 && L.bax4[dt] ? L.bax4[dt] : L.ax4[dt];
     if (L.Q == 8 && nb > 1)
       sem_ax8_batched<T>(L.E, L.gid, L.lat, static_cast<const T*>(L.G[dt]), x, y, c->dstat, L.beb[dt], nb, ld,
                          c->s, subtract);
     else if (L.Q == 8)
       sem_ax8<T>(L.E, L.gid, L.lat, static_cast<const T*>(L.G[dt]), x, y, c->dstat, L.eb[dt], c->s, subtract);
-    else if (L.Q == 4 && L.ax4[dt] % 100 == 41)
-      sem_ax4<T>(L.E, L.gid, L.ax4[dt] >= 100 ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]),
+    else if (ax4 % 100 == 41)
+      sem_ax4<T>(L.E, L.gid, ax4 >= 100 ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]),
                  static_cast<const T*>(L.D[dt]), x, y, c->s, nb, ld, subtract);
     else if (!(sem_axl_chosen<T>(L.Q, L.E * nb)
                    ? sem_axl<T>(L.Q, L.E, L.gid, L.boxed ? &L.lat : nullptr, static_cast<const T*>(L.G[dt]), x, y,
@@ -1116,7 +1119,7 @@ void autotune_ax4(chebmg_ctx* c, int j) {
     L.ax4[dt] = v;
     apply_into<T>(c, j, x, y);   // warm-up
     float t_min = 1e30f;
-    for (int rep = 0; rep < 3; ++rep) {
+    for (int rep = 0; rep < 6; ++rep) {
       CK(cudaEventRecord(e0, c->s));
       apply_into<T>(c, j, x, y);
       CK(cudaEventRecord(e1, c->s));
@@ -1529,6 +1532,38 @@ void autotune_batch(chebmg_ctx* c, int nrhs) {
           }
         }
         L.beb[dt] = best_v;
+        CK(cudaMemsetAsync(y, 0, es * (size_t)nrhs * L.ld, c->s));
+      }
+    }
+    // the order-3 operator as well: on one vector its kernels can be even where a batch parts them (512
+    // elements, FP32: setup chose either of them from run to run; 64 right-hand sides 22.8 us with a thread
+    // per point, 13.4 with line passes)
+    for (int j = 0; j < (int)c->L.size(); ++j) {
+      Level& L = c->L[j];
+      if (L.type != TYPE_SEM || L.Q != 4) continue;
+      for (int dt = 0; dt < 2; ++dt) {
+        if (!L.G[dt] || L.ax4_set[dt]) continue;
+        void* x = L.v[dt][VB];
+        void* y = L.v[dt][VY];
+        const size_t es = dt == CHEBMG_F64 ? 8 : 4;
+        CK(cudaMemsetAsync(x, 0, es * (size_t)nrhs * L.ld, c->s));
+        float best = 1e30f;
+        int best_v = L.bax4[dt];
+        for (int v : {40, 41, 141}) {
+          if (v >= 100 && !L.boxed) continue;
+          L.bax4[dt] = v;
+          const float t = time_it(
+              [&]() {
+                if (dt == CHEBMG_F64) apply_into<double>(c, j, static_cast<double*>(x), static_cast<double*>(y));
+                else apply_into<float>(c, j, static_cast<float*>(x), static_cast<float*>(y));
+              },
+              6);
+          if (t < best) {
+            best = t;
+            best_v = v;
+          }
+        }
+        L.bax4[dt] = best_v;
         CK(cudaMemsetAsync(y, 0, es * (size_t)nrhs * L.ld, c->s));
       }
     }
@@ -2800,6 +2835,8 @@ int chebmg_set_tile_choice(chebmg_ctx* c, int level, int dtype, int variant) {
   if (L.type == TYPE_SEM && L.Q == 4) {
     if ((variant != 40 && variant != 41 && variant != 141) || (variant == 141 && !L.boxed)) return CHEBMG_EINVAL;
     L.ax4[dtype] = variant;
+    L.bax4[dtype] = 0;
+    L.ax4_set[dtype] = true;
     drop_graphs(c);
     return CHEBMG_OK;
   }

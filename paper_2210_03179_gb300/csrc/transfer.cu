@@ -325,9 +325,9 @@ bool transfer_box_supported(int Qf, int Qc) {
 
 // Blocks of one element where full blocks leave SMs idle and the busiest SM then has fewer warps to issue
 // for.  Order 5 in FP64 alone: a full block's seven elements are FP64 work in series on one SM
-// (a single 5 -> 3 interpolation with the call's synchronisation on 64 to 392 elements 20.4 -> 18.2 us, a
-// restriction 20.8 -> 18.4; the lines meet at 456 elements).  Order 7 has two elements in a block, order 3 little work in each, and FP32 on so few elements is not
-// bound by its issue.
+// (a single 5 -> 3 interpolation, with its synchronisation, on 64 to 392 elements 20.4 -> 18.2 us, a
+// restriction 20.8 -> 18.4; both forms have the same warps from 457 elements on).  Order 7 has two elements in
+// a block, order 3 little work in each, and FP32 on so few elements is not bound by its issue.
 template <int QF>
 bool single_elements(int64_t E, int nb) {
   const int sms = sm_count() > 0 ? sm_count() : 1;
