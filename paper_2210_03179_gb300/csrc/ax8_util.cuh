@@ -18,6 +18,8 @@ namespace {
 // of 336).  The geometric factors of a plane are stored in the order of the threads (permute_g8), so
 // their reads are consecutive.
 __device__ __forceinline__ constexpr int line_of(int t) { return 2 * ((t & 31) >> 3) + (t >> 5); }
+// Where the factors of point (i, j) of a plane are: the thread that owns its line.
+__device__ __forceinline__ constexpr int factor_of(int i, int j) { return ((j & 1) << 5) + ((j >> 1) << 3) + i; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
