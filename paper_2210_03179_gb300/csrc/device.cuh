@@ -34,13 +34,17 @@ inline int device_attribute(cudaDeviceAttr attr) {
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, attr, dev) != cudaSuccess) return 0;
   return v;
 }
-inline int sm_count() {
+inline int sm_count() {   // at least 1
   static PerDevice sms;
-  return sms([] { return device_attribute(cudaDevAttrMultiProcessorCount); });
+  const int n = sms([] { return device_attribute(cudaDevAttrMultiProcessorCount); });
+  return n > 0 ? n : 1;
 }
 
 // Lets kernel k take `bytes` of dynamic shared memory on the current device; `done` is the kernel's own.
+// Blocks that stay below the 48 KB every kernel may take (8 KB left to static arrays) need nothing: small
+// calls are bound by the host, and asking for the device costs it.
 inline void allow_smem(PerDevice& done, const void* k, size_t bytes) {
+  if (bytes <= 40 * 1024) return;
   done([=] {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess ? 1 : 0;
   });

@@ -1107,7 +1107,7 @@ static const void* coarse_kernel(int rpt) {
 }
 
 void coarse_pcg_shape(int64_t n, int rpt_min, int* grid, int* rows_per_block) {
-  const int sms = sm_count() > 0 ? sm_count() : 1;
+  const int sms = sm_count();
   const int64_t per_block_min = (n + sms - 1) / sms;
   int rpt = 1;
   while (rpt < rpt_min && rpt < kCoarseMaxRowsPerThread) rpt *= 2;

@@ -274,7 +274,7 @@ void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, cons
   constexpr int EB = Q == 3 ? 14 : Q == 5 ? 5 : Q == 6 ? 7 : Q == 7 ? 5 : sizeof(T) == 4 ? 1 : Q == 9 ? 3 : 5;
   constexpr int SMALL = Q == 3 ? 3 : 1;
   if constexpr (EB > SMALL) {
-    const int sms = sm_count() > 0 ? sm_count() : 1;
+    const int sms = sm_count();
     auto warps = [&](int eb, int threads) {   // of the busiest SM
       const int64_t blocks = (E + eb - 1) / eb * nb;
       return (blocks + sms - 1) / sms * (threads / 32);
@@ -315,7 +315,7 @@ void fill(const double* S, int Q, LineTab<T>& t) {   // S: symmetrised D, [Q][Q]
 template <typename T>
 bool sem_axl_chosen(int Q, int64_t elements) {
   const int64_t few = sizeof(T) == 4 || Q == 3 ? 0 : Q >= 9 ? 1 : 4;   // elements per SM
-  return sem_axl_supported(Q) && elements > few * sm_count();
+  return sem_axl_supported(Q) && (few == 0 || elements > few * sm_count());
 }
 template bool sem_axl_chosen<float>(int, int64_t);
 template bool sem_axl_chosen<double>(int, int64_t);

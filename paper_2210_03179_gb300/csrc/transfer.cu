@@ -330,7 +330,7 @@ bool transfer_box_supported(int Qf, int Qc) {
 // a block, order 3 little work in each, and FP32 on so few elements is not bound by its issue.
 template <int QF>
 bool single_elements(int64_t E, int nb) {
-  const int sms = sm_count() > 0 ? sm_count() : 1;
+  const int sms = sm_count();
   auto warps = [&](int eb, int threads) { return ((E + eb - 1) / eb * nb + sms - 1) / sms * (threads / 32); };
   return warps(1, Shape<QF, 1>::THREADS) < warps(kElements<QF>, Shape<QF, kElements<QF>>::THREADS);
 }
