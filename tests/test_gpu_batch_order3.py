@@ -67,8 +67,9 @@ def test_the_choice_is_made_on_the_batch():
                 cm.chebmg_set_tile_choice(s.ctx, 0, F32, v)
                 by_hand[v] = product_us(s, F32, X, Y)
         s.close()
-    # the forms differ by more than half of the faster one here; a tenth is left to the timing
-    assert max(chosen) <= 1.1 * min(by_hand.values()), (chosen, by_hand)
+    # us a product: a thread per point 22.9, line passes by map or by lattice 18.7 and 17.0, which the tuner
+    # may take for each other
+    assert max(chosen) <= 1.2 * min(by_hand.values()), (chosen, by_hand)
     s = solver(mesh)
     cm.chebmg_set_tile_choice(s.ctx, 0, F32, 40)
     assert product_us(s, F32, X, Y) > 1.2 * min(by_hand.values())      # set by hand: not tuned away
