@@ -266,8 +266,9 @@ void launch_eb(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, c
 }
 
 // Elements per block: the number that fills whole warps best (FP64 issue is paid for every lane of a
-// warp), or one where that leaves SMs idle: the busiest SM then has fewer warps to issue for (36
-// elements of order 9 in FP64: 72.1 us in blocks of five, 21.6 in blocks of one).
+// warp), or fewer where the busiest SM then has fewer warps to issue for: one where that leaves SMs idle
+// (36 elements of order 9 in FP64: 72.1 us in blocks of five, 21.6 in blocks of one), and at order 5 in FP64,
+// whose blocks of seven are the largest, five where that makes a smaller last wave (XXX).
 template <typename T, int Q>
 void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s, int nb,
             int64_t ld, uint32_t neg) {
@@ -279,9 +280,21 @@ void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, cons
       const int64_t blocks = (E + eb - 1) / eb * nb;
       return (blocks + sms - 1) / sms * (threads / 32);
     };
-    if (warps(SMALL, AxL<T, Q, SMALL>::THREADS) < warps(EB, AxL<T, Q, EB>::THREADS)) {
-      launch_eb<T, Q, SMALL>(E, gid, lat, G, u, y, s, nb, ld, neg);
-      return;
+    int64_t least = warps(EB, AxL<T, Q, EB>::THREADS);
+    int eb = EB;
+    auto consider = [&](int e, int threads) {
+      const int64_t w = warps(e, threads);
+      if (w < least) least = w, eb = e;
+    };
+    if constexpr (sizeof(T) == 8 && Q == 6) {
+      consider(5, AxL<T, Q, 5>::THREADS);
+      consider(4, AxL<T, Q, 4>::THREADS);
+    }
+    consider(SMALL, AxL<T, Q, SMALL>::THREADS);
+    if (eb == SMALL) return launch_eb<T, Q, SMALL>(E, gid, lat, G, u, y, s, nb, ld, neg);
+    if constexpr (sizeof(T) == 8 && Q == 6) {
+      if (eb == 5) return launch_eb<T, Q, 5>(E, gid, lat, G, u, y, s, nb, ld, neg);
+      if (eb == 4) return launch_eb<T, Q, 4>(E, gid, lat, G, u, y, s, nb, ld, neg);
     }
   }
   launch_eb<T, Q, EB>(E, gid, lat, G, u, y, s, nb, ld, neg);
