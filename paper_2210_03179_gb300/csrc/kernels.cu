@@ -35,7 +35,7 @@ constexpr int kVecThreads = 256;
 }  // namespace
 
 // ===========================================================================
-// SEM element operator, one thread per point: orders 1 and 3, and in FP64 the orders of the line passes
+// SEM element operator, one thread per point: orders 1 and 3, and the orders of the line passes
 // (sem_axl.cu) on few elements; order 7 is in sem_ax8.cu, order 3 has k_sem_ax4 below as well, autotuned
 // ===========================================================================
 template <int Q>
@@ -284,16 +284,14 @@ bool sem_ax(int Q, int64_t E, const uint32_t* gid, const T* G, const T* D, const
   switch (Q) {
     case 2: launch_sem_ax<T, 2>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
     case 4: launch_sem_ax<T, 4>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+    // the orders of the line passes on few elements (sem_axl_chosen)
+    case 5: launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+    case 6: launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
+    case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
     default:
-      if constexpr (sizeof(T) == 8) {   // FP64 on few elements (sem_axl_chosen)
-        switch (Q) {
-          case 5: launch_sem_ax<T, 5>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
-          case 6: launch_sem_ax<T, 6>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
-          case 7: launch_sem_ax<T, 7>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
-          case 9: launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
-          case 10: launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg); return true;
-          default: break;
-        }
+      if constexpr (sizeof(T) == 8) {
+        if (Q == 9) return launch_sem_ax<T, 9>(E, gid, G, D, u, y, s, nb, ld, neg), true;
+        if (Q == 10) return launch_sem_ax<T, 10>(E, gid, G, D, u, y, s, nb, ld, neg), true;
       }
       return false;
   }

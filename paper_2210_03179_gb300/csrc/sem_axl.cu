@@ -268,7 +268,8 @@ void launch_eb(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, c
 // Elements per block: the number that fills whole warps best (FP64 issue is paid for every lane of a
 // warp), or fewer where the busiest SM then has fewer warps to issue for: one where that leaves SMs idle
 // (36 elements of order 9 in FP64: 72.1 us in blocks of five, 21.6 in blocks of one), and at order 5 in FP64,
-// whose blocks of seven are the largest, five where that makes a smaller last wave (XXX).
+// whose blocks of seven are the largest, five or four where that makes a smaller last wave (order-4
+// smoothing of 1,100 elements 135 -> 94.6 us, of 2,200 199 -> 157).
 template <typename T, int Q>
 void launch(int64_t E, const uint32_t* gid, const Lattice* lat, const T* G, const T* u, T* y, cudaStream_t s, int nb,
             int64_t ld, uint32_t neg) {
@@ -319,15 +320,20 @@ void fill(const double* S, int Q, LineTab<T>& t) {   // S: symmetrised D, [Q][Q]
 
 }  // namespace
 
-// FP64 on few elements: a thread per point has the shorter serial chains, and the line passes' fewer
+// On few elements a thread per point has the shorter serial chains, and the line passes' fewer
 // operations count only once every SM has warps enough to keep FP64 issue busy.  Four products of a
 // smoother, thread per point against line passes: order 4 on 512 elements 41.5 / 47.3 us, on 640 61.2 /
 // 47.3; order 5 on 294 39.4 / 57.4, on 512 60.0 / 80.0, on 640 82.7 / 82.5; order 6 on 294 55.8 / 65.6, on
 // 448 76.3 / 79.5, on 640 114.8 / 98.2; order 8 on 150 68.2 / 85.6, on 180 114.2 / 105.0; order 9 on 150
 // 91.7 / 97.9, on 180 170.0 / 155.9.  Order 2: even at every size.
+// FP32, the same: order 4 on 64 elements 15.8 / 16.7 us, on 512 16.6 / 18.1, on 729 19.1 / 18.1; order 5 on 64
+// 16.0 / 17.8, on 343 18.2 / 18.2, on 512 19.7 / 20.6, on 729 21.4 / 20.1; order 6 on 64 16.0 / 18.1, on 125
+// 16.3 / 18.2, on 216 18.6 / 18.6, on 343 21.4 / 18.8.  Orders 2, 8 and 9 are even on the fewest (order 9 on
+// 64 elements 22.7 / 23.4) and line passes soon the faster.
 template <typename T>
 bool sem_axl_chosen(int Q, int64_t elements) {
-  const int64_t few = sizeof(T) == 4 || Q == 3 ? 0 : Q >= 9 ? 1 : 4;   // elements per SM
+  const int64_t few = sizeof(T) == 4 ? (Q == 5 || Q == 6 ? 4 : Q == 7 ? 1 : 0)   // elements per SM
+                                     : Q == 3 ? 0 : Q >= 9 ? 1 : 4;
   return sem_axl_supported(Q) && (few == 0 || elements > few * sm_count());
 }
 template bool sem_axl_chosen<float>(int, int64_t);
