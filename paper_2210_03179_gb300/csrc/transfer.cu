@@ -323,16 +323,25 @@ bool transfer_box_supported(int Qf, int Qc) {
   return (Qf == 8 && Qc == 4) || (Qf == 4 && Qc == 2) || (Qf == 8 && Qc == 6) || (Qf == 6 && Qc == 4);
 }
 
-// Blocks of one element where full blocks leave SMs idle and the busiest SM then has fewer warps to issue
-// for.  Order 5 in FP64 alone: a full block's seven elements are FP64 work in series on one SM
-// (a single 5 -> 3 interpolation, with its synchronisation, on 64 to 392 elements 20.4 -> 18.2 us, a
-// restriction 20.8 -> 18.4; both forms have the same warps from 457 elements on).  Order 7 has two elements in
-// a block, order 3 little work in each, and FP32 on so few elements is not bound by its issue.
+// Elements per block at order 5 in FP64: seven, or fewer where the busiest SM then has fewer warps to issue
+// for -- a full block's seven elements are FP64 work in series on one SM.  One element on up to 456
+// elements (a single 5 -> 3 interpolation, with its synchronisation, on 64 to 392 elements 20.4 -> 18.2 us,
+// a restriction 20.8 -> 18.4), five where seven make a nearly empty last wave (1,100 elements 22.3 -> 21.0).
+// Order 7 has two elements in a block, order 3 little work in each, and FP32 is not bound by its issue on
+// so few.
 template <int QF>
-bool single_elements(int64_t E, int nb) {
+int elements_per_block(int64_t E, int nb) {
   const int sms = sm_count();
-  auto warps = [&](int eb, int threads) { return ((E + eb - 1) / eb * nb + sms - 1) / sms * (threads / 32); };
-  return warps(1, Shape<QF, 1>::THREADS) < warps(kElements<QF>, Shape<QF, kElements<QF>>::THREADS);
+  int eb = 0;
+  int64_t least = 0;
+  auto consider = [&](int e, int threads) {
+    const int64_t w = ((E + e - 1) / e * nb + sms - 1) / sms * (threads / 32);
+    if (eb == 0 || w < least) least = w, eb = e;
+  };
+  consider(kElements<QF>, Shape<QF, kElements<QF>>::THREADS);
+  consider(1, Shape<QF, 1>::THREADS);
+  consider(5, Shape<QF, 5>::THREADS);
+  return eb;
 }
 
 template <typename T, int QF, int QC, int EB>
@@ -350,16 +359,21 @@ static void launch_prolong_eb(int64_t E, const Lattice& Lf, const Lattice& Lc, c
 template <typename T, int QF, int QC>
 static void launch_restrict(int64_t E, const Lattice& Lf, const Lattice& Lc, const T* rf, T* rc, cudaStream_t s, int nb,
                             int64_t ldf, int64_t ldc) {
-  if constexpr (sizeof(T) == 8 && QF == 6)
-    if (single_elements<QF>(E, nb)) return launch_restrict_eb<T, QF, QC, 1>(E, Lf, Lc, rf, rc, s, nb, ldf, ldc);
+  if constexpr (sizeof(T) == 8 && QF == 6) {
+    const int eb = elements_per_block<QF>(E, nb);
+    if (eb == 1) return launch_restrict_eb<T, QF, QC, 1>(E, Lf, Lc, rf, rc, s, nb, ldf, ldc);
+    if (eb == 5) return launch_restrict_eb<T, QF, QC, 5>(E, Lf, Lc, rf, rc, s, nb, ldf, ldc);
+  }
   launch_restrict_eb<T, QF, QC, kElements<QF>>(E, Lf, Lc, rf, rc, s, nb, ldf, ldc);
 }
 template <typename T, int QF, int QC>
 static void launch_prolong(int64_t E, const Lattice& Lf, const Lattice& Lc, const T* zc, T* zf, int accumulate,
                            cudaStream_t s, int nb, int64_t ldf, int64_t ldc) {
-  if constexpr (sizeof(T) == 8 && QF == 6)
-    if (single_elements<QF>(E, nb))
-      return launch_prolong_eb<T, QF, QC, 1>(E, Lf, Lc, zc, zf, accumulate, s, nb, ldf, ldc);
+  if constexpr (sizeof(T) == 8 && QF == 6) {
+    const int eb = elements_per_block<QF>(E, nb);
+    if (eb == 1) return launch_prolong_eb<T, QF, QC, 1>(E, Lf, Lc, zc, zf, accumulate, s, nb, ldf, ldc);
+    if (eb == 5) return launch_prolong_eb<T, QF, QC, 5>(E, Lf, Lc, zc, zf, accumulate, s, nb, ldf, ldc);
+  }
   launch_prolong_eb<T, QF, QC, kElements<QF>>(E, Lf, Lc, zc, zf, accumulate, s, nb, ldf, ldc);
 }
 

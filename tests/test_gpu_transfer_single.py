@@ -1,5 +1,5 @@
-"""The order 5 <-> 3 box transfers in FP64 on both sides of the element count up to which a block takes one
-element, single vectors and a batch's cycle, against the oracle."""
+"""The order 5 <-> 3 box transfers in FP64 at element counts where a block takes one, five and seven elements,
+single vectors and a batch's cycle, against the oracle."""
 import numpy as np
 import pytest
 
@@ -18,7 +18,8 @@ import paper_2210_03179_gb300 as cm  # noqa: E402
 from gpu_util import N, T  # noqa: E402
 
 
-@pytest.mark.parametrize("mesh", [(1, 1, 2), (5, 3, 7), (9, 8, 7), (8, 8, 8), (9, 9, 7)])   # up to 567 elements
+# one element a block up to 456 elements of 152 SMs, five on 512, 567 and 1,188, seven on 1,001
+@pytest.mark.parametrize("mesh", [(1, 1, 2), (5, 3, 7), (9, 8, 6), (8, 8, 8), (9, 9, 7), (13, 11, 7), (12, 11, 9)])
 def test_transfers(mesh):
     v = W.sem_box_vertices(*mesh)
     F, C = SemLevel(v, 5), SemLevel(v, 3)
